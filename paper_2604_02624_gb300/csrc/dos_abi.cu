@@ -142,6 +142,7 @@ struct dos_ctx {
   float* h_fwd = nullptr;
   dos::LossStats* stats = nullptr;
   double* d_loss = nullptr;
+  unsigned* loss_ticket = nullptr;  // channels done in the running loss kernel (zero between launches)
   double* h_loss = nullptr;  // pinned
   int chunk = 1, n_chunks = 1;
   // multi-pass passes that run their bulk-async prefetching kernels
@@ -467,6 +468,8 @@ int build(dos_ctx* x, const dos_config* c) {
   if ((rc = x->alloc(&x->h_fwd, (size_t)x->K * n2, "saved thickness"))) return rc;
   if ((rc = x->alloc(&x->stats, (size_t)x->nw, "loss statistics"))) return rc;
   if ((rc = x->alloc(&x->d_loss, 1, "loss"))) return rc;
+  if ((rc = x->alloc(&x->loss_ticket, 1, "loss ticket"))) return rc;
+  DOS_CUDA(cudaMemsetAsync(x->loss_ticket, 0, sizeof(unsigned), x->stream), "loss ticket");
   if ((rc = x->alloc(&x->dLdI_step, (size_t)x->nw * x->fov * x->fov, "step seed"))) return rc;
   DOS_CUDA(cudaMallocHost(&x->h_loss, sizeof(double)), "cudaMallocHost(loss)");
 
@@ -601,7 +604,7 @@ int gemm_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dL
     }
   }
   DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
-            dos::launch_grad_reduce_flat(c->partial, d_dLdh, c->gchunks, (size_t)c->K * n2, c->stream),
+            dos::launch_grad_reduce(c->partial, d_dLdh, c->gchunks, (size_t)c->K * n2, (size_t)c->K * n2, c->stream),
             "gradient reduction");
   ++c->launches;
   return gemm_check(c);
@@ -827,8 +830,8 @@ int run_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dLd
     DOS_TIMED(c, DOS_KERNEL_FUSED_ADJOINT, c->fops->launch(f, true, c->n_clusters, c->stream),
               "fused adjoint sweep");
     DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
-              dos::launch_grad_reduce_flat(c->partial, d_dLdh, std::min(c->n_clusters, c->nw), (size_t)c->K * n2,
-                                           c->stream),
+              dos::launch_grad_reduce(c->partial, d_dLdh, std::min(c->n_clusters, c->nw), (size_t)c->K * n2,
+                                      (size_t)c->K * n2, c->stream),
               "gradient reduction");
     c->launches = 2;
     return DOS_OK;
@@ -1140,11 +1143,10 @@ DOS_API int dos_loss(dos_ctx* c, const float* d_T, double* h_loss, float* d_psnr
   const double norm = (double)c->nw_total * det2;
   c->launches = 0;
   DOS_TIMED(c, DOS_KERNEL_LOSS,
-            dos::launch_loss_stats(c->o, d_T, c->stats, c->nw, c->fov, c->bin, d_dLdI, norm, c->loss, c->stream),
-            "loss statistics and dL/dI");
-  DOS_TIMED(c, DOS_KERNEL_LOSS, dos::launch_loss_final(c->stats, c->nw, det2, norm, c->loss, c->d_loss, d_psnr, c->stream),
-            "loss total");
-  c->launches += 2;
+            dos::launch_loss(c->o, d_T, c->stats, c->nw, c->fov, c->bin, d_dLdI, norm, c->loss, d_psnr, c->d_loss,
+                             c->loss_ticket, c->stream),
+            "loss, PSNR and dL/dI");
+  c->launches += 1;
   c->have_loss = true;
   if (h_loss) return dos_read_loss(c, h_loss);
   return DOS_OK;
@@ -1248,12 +1250,10 @@ DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dL
       rc = run_forward(c, d_h, d_I, 1);
       const int fwd_launches = c->launches;
       if (!rc)
-        e = dos::launch_loss_stats(c->o, d_T, c->stats, c->nw, c->fov, c->bin, c->dLdI_step, norm, c->loss,
-                                   c->gstream);
-      if (!rc && e == cudaSuccess)
-        e = dos::launch_loss_final(c->stats, c->nw, det2, norm, c->loss, c->d_loss, d_psnr, c->gstream);
+        e = dos::launch_loss(c->o, d_T, c->stats, c->nw, c->fov, c->bin, c->dLdI_step, norm, c->loss, d_psnr,
+                             c->d_loss, c->loss_ticket, c->gstream);
       if (!rc && e == cudaSuccess) rc = run_backward(c, d_h, c->dLdI_step, d_dLdh);
-      if (!rc) c->step_launches = fwd_launches + 2 + c->launches;
+      if (!rc) c->step_launches = fwd_launches + 1 + c->launches;
       cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
       if (e == cudaSuccess) e = e2;
     }

@@ -122,16 +122,17 @@ struct LossStats {
 };
 // o: [nw][fov][fov] output field; T: [nw][fov/bin][fov/bin] targets of the
 // detector pixels (bin x bin simulation pixels each); dLdI: [nw][fov][fov] or
-// null (then not written); norm: the loss's divisor; mode: DOS_LOSS_*
-cudaError_t launch_loss_stats(const float2* o, const float* T, LossStats* st, int nw, int fov, int bin,
-                              float* dLdI, double norm, int mode, cudaStream_t s);
-// det2: detector pixels per channel (PSNR mean)
+// null (then not written); psnr: [nw] or null; norm: the loss's divisor; mode:
+// DOS_LOSS_*; ticket: zero before the first launch, left at zero by each
+cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, int fov, int bin, float* dLdI,
+                        double norm, int mode, float* psnr, double* d_loss, unsigned* ticket, cudaStream_t s);
+// total and PSNR from records made elsewhere (dos_loss_noalloc); det2: detector
+// pixels per channel (PSNR mean)
 cudaError_t launch_loss_final(const LossStats* st, int nw, int det2, double norm, int mode,
                               double* d_loss, float* d_psnr, cudaStream_t s);
-cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_chunks, size_t count,
-                               size_t chunk_stride, cudaStream_t s);
-cudaError_t launch_grad_reduce_flat(const float* partial, float* grad, int n_parts, size_t count,
-                                    cudaStream_t s);
+// partial: [count / n2][n_parts][n2] -> grad [count] (n2 = count: flat parts)
+cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2,
+                               cudaStream_t s);
 
 // Evaluation variants (dos_eval.cu).
 cudaError_t launch_quantize(const float* h, float* q, size_t count, double h_max, int bits, cudaStream_t s);

@@ -40,17 +40,68 @@ __device__ __forceinline__ float detector(const float2* ow, int fov, int b, int 
   return s;
 }
 
-// per channel: sum (D-T)^2, sigma = sum D T / sum D^2, sum (sigma D - T)^2,
-// and (dLdI not null) dL/dI of the channel's simulation pixels: dL/dD of the
-// detector pixel covering it, 2 (D - T) / norm, or 2 sigma (sigma D - T) / norm
-// for the scaled loss (scale = 2 / norm)
-__global__ void __launch_bounds__(kRedThreads) k_loss_stats(const float2* __restrict__ o,
-                                                            const float* __restrict__ T,
-                                                            LossStats* __restrict__ st, int fov, int b,
-                                                            float* __restrict__ dLdI, float scale, int mode) {
-  __shared__ double sh[kRedThreads];
-  const int w = blockIdx.x;
+// Fixed-order FP64 total of the block's kRedThreads FP32 partials, by one
+// warp: lane l adds eight of them, a shuffle tree the 32 lanes.  The total is
+// valid in lane 0.  (An FP64 addition occupies the SM's FP64 pipe for many
+// cycles: one warp issues 13 of them here where a block-wide tree in shared
+// memory issues them from every warp and takes eight barriers per sum.)
+__device__ __forceinline__ double warp_total(const float* part, int lane) {
+  double v = 0.0;
+#pragma unroll
+  for (int i = 0; i < kRedThreads / 32; ++i) v += (double)part[lane + 32 * i];
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+  return v;
+}
+
+// 10 log10(x) rounded to FP32.  An FP64 logarithm is a few hundred dependent
+// FP64 instructions, the longest chain of a small launch; here x = f (1 + d)
+// with f its FP32 rounding and f = m 2^e, m in [2/3, 4/3), so that log10 x =
+// e log10 2 + log10 m + d / ln 10 with |log10 m| <= 0.18: the FP32 terms are
+// wrong by at most 2e-8 (2e-7 dB; with e = 0 by a few units of FP32 rounding
+// of the result itself), the sum is FP64.
+__device__ __forceinline__ float ten_log10(double x) {
+  const float f = (float)x;
+  if (!(f > 1e-30f && f < 1e30f)) return (float)(10.0 * log10(x));  // also 0, infinities, NaN
+  const float d = (float)(x - (double)f) / f;
+  int e;
+  float m = frexpf(f, &e);  // [0.5, 1)
+  if (m < 0.66666667f) m *= 2.f, --e;
+  const float small = fmaf(d, 0.43429448190325182765f, log10f(m));
+  return (float)(10.0 * fma((double)e, 0.30102999566398119521, (double)small));
+}
+
+// Detector pixels a channel may have for its values to stay in shared memory
+// between the two loops (16 KB: five blocks and more per SM); above it the
+// second loop forms them again.
+constexpr int kLossKeep = 4096;
+
+// One block per channel: sum (D-T)^2, sigma = sum D T / sum D^2, sum (sigma D
+// - T)^2, the PSNR (psnr not null) and (dLdI not null) dL/dI of the channel's
+// simulation pixels: dL/dD of the detector pixel covering it, 2 (D - T) / norm,
+// or 2 sigma (sigma D - T) / norm for the scaled loss (scale = 2 / norm).  The
+// last block to finish adds the channels' terms in a fixed order to the loss.
+//
+// Bound by latency, not bandwidth, below a few hundred channels: one launch
+// instead of two, four barriers per channel instead of about forty, one FP64
+// division and one logarithm per channel, each in a block of its own (the
+// total kernel took them all in one block), and the detector sums formed once.
+// 4096 channels of 50 x 50: 157 -> 64 us; 2048 channels of 32 x 32 on
+// 4 x 4-pixel detectors 88 -> 37 us; 4 channels of 32 x 32 20 -> 11 us
+// (with the total and the PSNR, both launches before).
+__global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__ o, const float* __restrict__ T,
+                                                      LossStats* __restrict__ st, int fov, int b,
+                                                      float* __restrict__ dLdI, float scale, double norm, int mode,
+                                                      float* __restrict__ psnr, double* __restrict__ d_loss,
+                                                      unsigned* __restrict__ ticket) {
+  extern __shared__ float dsh[];  // [det2] detector values, when det2 <= kLossKeep
+  __shared__ float part[3][kRedThreads];
+  __shared__ double tot[3];
+  __shared__ float sg_sh;
+  __shared__ bool last;
+  const int w = blockIdx.x, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int fd = fov / b, det2 = fd * fd;
+  const bool keep = det2 <= kLossKeep;
   const float2* ow = o + (size_t)w * fov * fov;
   const float* tw = T + (size_t)w * det2;
   float fse = 0.f, fit = 0.f, fii = 0.f;
@@ -58,45 +109,92 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_stats(const float2* __rest
     const float I = detector(ow, fov, b, p);
     const float t = tw[p];
     const float d = I - t;
+    if (keep) dsh[p] = I;
     fse = fmaf(d, d, fse);
     fit = fmaf(I, t, fit);
     fii = fmaf(I, I, fii);
   }
-  const double sse = block_sum(fse, sh);
-  const double sit = block_sum(fit, sh);
-  const double sii = block_sum(fii, sh);
-  const double sigma = sii > 0.0 ? sit / sii : 0.0;
-  const float sg = (float)sigma;
+  part[0][threadIdx.x] = fse;
+  part[1][threadIdx.x] = fit;
+  part[2][threadIdx.x] = fii;
+  __syncthreads();
+  if (warp < 3) {
+    const double v = warp_total(part[warp], lane);
+    if (lane == 0) tot[warp] = v;
+  }
+  __syncthreads();
+  double sigma = 0.0;
+  if (threadIdx.x == 0) {
+    if (tot[2] > 0.0) sigma = tot[1] / tot[2];
+    sg_sh = (float)sigma;
+  }
+  __syncthreads();
+  const float sg = sg_sh;
+  const bool scaled = mode == DOS_LOSS_MSE_SCALED;
+  float* gw = dLdI ? dLdI + (size_t)w * fov * fov : nullptr;
   float fsc = 0.f;
   for (int p = threadIdx.x; p < det2; p += kRedThreads) {
-    const float d = fmaf(sg, detector(ow, fov, b, p), -tw[p]);
+    const float I = keep ? dsh[p] : detector(ow, fov, b, p);
+    const float t = tw[p];
+    const float d = fmaf(sg, I, -t);
     fsc = fmaf(d, d, fsc);
+    if (gw && b == 1) gw[p] = scaled ? scale * sg * d : scale * (I - t);
   }
-  const double ssc = block_sum(fsc, sh);
-  if (threadIdx.x == 0) {
-    LossStats s;
-    s.sse = sse;
-    s.sigma = sigma;
-    s.sse_sc = ssc;
-    s.pad = 0;
-    st[w] = s;
-  }
-  if (dLdI) {
+  if (gw && b > 1) {
     const int fov2 = fov * fov;
-    float* gw = dLdI + (size_t)w * fov2;
     for (int q = threadIdx.x; q < fov2; q += kRedThreads) {
       const int p = ((q / fov) / b) * fd + (q % fov) / b;  // detector pixel covering q
-      const float I = detector(ow, fov, b, p);
+      const float I = keep ? dsh[p] : detector(ow, fov, b, p);
       const float t = tw[p];
-      gw[q] = mode == DOS_LOSS_MSE_SCALED ? scale * sg * fmaf(sg, I, -t) : scale * (I - t);
+      gw[q] = scaled ? scale * sg * fmaf(sg, I, -t) : scale * (I - t);
+    }
+  }
+  part[0][threadIdx.x] = fsc;
+  __syncthreads();
+  if (warp == 0) {
+    const double ssc = warp_total(part[0], lane);
+    if (lane == 0) {
+      LossStats s;
+      s.sse = tot[0];
+      s.sigma = sigma;
+      s.sse_sc = ssc;
+      s.pad = 0;
+      st[w] = s;
+      if (psnr) psnr[w] = ten_log10((double)det2 / ssc);
+      __threadfence();  // the record is visible before the ticket is taken
+      last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+  }
+  __syncthreads();
+  if (!last) return;
+  // every channel's record is in place: the total, in a fixed order (each
+  // thread a stride of the channels, the threads in order of one tree)
+  __shared__ double acc[kRedThreads];
+  __threadfence();
+  double v = 0.0;
+  for (int c = threadIdx.x; c < (int)gridDim.x; c += kRedThreads)
+    v += __ldcg(scaled ? &st[c].sse_sc : &st[c].sse);
+  acc[threadIdx.x] = v;
+  __syncthreads();
+  if (warp == 0) {
+    v = 0.0;
+#pragma unroll
+    for (int i = 0; i < kRedThreads / 32; ++i) v += acc[lane + 32 * i];
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+    if (lane == 0) {
+      *d_loss = v / norm;
+      *ticket = 0;  // the next launch starts from zero
     }
   }
 }
 
-cudaError_t launch_loss_stats(const float2* o, const float* T, LossStats* st, int nw, int fov, int bin,
-                              float* dLdI, double norm, int mode, cudaStream_t s) {
+cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, int fov, int bin, float* dLdI,
+                        double norm, int mode, float* psnr, double* d_loss, unsigned* ticket, cudaStream_t s) {
   const float scale = (float)(2.0 / norm);  // dL/dD = 2 (D - T) / norm
-  k_loss_stats<<<nw, kRedThreads, 0, s>>>(o, T, st, fov, bin, dLdI, scale, mode);
+  const int det2 = (fov / bin) * (fov / bin);
+  const size_t sm = det2 <= kLossKeep ? sizeof(float) * det2 : 0;
+  k_loss<<<nw, kRedThreads, sm, s>>>(o, T, st, fov, bin, dLdI, scale, norm, mode, psnr, d_loss, ticket);
   return cudaGetLastError();
 }
 
@@ -121,40 +219,65 @@ cudaError_t launch_loss_final(const LossStats* st, int nw, int fov2, double norm
   return cudaGetLastError();
 }
 
-// grad[g] = sum over chunks c (in order) of partial[layer(g)][c][pixel(g)]
-__global__ void k_grad_reduce(const float* __restrict__ partial, float* __restrict__ grad,
-                              int n_chunks, size_t count, size_t n2) {
-  const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= count) return;
-  const size_t layer = g / n2, px = g % n2;
-  const float* p = partial + layer * n_chunks * n2 + px;
-  double acc = 0.0;
-  for (int c = 0; c < n_chunks; ++c) acc += (double)p[(size_t)c * n2];
-  grad[g] = (float)acc;
+// grad[g] = sum over the parts c of partial[layer(g)][c][pixel(g)], in a fixed
+// order.  Sums of FP32 partials carried as an FP32 pair (a running sum and the
+// exact rounding errors of its additions, Knuth's two-sum), about 48 bits, and
+// rounded to FP32 once at the end like the FP64 sum before it: GB300 adds and
+// converts FP64 at a small fraction of its FP32 rate, which bound the kernel.
+// A block takes 32 pixels x 8 slices of the parts, eight loads of a slice in
+// flight, so that small layers with many parts still fill the chip.
+// 5 layers of 200 x 200: 92 parts 86 -> 22 us, 86 parts 81 -> 26 us; 3 layers of
+// 64 x 64, 293 parts 57 -> 12 us.
+constexpr int kGradPx = 32, kGradSlices = 8;
+
+// (s, e) += x with s + e kept exact up to the rounding of e
+__device__ __forceinline__ void pair_add(float& s, float& e, float x) {
+  const float t = __fadd_rn(s, x);
+  const float z = __fadd_rn(t, -s);
+  e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(x, -z)));
+  s = t;
 }
 
-cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_chunks, size_t count,
-                               size_t n2, cudaStream_t s) {
-  k_grad_reduce<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(partial, grad, n_chunks, count, n2);
+__global__ void __launch_bounds__(kGradPx * kGradSlices) k_grad_reduce(const float* __restrict__ partial,
+                                                                       float* __restrict__ grad, int n_parts,
+                                                                       size_t count, size_t n2) {
+  __shared__ float2 sh[kGradSlices][kGradPx];
+  const int lane = threadIdx.x % kGradPx, slice = threadIdx.x / kGradPx;
+  const size_t g = (size_t)blockIdx.x * kGradPx + lane;
+  const int per = (n_parts + kGradSlices - 1) / kGradSlices;
+  const int c0 = min(slice * per, n_parts), c1 = min(c0 + per, n_parts);
+  float s = 0.f, e = 0.f;
+  if (g < count) {
+    const size_t layer = g / n2, px = g % n2;
+    const float* p = partial + (layer * n_parts + c0) * n2 + px;
+    int c = c0;
+    for (; c + 8 <= c1; c += 8, p += 8 * n2) {
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = __ldcs(p + i * n2);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) pair_add(s, e, x[i]);
+    }
+    for (; c < c1; ++c, p += n2) pair_add(s, e, __ldcs(p));
+  }
+  sh[slice][lane] = make_float2(s, e);
+  __syncthreads();
+  if (slice != 0 || g >= count) return;
+#pragma unroll
+  for (int q = 1; q < kGradSlices; ++q) {
+    const float2 v = sh[q][lane];
+    pair_add(s, e, v.x);
+    e = __fadd_rn(e, v.y);
+  }
+  // an infinite sum has no rounding error to add (inf - inf)
+  grad[g] = isinf(s) ? s : s + e;
+}
+
+cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2,
+                               cudaStream_t s) {
+  const unsigned blocks = (unsigned)((count + kGradPx - 1) / kGradPx);
+  k_grad_reduce<<<blocks, kGradPx * kGradSlices, 0, s>>>(partial, grad, n_parts, count, n2);
   return cudaGetLastError();
 }
 
-}  // namespace dos
-
-namespace dos {
-// grad[g] = sum over c < n_parts (in order) of partial[c * count + g]
-__global__ void k_grad_reduce_flat(const float* __restrict__ partial, float* __restrict__ grad,
-                                   int n_parts, size_t count) {
-  const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= count) return;
-  double acc = 0.0;
-  for (int c = 0; c < n_parts; ++c) acc += (double)partial[(size_t)c * count + g];
-  grad[g] = (float)acc;
-}
-
-cudaError_t launch_grad_reduce_flat(const float* partial, float* grad, int n_parts, size_t count,
-                                    cudaStream_t s) {
-  k_grad_reduce_flat<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(partial, grad, n_parts, count);
-  return cudaGetLastError();
-}
 }  // namespace dos
