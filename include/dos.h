@@ -83,9 +83,8 @@ enum {
  *    (a column tile by a TMA tensor copy, or the next channel's rows by
  *    bulk-async copies) into shared memory while computing the current one;
  *    the adjoint row pass stages both the spectra rows and the checkpoint
- *    rows. A pass whose stage does not fit (column: 128 N bytes + exchange
- *    within 227 KB, N <= 256) or whose rows are not 16-byte multiples (odd N)
- *    runs the plain kernel.
+ *    rows. A pass whose stage does not fit (column: N <= 256) or whose rows
+ *    are not 16-byte multiples (odd N) runs the plain kernel.
  *  DOS_PATH_FUSED: one persistent launch per sweep (forward or adjoint) in
  *    which a thread-block cluster carries one channel at a time through every
  *    gap with the field held in distributed shared memory (needs N <= M/2 and
@@ -251,7 +250,11 @@ DOS_API int dos_loss_noalloc(const float *d_I, const float *d_T, int n_lambda, i
  * which is how the engine applies it (exact up to the layer window).
  * Applies to every later dos_forward / dos_backward / dos_step / dos_propagate
  * until changed; a backward must follow a forward with the same setting.
- * The first call builds a table of sqrt(|q|) (N_w (M/2+1)^2 floats, FP64 roots).
+ * The first call builds a table of sqrt(|q|) (N_w (M/2+2)^2 floats, FP64 roots;
+ * the multi-pass paths keep what their rounding left as well) and, on the
+ * multi-pass paths, reserves K+1 transfer tables for the gaps whose length
+ * changes (one where those do not fit, none where that does not either: the
+ * column passes are then slower).
  * Errors: DOS_ERR_ARG, DOS_ERR_OOM, DOS_ERR_CUDA.
  */
 DOS_API int dos_set_misalignment(dos_ctx *ctx, const double *h_disp);

@@ -184,15 +184,32 @@ struct dos_ctx {
   double* d_lam = nullptr;      // wavelengths on the device (kept for the root table)
   float* sq = nullptr;          // signed sqrt(|q|) quadrant table, built on first use
   bool mis_on = false;
-  std::vector<float> mis;       // (K+1) x 3 per gap: lateral shift x, y and length change [m]
+  float* sq_lo = nullptr;       // what the roots' rounding to FP32 left (with hmis)
+  std::vector<double> mis;      // (K+1) x 3 per gap: lateral shift x, y and length change [m]
   long mis_gen = 0;
+  // transfer tables with the displaced gaps' length changes, for the column
+  // passes: [mis_tables][nw][hs][hs], gap g's in slot g % mis_tables; one per
+  // gap where they fit, else one that every pass rebuilds, else none (the plain
+  // kernel then forms the factor from sq).  A forward builds its gaps' tables
+  // anew; the adjoint of the same displacement reads them.
+  float2* hmis = nullptr;
+  int mis_tables = 0;
+  long mis_built = -1;        // mis_gen of the tables in place (mis_tables > 1)
+  CUtensorMap tmap_Hm;        // hmis as [mis_tables * nw][hs][hs], box as tmap_H
   dos::Misalign gap_mis(int g) const {
     dos::Misalign m;
-    m.sq = mis_on ? sq : nullptr;
-    m.df = (float)(1.0 / ((double)this->m * pitch));
-    m.ax = mis_on ? mis[3 * g] : 0.f;
-    m.ay = mis_on ? mis[3 * g + 1] : 0.f;
-    m.dz = mis_on ? mis[3 * g + 2] : 0.f;
+    std::memset(&m, 0, sizeof(m));
+    const double df = 1.0 / ((double)this->m * pitch);
+    m.df = (float)df;
+    if (!mis_on) return m;
+    auto pair = [](double v) { return make_float2((float)v, (float)(v - (double)(float)v)); };
+    m.sq = sq;
+    m.ax = (float)mis[3 * g];
+    m.ay = (float)mis[3 * g + 1];
+    m.dz = (float)mis[3 * g + 2];
+    m.sx = pair(df * mis[3 * g]);
+    m.sy = pair(df * mis[3 * g + 1]);
+    m.dz2 = pair(mis[3 * g + 2]);
     return m;
   }
   // split-BF16 DFT-GEMM path
@@ -253,7 +270,7 @@ struct dos_ctx {
     a.err = d_err;
     a.tmap = have_tmap ? &tmap_S : nullptr;
     a.tmap_rows = n;
-    a.hmap = (have_tmap && ops->h_box_cols > 0) ? &tmap_H : nullptr;
+    a.hmap = have_tmap ? &tmap_H : nullptr;
     return a;
   }
 };
@@ -310,18 +327,37 @@ int choose_path(dos_ctx* x, int requested);
 // columns, n rows, 1 channel} (tmap_S) or {col_group, fov, 1} (tmap_F); the
 // transfer tables as [slots * nw][hs][hs] (rows of hs = m/2 + 2 entries, a
 // 16-byte multiple), box {h_box_cols, h_box_rows, 1} (tmap_H: whole table rows,
-// the quadrant being symmetric), when the column kernel stages an H tile.
+// the quadrant being symmetric).
 // A driver without the entry point leaves the plain column kernel in use.
-int make_spectra_map(dos_ctx* x) {
-  x->have_tmap = false;
-  if (x->n > 256) return DOS_OK;  // one box covers at most 256 rows
+PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
   if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess || !fn) {
+      q != cudaDriverEntryPointSuccess) {
     (void)cudaGetLastError();
-    return DOS_OK;
+    return nullptr;
   }
+  return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+}
+
+int make_table_map(dos_ctx* x, CUtensorMap* map, float2* tables, int count) {
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const cuuint64_t hdims[3] = {(cuuint64_t)x->hs, (cuuint64_t)x->hs, (cuuint64_t)count * x->nw};
+  const cuuint64_t hstrides[2] = {(cuuint64_t)x->hs * 8, (cuuint64_t)x->hs * x->hs * 8};
+  const cuuint32_t hbox[3] = {(cuuint32_t)x->ops->h_box_cols, (cuuint32_t)x->ops->h_box_rows, 1};
+  const CUresult r = map_encoder()(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, tables, hdims, hstrides, hbox, estr,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    return fail(DOS_ERR_CUDA, "cuTensorMapEncodeTiled(transfer tables) failed: " + std::to_string((int)r));
+  return DOS_OK;
+}
+
+int make_spectra_map(dos_ctx* x) {
+  x->have_tmap = false;
+  if (x->n > 256) return DOS_OK;  // one box covers at most 256 rows
+  const PFN_cuTensorMapEncodeTiled_v12000 encode = map_encoder();
+  if (!encode) return DOS_OK;
   const cuuint64_t dims[3] = {(cuuint64_t)x->m, (cuuint64_t)x->n, (cuuint64_t)x->nw};
   const cuuint64_t strides[2] = {(cuuint64_t)x->m * 8, (cuuint64_t)x->n * x->m * 8};
   const cuuint32_t estr[3] = {1, 1, 1};
@@ -329,24 +365,15 @@ int make_spectra_map(dos_ctx* x) {
   CUtensorMap* maps[2] = {&x->tmap_S, &x->tmap_F};
   for (int i = 0; i < 2; ++i) {  // both are encoded, also when fov == n
     const cuuint32_t box[3] = {(cuuint32_t)x->ops->col_group, (cuuint32_t)box_rows[i], 1};
-    const CUresult r = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)(
+    const CUresult r = encode(
         maps[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, x->S, dims, strides, box, estr,
         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
       return fail(DOS_ERR_CUDA, "cuTensorMapEncodeTiled(row spectra) failed: " + std::to_string((int)r));
   }
-  if (x->ops->h_box_cols > 0) {  // the column kernel of this size stages an H tile
-    const cuuint64_t hdims[3] = {(cuuint64_t)x->hs, (cuuint64_t)x->hs, (cuuint64_t)x->n_slots * x->nw};
-    const cuuint64_t hstrides[2] = {(cuuint64_t)x->hs * 8, (cuuint64_t)x->hs * x->hs * 8};
-    const cuuint32_t hbox[3] = {(cuuint32_t)x->ops->h_box_cols, (cuuint32_t)x->ops->h_box_rows, 1};
-    const CUresult r = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)(
-        &x->tmap_H, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, x->Hq, hdims, hstrides, hbox, estr,
-        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS)
-      return fail(DOS_ERR_CUDA, "cuTensorMapEncodeTiled(transfer tables) failed: " + std::to_string((int)r));
-  }
+  int rc = make_table_map(x, &x->tmap_H, x->Hq, x->n_slots);
+  if (rc) return rc;
   x->have_tmap = true;
   return DOS_OK;
 }
@@ -632,12 +659,43 @@ dos::PassArgs range_args(const dos_ctx* c, int w0, int w1) {
   return a;
 }
 
-// transfer table and displacement table of gap g for the channels from w0
-const float2* range_hq(const dos_ctx* c, int g, int w0) { return c->hq_slot(g) + (size_t)w0 * c->hs * c->hs; }
-dos::Misalign range_mis(const dos_ctx* c, int g, int w0) {
-  dos::Misalign m = c->gap_mis(g);
-  if (m.sq) m.sq += (size_t)w0 * c->hs * c->hs;
-  return m;
+// The transfer table of gap g for the column passes over a's channels (from
+// w0) and, with displaced layers, what the table does not hold.  A gap whose
+// length changes gets a table of its own; its launch goes to L (kind) first
+// when `build` is set or the table in place is another one.
+void use_gap(dos_ctx* c, dos::PassArgs& a, int g, int w0, bool build, int kind, std::vector<Launch>& L) {
+  const size_t hs2 = (size_t)c->hs * c->hs;
+  a.Hq = c->hq_slot(g) + (size_t)w0 * hs2;
+  a.hmap = c->have_tmap ? &c->tmap_H : nullptr;
+  a.hmap_z0 = c->gap_slot[g] * c->nw + w0;
+  a.mis = c->gap_mis(g);
+  a.displaced = c->mis_on && (a.mis.ax != 0.f || a.mis.ay != 0.f);
+  if (!c->mis_on || a.mis.dz == 0.f) {
+    a.mis.sq = nullptr;
+    return;
+  }
+  const float *sq = c->sq + (size_t)w0 * hs2, *sq_lo = c->sq_lo + (size_t)w0 * hs2;
+  if (c->mis_tables == 0) {
+    a.mis.sq = sq;
+    a.displaced = true;
+    return;
+  }
+  const int slot = g % c->mis_tables;
+  float2* table = c->hmis + ((size_t)slot * c->nw + w0) * hs2;
+  if (build || c->mis_tables == 1 || c->mis_built != c->mis_gen) {
+    const float2 *hq = a.Hq, dz = a.mis.dz2;
+    const size_t count = (size_t)a.nw * hs2;
+    L.push_back({kind,
+                 [table, hq, sq, sq_lo, dz, count](cudaStream_t s) {
+                   return dos::launch_longer_table(table, hq, sq, sq_lo, dz, count, s);
+                 },
+                 "displaced gap's transfer table"});
+  }
+  a.Hq = table;
+  a.hmap = c->have_tmap ? &c->tmap_Hm : nullptr;
+  a.hmap_z0 = slot * c->nw + w0;
+  a.mis.sq = nullptr;
+  a.mis.dz = 0.f;
 }
 
 // forward: [gap 0 column pass,] K x (row pass + column pass), output row pass
@@ -648,8 +706,7 @@ std::vector<Launch> forward_launches(dos_ctx* c, const float* d_h, float* d_I, i
   dos::PassArgs a = range_args(c, w0, w1);
   if (!c->ckpt1_is_v1) {
     // the aperture field has the separable spectrum Arow[ky] Arow[kx]
-    a.Hq = range_hq(c, 0, w0);
-    a.mis = range_mis(c, 0, w0);
+    use_gap(c, a, 0, w0, true, DOS_KERNEL_COLUMN_FORWARD, L);
     a.out_r0 = 0;
     a.out_r1 = c->n;
     L.push_back({DOS_KERNEL_COLUMN_FORWARD, [op, a](cudaStream_t s) { return op->col(a, false, true, s); },
@@ -671,9 +728,7 @@ std::vector<Launch> forward_launches(dos_ctx* c, const float* d_h, float* d_I, i
                    [op, a, brow, sv](cudaStream_t s) { return brow ? op->bulk_row_fwd(a, sv, s) : op->row_fwd(a, sv, s); },
                    "forward row pass"});
     }
-    a.Hq = range_hq(c, l, w0);
-    a.hmap_z0 = c->gap_slot[l] * c->nw + w0;
-    a.mis = range_mis(c, l, w0);
+    use_gap(c, a, l, w0, true, DOS_KERNEL_COLUMN_FORWARD, L);
     a.in_r0 = 0;
     a.in_r1 = c->n;
     a.out_r0 = l == c->K ? c->of : 0;
@@ -699,9 +754,7 @@ std::vector<Launch> backward_launches(dos_ctx* c, const float* d_h, const float*
   a.dLdI = d_dLdI + (size_t)w0 * c->fov * c->fov;
   L.push_back({DOS_KERNEL_ROW_SEED, [op, a](cudaStream_t s) { return op->row_seed(a, s); }, "adjoint seed row pass"});
   for (int l = c->K; l >= 1; --l) {
-    a.Hq = range_hq(c, l, w0);
-    a.hmap_z0 = c->gap_slot[l] * c->nw + w0;
-    a.mis = range_mis(c, l, w0);
+    use_gap(c, a, l, w0, false, DOS_KERNEL_COLUMN_ADJOINT, L);
     a.in_r0 = l == c->K ? c->of : 0;
     a.in_r1 = l == c->K ? c->of + c->fov : c->n;
     a.tmap = !c->have_tmap ? nullptr : l == c->K ? &c->tmap_F : &c->tmap_S;
@@ -790,7 +843,9 @@ int run_forward(dos_ctx* c, const float* d_h, float* d_I, int save) {
   // gap 0 is the create-time table v1 unless the layers are displaced (then the
   // first gap depends on layer 1's displacement)
   c->ckpt1_is_v1 = c->v1 && !c->mis_on;
-  return run_launches(c, forward_launches(c, d_h, d_I, save, 0, c->nw));
+  const int rc = run_launches(c, forward_launches(c, d_h, d_I, save, 0, c->nw));
+  c->mis_built = (!rc && c->mis_on && c->mis_tables > 1) ? c->mis_gen : -1;
+  return rc;
 }
 
 int run_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dLdh) {
@@ -1163,17 +1218,29 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
   for (int i = 0; i < 3 * c->K; ++i)
     if (!std::isfinite(disp[i])) return fail(DOS_ERR_ARG, "displacements must be finite");
   if (!c->sq) {
-    if ((rc = c->alloc(&c->sq, (size_t)c->nw * c->hs * c->hs, "root table"))) return rc;
-    DOS_CUDA(dos::launch_sqtable(c->sq, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream), "root table");
+    const size_t count = (size_t)c->nw * c->hs * c->hs;
+    if ((rc = c->alloc(&c->sq, count, "root table"))) return rc;
+    // the column passes' tables: where they do not fit, the plain kernel does without
+    if ((c->path == DOS_PATH_MULTIPASS || c->path == DOS_PATH_MULTIPASS_BULK) &&
+        c->alloc(&c->sq_lo, count, "root table") == DOS_OK) {
+      for (int tables : {c->K + 1, 1}) {
+        if (c->alloc(&c->hmis, tables * count, "displaced transfer tables") != DOS_OK) continue;
+        if (c->have_tmap && (rc = make_table_map(c, &c->tmap_Hm, c->hmis, tables))) return rc;
+        c->mis_tables = tables;
+        break;
+      }
+    }
+    DOS_CUDA(dos::launch_sqtable(c->sq, c->sq_lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream),
+             "root table");
   }
   // layer l (1..K) displaced by D_l; planes 0 (aperture) and K+1 (detector) fixed:
   // gap g carries the lateral shift D_g - D_{g+1} and the length change dz_{g+1} - dz_g
-  c->mis.assign(3 * (c->K + 1), 0.f);
+  c->mis.assign(3 * (c->K + 1), 0.0);
   auto D = [&](int l, int k) { return (l >= 1 && l <= c->K) ? disp[3 * (l - 1) + k] : 0.0; };
   for (int g = 0; g <= c->K; ++g) {
-    c->mis[3 * g] = (float)(D(g, 0) - D(g + 1, 0));
-    c->mis[3 * g + 1] = (float)(D(g, 1) - D(g + 1, 1));
-    c->mis[3 * g + 2] = (float)(D(g + 1, 2) - D(g, 2));
+    c->mis[3 * g] = D(g, 0) - D(g + 1, 0);
+    c->mis[3 * g + 1] = D(g, 1) - D(g + 1, 1);
+    c->mis[3 * g + 2] = D(g + 1, 2) - D(g, 2);
   }
   c->mis_on = true;
   return DOS_OK;
@@ -1313,21 +1380,22 @@ DOS_API int dos_propagate(dos_ctx* c, int gap, const float* d_in, float* d_out, 
   if (gap < 0 || gap > c->K) return fail(DOS_ERR_ARG, "gap must be in [0, n_layers]");
   if (!d_in || !d_out || d_in == d_out) return fail(DOS_ERR_ARG, "d_in and d_out must be distinct non-NULL");
   const dos::PassOps* op = c->ops;
-  c->launches = 0;
   c->have_fwd = c->have_ckpt = c->have_loss = false;  // the spectra buffer is reused
-  dos::PassArgs a = c->base();
+  std::vector<Launch> L;
+  dos::PassArgs a = range_args(c, 0, c->nw);
   a.fin = reinterpret_cast<const float2*>(d_in);
   a.fout = reinterpret_cast<float2*>(d_out);
-  a.Hq = c->hq_slot(gap);
-  a.mis = c->gap_mis(gap);
+  use_gap(c, a, gap, 0, true, DOS_KERNEL_COLUMN_FORWARD, L);
   a.in_r0 = 0;
   a.in_r1 = c->n;
   a.out_r0 = 0;
   a.out_r1 = c->n;
+  for (const Launch& l : L) DOS_CUDA(l.go(c->stream), l.what);
   DOS_CUDA(op->row_in(a, c->stream), "propagate row pass");
-  DOS_CUDA(op->col(a, adjoint != 0, false, c->stream), "propagate column pass");
+  if (c->bulk & kBulkCol) DOS_CUDA(op->bulk_col(a, adjoint != 0, c->stream), "propagate column pass");
+  else DOS_CUDA(op->col(a, adjoint != 0, false, c->stream), "propagate column pass");
   DOS_CUDA(op->row_back(a, c->stream), "propagate back row pass");
-  c->launches = 3;
+  c->launches = 3 + (int)L.size();
   return DOS_OK;
 }
 

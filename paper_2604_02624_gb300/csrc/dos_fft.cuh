@@ -542,11 +542,14 @@ struct Line {
   // reserve for it in shared memory
   static constexpr int TWP = twiddle_pitch(P), TWS = Q * TWP;
   static_assert(P % T == 0 && Q % T == 0, "T must divide P and Q");
-  // TR: the exchange matrix stored transposed (entry (q, k1) at k1 * RP + q).
-  // For a square line (P = Q = T) step 1 of thread t writes exactly the
-  // entries that step 2 of thread t read in the other layout, so two line
-  // DFTs in alternating layouts need no barrier between them.
+  // TR: the exchange matrix stored in transposed T x T blocks: entry (q, k1),
+  // q = u + T j, lives at row k1 + T j, column u (a square line, P = Q = T, has
+  // one block: the plain transpose).  With P = T (ALT) step 1 of thread t
+  // writes exactly the entries that step 2 of thread t read in the other
+  // layout, so two line DFTs in alternating layouts need no barrier between
+  // them, and neither does the next pair.
   static constexpr bool SQUARE = P == Q && T == P;
+  static constexpr bool ALT = P == T;
 
   // Step 1: the Q/T sub-DFTs of length P owned by thread t (q = t + T*j),
   // twiddled and written to the exchange matrix z[q][k1].
@@ -554,11 +557,12 @@ struct Line {
   // ZR: pitch of the exchange matrix (RP, or an even pitch for kernels whose
   // lines are laid out so that 16-byte accesses are conflict-free: then a
   // thread's entries k1, k1 + 1 (k1 even) of a row are one 16-byte store, and
-  // in step 2 of the transposed layout q, q + 1 are one 16-byte load).
+  // in step 2 of the transposed layout two neighbours of a row are one 16-byte
+  // load).
   template <bool INV, int NZP = P, bool PK = false, bool TR = false, int ZR = RP>
   DOS_HD static void step1(const float2 (&r)[E], int t, float2* z, const float2* tw) {
-    static_assert(!TR || SQUARE, "the transposed exchange is for square lines");
-    static_assert(ZR >= P && (!TR || ZR >= Q), "the pitch holds a row");
+    static_assert(!TR || ALT, "the transposed exchange needs one column per thread");
+    static_assert(ZR >= P, "the pitch holds a row");
     constexpr bool V = !TR && ZR % 2 == 0;  // paired row stores
     static_for<0, QJ>([&](auto jj) {
       constexpr int j = jj;
@@ -567,7 +571,7 @@ struct Line {
       dft<P, INV, NZP, P, PK>(a);
       const int q = t + T * j;
       const float4* twq = reinterpret_cast<const float4*>(tw + q * TWP);  // twiddle pairs
-      float2* zq = TR ? z + q : z + q * ZR;
+      float2* zq = TR ? z + T * j * ZR + t : z + q * ZR;
       constexpr int ZK = TR ? ZR : 1;  // stride of k1
       static_for<0, (P + 1) / 2>([&](auto pp) {
         constexpr int k0 = 2 * pp, k1 = 2 * pp + 1;
@@ -595,21 +599,22 @@ struct Line {
   // NOQ: leading outputs of each sub-DFT that are needed (cropping).
   template <bool INV, int NOQ = Q, bool PK = false, bool TR = false, int ZR = RP>
   DOS_HD static void step2(float2 (&r)[E], int t, const float2* z) {
-    constexpr bool V = TR && ZR % 2 == 0;  // paired row loads
+    constexpr bool V = TR && ZR % 2 == 0 && T % 2 == 0;  // paired row loads
     static_for<0, PJ>([&](auto jj) {
       constexpr int j = jj;
       const int k1 = t + T * j;
       float2 b[Q];
       if constexpr (V) {
-        const float4* zr = reinterpret_cast<const float4*>(z + k1 * ZR);
-        static_for<0, Q / 2>([&](auto qq) {
-          const float4 v = zr[qq];
-          b[2 * qq] = make_float2(v.x, v.y);
-          b[2 * qq + 1] = make_float2(v.z, v.w);
+        static_for<0, QJ>([&](auto bb) {
+          const float4* zr = reinterpret_cast<const float4*>(z + (k1 + T * bb) * ZR);
+          static_for<0, T / 2>([&](auto uu) {
+            const float4 v = zr[uu];
+            b[T * bb + 2 * uu] = make_float2(v.x, v.y);
+            b[T * bb + 2 * uu + 1] = make_float2(v.z, v.w);
+          });
         });
-        if constexpr (Q % 2 == 1) b[Q - 1] = z[k1 * ZR + Q - 1];
       } else {
-        static_for<0, Q>([&](auto qq) { b[qq] = TR ? z[k1 * ZR + qq] : z[qq * ZR + k1]; });
+        static_for<0, Q>([&](auto qq) { b[qq] = TR ? z[(k1 + qq / T * T) * ZR + qq % T] : z[qq * ZR + k1]; });
       }
       dft<Q, INV, Q, NOQ, PK>(b);
       static_for<0, NOQ>([&](auto k2) { r[j + PJ * k2] = b[k2]; });

@@ -25,12 +25,33 @@ struct Misalign {
   const float* sq;   // [nw][hs][hs] signed sqrt(|q|) [1/m], or null when off
   float df;          // DFT bin spacing 1 / (M pitch) [1/m]
   float ax, ay, dz;  // this gap [m]
+  // the same as FP32 pairs (x: value, y: what its rounding left): the shift's
+  // phase per bin, df ax and df ay [cycles], and the length change [m]
+  float2 sx, sy, dz2;
 };
+
+// signed index of bin k of an M-point grid
+__device__ __forceinline__ int signed_bin(int k, int m) { return k < m / 2 ? k : k - m; }
+
+// a * b reduced to [-1/2, 1/2] cycles, to about 1e-8: b is an FP32 pair, the
+// product's rounding error is kept
+__device__ __forceinline__ float cycles(float a, float2 b) {
+  const float p = a * b.x;
+  const float e = fmaf(a, b.y, fmaf(a, b.x, -p));
+  return (p - rintf(p)) + e;
+}
+
+// exp(-2 pi j k s): the phase of a lateral shift at signed bin k, s cycles per bin
+__device__ __forceinline__ float2 shift_phase(int k, float2 s) {
+  float sn, cs;
+  sincospif(-2.0f * cycles((float)k, s), &sn, &cs);
+  return make_float2(cs, sn);
+}
 
 // exp(-2 pi j (fx ax + fy ay)) * H(dz) for bins (ky, kx) of an M-point grid
 __device__ __forceinline__ float2 misalign_factor(const Misalign& g, int ky, int kx, int m, float sq) {
-  const float fx = (float)(kx < m / 2 ? kx : kx - m) * g.df;
-  const float fy = (float)(ky < m / 2 ? ky : ky - m) * g.df;
+  const float fx = (float)signed_bin(kx, m) * g.df;
+  const float fy = (float)signed_bin(ky, m) * g.df;
   float ph = -fmaf(fx, g.ax, fy * g.ay);  // cycles
   float amp = 1.0f;
   if (sq >= 0.0f) ph = fmaf(g.dz, sq, ph);
@@ -60,7 +81,8 @@ struct PassArgs {
   int out_r0, out_r1;     // column pass: rows stored on output
   int chunk;              // channels per block of the adjoint row pass
   int n_chunks;
-  Misalign mis;           // misaligned layers (mis.sq null: none)
+  bool displaced;         // column pass: the gap carries a displacement that Hq does not hold (mis)
+  Misalign mis;           // its lateral shift; and, with mis.sq, its length change (plain kernel only)
   int* err;               // set to 1 by a bulk-copy pass whose bounded wait expired
   int stall;              // fault injection (tests): 1 = the bulk pass expects bytes that are never
                           // copied; 2 = its copies land but odd threads give up their first wait;
@@ -106,8 +128,13 @@ int supported_m_list(int* out, int cap);
 cudaError_t launch_htable(float2* Hq, const double* d_lambda, int nw, double z, double n_medium,
                           double pitch, int m, int hs, int evanescent, cudaStream_t s);
 cudaError_t launch_arow(float2* arow, int m, int offset, int width, cudaStream_t s);
-cudaError_t launch_sqtable(float* sq, const double* d_lambda, int nw, double n_medium, double pitch, int m, int hs,
+// sq_lo: what the rounding of sq left (null: not wanted)
+cudaError_t launch_sqtable(float* sq, float* sq_lo, const double* d_lambda, int nw, double n_medium, double pitch, int m, int hs,
                            cudaStream_t s);
+// out = Hq * H(dz) over the count quadrant entries of the channels (from the
+// signed roots, FP32 value and remainder): the table of a gap that is dz longer
+cudaError_t launch_longer_table(float2* out, const float2* Hq, const float* sq, const float* sq_lo, float2 dz,
+                                size_t count, cudaStream_t s);
 cudaError_t launch_twiddles(float2* tw, int P, int Q, int TWP, int m, cudaStream_t s);
 cudaError_t launch_chan(ChanConst* chan, const double* d_lambda, const double* d_nidx,
                         const double* d_kappa, int nw, double n_medium, double h_base,

@@ -82,7 +82,10 @@ struct Pass {
   }
 
   // ------------------------------------------------------------ column pass
-  template <bool ADJ, bool APERTURE>
+  // MIS: displaced layers.  Kernels of their own: the displacement's phase,
+  // formed per element, would triple the code of the loop that all aligned
+  // designs run, and with it the instruction-cache misses.
+  template <bool ADJ, bool APERTURE, bool MIS>
   __device__ static void col(const PassArgs& a) {
     extern __shared__ __align__(16) float2 smem[];
     float2* tw = smem;
@@ -110,14 +113,16 @@ struct Pass {
       LF::template fft<false, NZF, LF::Q, true, PKC>(r, t, z, tw);
     }
     const float2* Hw = a.Hq + (size_t)w * a.hs * a.hs;
-    const float* Sw = a.mis.sq ? a.mis.sq + (size_t)w * a.hs * a.hs : nullptr;
+    const float* Sw = MIS && a.mis.sq ? a.mis.sq + (size_t)w * a.hs * a.hs : nullptr;
     const int bc = min(cc, M - cc);
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       const int k = t + T * i;
       const size_t qi = (size_t)min(k, M - k) * a.hs + bc;
       float2 hv = Hw[qi];
-      if (Sw) hv = cmul(hv, misalign_factor(a.mis, k, cc, M, Sw[qi]));
+      if constexpr (MIS)
+        hv = cmul(hv, Sw ? misalign_factor(a.mis, k, cc, M, Sw[qi])
+                         : cmul(shift_phase(signed_bin(k, M), a.mis.sy), shift_phase(signed_bin(cc, M), a.mis.sx)));
       r[i] = ADJ ? cmulc(r[i], hv) : cmul(r[i], hv);
     }
     LF::template fft<true, LF::P, NOI, true, PKC>(r, t, z, tw);
@@ -376,9 +381,9 @@ constexpr int pass_min_blocks() { return LF::E <= 20 ? 3 : 1; }
 template <class LF, bool HALF>
 constexpr int col_min_blocks() { return HALF && LF::M == 400 ? 3 : 0; }
 
-template <class LF, bool HALF, bool ADJ, bool APERTURE>
+template <class LF, bool HALF, bool ADJ, bool APERTURE, bool MIS>
 __global__ void __launch_bounds__(LF::T * Pass<LF>::COLL, col_min_blocks<LF, HALF>()) k_col(PassArgs a) {
-  Pass<LF, HALF>::template col<ADJ, APERTURE>(a);
+  Pass<LF, HALF>::template col<ADJ, APERTURE, MIS>(a);
 }
 template <class LF, bool HALF, bool SAVE>
 __global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, pass_min_blocks<LF>()) k_row_fwd(PassArgs a) {
@@ -434,10 +439,13 @@ struct PassLaunch {
   static cudaError_t col_h(const PassArgs& a, bool adj, bool ap, cudaStream_t s) {
     const dim3 g((LF::M + PS::COLL - 1) / PS::COLL, a.nw);
     const size_t sm = PS::smem_bytes(PS::COLL);
-    if (ap) return adj ? launch_k(k_col<LF, H, true, true>, g, CT, sm, a, s)
-                       : launch_k(k_col<LF, H, false, true>, g, CT, sm, a, s);
-    return adj ? launch_k(k_col<LF, H, true, false>, g, CT, sm, a, s)
-               : launch_k(k_col<LF, H, false, false>, g, CT, sm, a, s);
+    // the aperture field is only ever propagated forward
+    if (ap) return a.displaced ? launch_k(k_col<LF, H, false, true, true>, g, CT, sm, a, s)
+                               : launch_k(k_col<LF, H, false, true, false>, g, CT, sm, a, s);
+    if (a.displaced) return adj ? launch_k(k_col<LF, H, true, false, true>, g, CT, sm, a, s)
+                                : launch_k(k_col<LF, H, false, false, true>, g, CT, sm, a, s);
+    return adj ? launch_k(k_col<LF, H, true, false, false>, g, CT, sm, a, s)
+               : launch_k(k_col<LF, H, false, false, false>, g, CT, sm, a, s);
   }
   static cudaError_t col(const PassArgs& a, bool adj, bool ap, cudaStream_t s) {
     return half(a) ? col_h<true>(a, adj, ap, s) : col_h<false>(a, adj, ap, s);

@@ -108,49 +108,53 @@ struct PassBulk {
   static constexpr int SR = row_stage_stride(M);  // even: every staged row starts 16-byte aligned
   static_assert(SR % 2 == 0 && SR >= M, "staged rows must be 16-byte aligned and hold M values");
   static_assert(Pass<LF>::RZL >= LF::ZS, "exchange buffers must not overlap");
-  static constexpr int CT = T * COLL, RT = T * RL;
+  static constexpr int RT = T * RL;
 
   // ------------------------------------------------------------ column pass
-  // An item is a mirrored pair of column groups of one channel: columns
-  // c0 .. c0+7 (lines 0-7) and M-c0-8 .. M-c0-1 (lines 8-15), c0 = 8 p for
-  // p < M/16.  H depends on |kx| only, and the two groups' |kx| are c0 .. c0+8,
-  // so one tile of 10 |kx| values (c0 .. c0+9) serves all 16 columns.  The
-  // quadrant table is symmetric, H(|ky|, |kx|) = H(|kx|, |ky|) (the setup forms
-  // q = k^2 - (fx^2 + fy^2), the same in either order), so the tile is fetched
-  // as the table's rows c0 .. c0+9, all M/2 + 2 entries each (box {M/2+2, 10,
-  // 1}; a row is a 16-byte multiple), and held as tile[|kx| - c0][|ky|]: then
-  // the 16 reads of a half-warp (8 lines x 2 element owners) fall on distinct
-  // bank pairs.  Per item, three tensor copies: the two groups' input rows (box
-  // {8, in_r1 - in_r0, 1} of the row spectra, one dense [rows][8] block per
-  // group) and the H tile.  The spectra of the next item are fetched at the
-  // barrier inside the forward DFT (the stage has been read) and waited for at
-  // the top of the item, with one block-wide verdict; the H tile of an item is
-  // fetched at its top (every thread is past the previous item's multiply)
-  // and waited for just before the H multiply, so its copy overlaps the
-  // forward DFT.  A thread whose H wait expires marks a shared flag (its
-  // item's results are then invalid, and reported so) that the next
-  // block-wide verdict reads.
+  // An item is a group of 8 columns of one channel: c0 .. c0 + 7, c0 = 8 gi.
+  // H depends on |kx| only and the quadrant table is symmetric, H(|ky|, |kx|)
+  // = H(|kx|, |ky|) (the setup forms q = k^2 - (fx^2 + fy^2), the same in
+  // either order), so the 8 table rows h0 .. h0 + 7 that hold the group's
+  // |kx| (h0 = c0 below M/2, M - c0 - 7 above) are fetched whole, all M/2 + 2
+  // entries each (a row is a 16-byte multiple), and held as tile[|kx| -
+  // h0][|ky|]: then the 16 reads of a half-warp (8 lines x 2 element owners)
+  // fall on distinct bank pairs.  Items are numbered so that a group and its
+  // mirror image, which read the same rows but one, run side by side (L2).
+  //
+  // A block holds one group, 8 lines of T threads (thread = element owner t,
+  // line lc: t = tid / 8, lc = tid % 8), and four such blocks fit an SM: the
+  // exchanges inside the line DFTs synchronise 8 lines and nothing else.  (Two
+  // groups to a block, tied by a barrier at the top of the item, left the
+  // warps of both waiting for the slower one.)  The item takes two barriers,
+  // the ones inside its two line DFTs: the exchange layouts alternate
+  // (Line::ALT), so every thread overwrites only what it read itself, and each
+  // barrier also carries the block's verdict on the wait before it: on the
+  // input rows at the first, on the H tile at the second.  A copy into a
+  // buffer is issued by thread 0 after the barrier that ends its reads.
+  //
+  // Bound by FP32 arithmetic and shared-memory accesses (each near 60 % of its
+  // rate), by instruction fetch at M = 512.  One group to a block, two barriers
+  // instead of three, and a loop without the displaced layers' code (48 -> 24
+  // KB, 73 -> 35 KB at M = 512): 4096 channels, M = 400, 1.56 -> 1.50 ms a
+  // launch; 2048 channels, M = 512, 1.40 -> 1.19 ms (with one group to a block
+  // but that code still in the loop: 1.46 ms).
   static constexpr int GW = Pass<LF>::COLL / 2;       // columns per group
-  static constexpr int HW = GW + 2;                   // |kx| values per H tile (c0 .. c0+9)
+  static constexpr int HW = GW;                       // |kx| values per H tile
   static constexpr int HP = M / 2 + 2;                // quadrant pitch (rows and columns)
   static_assert(GW == 8, "column groups of 8");
-  // The H tile is staged in a region of its own where the block still fits
-  // twice on an SM with it and a table row fits one box (M <= 400: 96.8 KB
-  // at N = 200).  At M = 512 the exchange buffers alone take 66 KB and a
-  // separate tile would leave one block per SM, so each group stages its own
-  // 8 rows of the table in its stage slot instead (SLOT_H): the copy is
-  // issued once the group's input rows are in registers (at the barrier
-  // inside the forward DFT) and waited for just before the H multiply, and
-  // the next item's input rows are fetched at the barrier inside the inverse
-  // DFT, when the group is past its H reads.  A table row of M/2 + 2 > 256
-  // entries is then two boxes of HB entries, at x = 0 and x = HP - HB.
+  // The H tile is staged in a region of its own where four blocks fit an SM
+  // with it and a table row fits one box (M <= 400: 55 KB at N = 200): the
+  // next item's tile is fetched after the second barrier of an item.  At M =
+  // 512 the tile takes the input rows' stage slot once they are in registers
+  // (SLOT_H): fetched at the first barrier, with the next input rows fetched
+  // at the second.  A table row of M/2 + 2 > 256 entries is then two boxes of
+  // HB entries, at x = 0 and x = HP - HB.
   static constexpr bool STAGE_H = M <= 400;
   static constexpr bool SLOT_H = !STAGE_H;
   static_assert(!STAGE_H || HP <= 256, "a staged H tile row is one box row (at most 256 entries)");
   static constexpr int HTILE = STAGE_H ? HW * HP : 0;  // float2 of the H tile in shared memory
-  static_assert(HTILE % 2 == 0, "the exchange buffers after the tile start 16-byte aligned");
   static constexpr int HB = (HP / 2 + 1) / 2 * 2;         // SLOT_H box width: even (16-byte box rows)
-  static constexpr int HSLOT = SLOT_H ? 2 * GW * HB : 0;  // float2 of a group's H tile: [2 boxes][8][HB]
+  static constexpr int HSLOT = SLOT_H ? 2 * GW * HB : 0;  // float2 of the H tile: [2 boxes][8][HB]
   static_assert(!SLOT_H || (HB <= 256 && (HP - HB) % 2 == 0 && 2 * HB >= HP),
                 "two 16-byte aligned boxes cover a table row");
   // every register's |ky| range (over the T element owners) lies in one box
@@ -162,80 +166,77 @@ struct PassBulk {
     return true;
   }
   static_assert(!SLOT_H || slot_boxes_cover(), "each register's H values come from one box");
-  // group stride in the stage (float2): whole 128-byte lines for any row
-  // count, and room for the group's H tile under SLOT_H
-  __host__ __device__ static int col_group_stride(int rows) {
+  // the stage (float2): whole 128-byte lines for any row count, and room for
+  // the H tile under SLOT_H
+  __host__ __device__ static int col_stage(int rows) {
     const int s = (rows + 1) / 2 * 2 * GW, h = (HSLOT + 15) / 16 * 16;
     return s > h ? s : h;
   }
-  // The two groups of an item share only the H tile: a group's 8 lines are
-  // held by warps of their own (thread = group g, line lc, element owner t:
-  // g = tid / GT, lc = tid % 8, t = (tid % GT) / 8), so the exchanges inside
-  // the line DFTs synchronise the group's warps on a named barrier, and only
-  // the top of an item is a block-wide barrier.  With GT not a multiple of the
-  // warp size (M = 200) the groups share warps and the block barrier serves.
-  static constexpr int GT = GW * T;                    // threads of a group
-  static constexpr bool GROUP_BARS = GT % 32 == 0;
+  static constexpr int GT = GW * T;                    // threads of a block
+  static constexpr bool GROUP_BARS = GT % 32 == 0;     // whole warps (all sizes but M = 200)
   // Exchange matrices of the column lines: even pitch ZX (row entries k1,
   // k1 + 1 are one 16-byte access), stride ZLB between the lines at least
-  // Q ZX and 2 mod 16.  A group warp holds 8 lines x 4 consecutive element
-  // owners; its 8-byte accesses (the column side of either layout) then fall
-  // on distinct bank pairs in each half-warp (8 lines x 2 owners) and its
+  // Q ZX and 2 mod 16.  A warp holds 8 lines x 4 consecutive element owners;
+  // its 8-byte accesses (the column side of either layout) then fall on
+  // distinct bank pairs in each half-warp (8 lines x 2 owners) and its
   // 16-byte ones (the row side) on distinct bank quads in each quarter-warp
   // (8 lines, one owner).
   static constexpr int ZX = LF::P + (LF::P & 1), ZSX = LF::Q * ZX;
   static constexpr int ZLB = ZSX + ((2 - ZSX % 16) + 16) % 16;
   static_assert(ZX % 2 == 0 && ZLB % 16 == 2, "16-byte aligned rows, conflict-free line stride");
-  __device__ static __forceinline__ void group_sync(int g) {
-    if constexpr (GROUP_BARS) {
-      // g is uniform over a warp; immediate barrier ids keep the count of
-      // barriers the kernel reserves at three
-      if (g == 0) asm volatile("bar.sync 1, %0;" ::"n"(GT) : "memory");
-      else asm volatile("bar.sync 2, %0;" ::"n"(GT) : "memory");
-    } else {
-      __syncthreads();
-    }
-  }
+  static_assert(LF::ALT, "the two line DFTs of an item alternate their exchange layouts");
   // dynamic shared memory (from a 128-byte aligned base):
-  //   stage[2][rows][8] | H tile[10][M/2+2] | exchange[COLL][ZLB] | tw[TWS] | barrier[4] | flag
-  static size_t col_smem(int n) {
-    return 128 + sizeof(float2) * (2 * (size_t)col_group_stride(n) + (size_t)HTILE + (size_t)COLL * ZLB +
-                                   LF::TWS + 1) + 4 * sizeof(uint64_t) + sizeof(int);
+  //   stage[rows][8] | H tile[8][M/2+2] | exchange[8][ZLB] | tw[TWS] | barrier[2] | ey[M/2+1] (MIS)
+  // (the H tile starts on a 128-byte boundary, as tensor copies need)
+  static constexpr int HTILE_PAD = (HTILE + 15) / 16 * 16;
+  static size_t col_smem(int n, bool mis) {
+    return 128 + sizeof(float2) * ((size_t)col_stage(n) + (size_t)HTILE_PAD + (size_t)GW * ZLB + LF::TWS + 1 +
+                                   (mis ? M / 2 + 1 : 0)) +
+           2 * sizeof(uint64_t);
   }
 
-  template <bool ADJ>
+  // MIS: displaced layers.  The table of the copies already holds the gap's
+  // length change; the lateral shift exp(-2 pi j (fx ax + fy ay)) is separable:
+  // ey[|ky|] is tabled once per block (its conjugate at negative ky, the bin
+  // M/2 counting as negative) and multiplies H, and the line's ex(kx), a
+  // constant of its column, multiplies the kept outputs.  Four blocks per SM
+  // still fit.
+  template <bool ADJ, bool MIS>
   __device__ static void col(const PassArgs& a, const CUtensorMap* smap, const CUtensorMap* hmap) {
     extern __shared__ __align__(16) unsigned char col_raw[];
     // 128-byte aligned start, by pointer arithmetic on the shared array: the
     // compiler keeps seeing shared-memory pointers (an integer round trip
     // would turn every access below into a generic one)
     float2* stage = reinterpret_cast<float2*>(col_raw + ((128u - (sh_addr(col_raw) & 127u)) & 127u));
-    const int GS = col_group_stride(a.n);
-    float2* htile = stage + 2 * (size_t)GS;
-    float2* zb = htile + HTILE;
-    float2* tw = tw_align(zb + (size_t)COLL * ZLB);
-    // [0], [1] spectra of group 0, 1; [2] transfer-table tile (STAGE_H), or
-    // [2], [3] the H tiles of group 0, 1 (SLOT_H)
-    uint64_t* bar = reinterpret_cast<uint64_t*>(tw + LF::TWS);
-    int* h_late = reinterpret_cast<int*>(bar + 4);  // an H wait of this block expired
-    const int g = threadIdx.x / GT, lc = threadIdx.x % GW, t = (threadIdx.x % GT) / GW;
-    const bool leader = threadIdx.x % GT == 0;  // issues the group's copies
-    float2* z = zb + (g * GW + lc) * ZLB;
-    constexpr int npairs = M / (2 * GW);
-    const int items = a.nw * npairs;
+    float2* htile = SLOT_H ? stage : stage + (size_t)col_stage(a.n);
+    float2* zb = stage + (size_t)col_stage(a.n) + HTILE_PAD;
+    float2* tw = tw_align(zb + (size_t)GW * ZLB);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(tw + LF::TWS);  // [0] input rows, [1] H tile
+    const int lc = threadIdx.x % GW, t = threadIdx.x / GW;
+    const bool leader = threadIdx.x == 0;  // issues the copies
+    float2* z = zb + lc * ZLB;
+    constexpr int ngroups = M / GW;
+    const int items = a.nw * ngroups;
     const uint32_t sbytes = GW * 8u * (uint32_t)(a.in_r1 - a.in_r0);
-    constexpr uint32_t hbytes = (uint32_t)HW * HP * 8u;
-    constexpr uint32_t hsbytes = (uint32_t)HSLOT * 8u;
-    if (threadIdx.x == 0) {
+    constexpr uint32_t hbytes = (uint32_t)(SLOT_H ? HSLOT : HTILE) * 8u;
+    // item -> channel and first column: neighbouring items are mirror images
+    auto place = [](int it, int& w, int& c0) {
+      w = it / ngroups;
+      const int q = it - w * ngroups;
+      c0 = GW * ((q & 1) ? ngroups - 1 - (q >> 1) : q >> 1);
+    };
+    auto table_row = [](int c0) { return c0 < M / 2 ? c0 : M - c0 - (GW - 1); };
+    if (leader) {
       bulk_bar_init(&bar[0]);
       bulk_bar_init(&bar[1]);
-      bulk_bar_init(&bar[2]);
-      bulk_bar_init(&bar[3]);
-      *h_late = 0;
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(smap)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(hmap)) : "memory");
     }
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
+    float2* ey = reinterpret_cast<float2*>(bar + 2);
+    if constexpr (MIS) {
+      for (int i = threadIdx.x; i <= M / 2; i += blockDim.x) ey[i] = shift_phase(i, a.mis.sy);
+    }
     __syncthreads();
     auto tensor_copy = [](float2* dst, const CUtensorMap* map, int x, int y, int zc, uint64_t* b) {
       asm volatile(
@@ -244,78 +245,72 @@ struct PassBulk {
           "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(zc), "r"(sh_addr(b))
           : "memory");
     };
-    // the input rows of group gg of item it (its leader)
-    auto fetch_s = [&](int it, int gg) {
+    // the input rows of item it (thread 0)
+    auto fetch_s = [&](int it) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bulk_expect(&bar[gg], sbytes);
+      bulk_expect(&bar[0], sbytes);
       if (a.stall == 1) return;  // injected fault: the expected bytes never arrive
-      const int w = it / npairs, c0 = GW * (it % npairs);
-      tensor_copy(stage + gg * GS, smap, gg == 0 ? c0 : M - c0 - GW, a.in_r0, a.tmap_w0 + w, &bar[gg]);
+      int w, c0;
+      place(it, w, c0);
+      tensor_copy(stage, smap, c0, a.in_r0, a.tmap_w0 + w, &bar[0]);
     };
     // the H tile of item it (thread 0)
     auto fetch_h = [&](int it) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bulk_expect(&bar[2], hbytes);
+      bulk_expect(&bar[1], hbytes);
       if (a.stall == 1) return;
-      const int w = it / npairs, c0 = GW * (it % npairs);
-      tensor_copy(htile, hmap, 0, c0, a.hmap_z0 + w, &bar[2]);
-    };
-    // the 8 table rows |kx| = c0 + gg .. c0 + gg + 7 that group gg of item it
-    // reads, into its stage slot (its leader; SLOT_H)
-    auto fetch_hs = [&](int it, int gg) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bulk_expect(&bar[2 + gg], hsbytes);
-      if (a.stall == 1) return;
-      const int w = it / npairs, c0 = GW * (it % npairs);
-      float2* dst = stage + gg * GS;
-      tensor_copy(dst, hmap, 0, c0 + gg, a.hmap_z0 + w, &bar[2 + gg]);
-      tensor_copy(dst + GW * HB, hmap, HP - HB, c0 + gg, a.hmap_z0 + w, &bar[2 + gg]);
+      int w, c0;
+      place(it, w, c0);
+      tensor_copy(htile, hmap, 0, table_row(c0), a.hmap_z0 + w, &bar[1]);
+      if constexpr (SLOT_H) tensor_copy(htile + GW * HB, hmap, HP - HB, table_row(c0), a.hmap_z0 + w, &bar[1]);
     };
     bool ok = true;
-    int k = 0;
-    if ((int)blockIdx.x < items && leader) fetch_s(blockIdx.x, g);
+    int k = 0, issued_s = 0, issued_h = 0, done_s = 0, done_h = 0;  // copies per barrier (thread 0's view)
+    if ((int)blockIdx.x < items) {
+      if (leader) fetch_s(blockIdx.x);
+      issued_s = 1;
+      if constexpr (STAGE_H) {
+        if (leader) fetch_h(blockIdx.x);
+        issued_h = 1;
+      }
+    }
     for (int it = blockIdx.x; it < items; it += gridDim.x, ++k) {
-      const int w = it / npairs, c0 = GW * (it % npairs);
-      const int cc = g == 0 ? c0 + lc : M - c0 - GW + lc;  // this line's column
-      const int hc = g == 0 ? lc : GW - lc;                 // its |kx| - c0: the column in the H tile
-      // this group's input rows, and no expired H wait in the previous item
-      const bool got = bulk_wait(&bar[g], (uint32_t)(k & 1), split_verdict(a, k)) && *h_late == 0;
-      ok = __syncthreads_and(got) != 0;  // one verdict for the whole block
-      if (!ok) break;
-      // every thread is past the previous item's H multiply: this item's tile
-      // may land (it is waited for just before the multiply)
-      if (STAGE_H && threadIdx.x == 0) fetch_h(it);
+      int w, c0;
+      place(it, w, c0);
+      const int cc = c0 + lc;  // this line's column
+      const int hc = min(cc, M - cc) - table_row(c0);  // |kx|'s row of the H tile
+      const bool more = it + (int)gridDim.x < items;
+      // this item's input rows; a thread whose wait expires goes on to the
+      // barrier with what is there, where the whole block stops
+      const bool got_s = bulk_wait(&bar[0], (uint32_t)(k & 1), split_verdict(a, k));
       float2 r[E];
-      const float2* sg = stage + (size_t)g * GS + lc - (ptrdiff_t)a.in_r0 * GW;  // row y at sg[y * GW]
+      const float2* sg = stage + lc - (ptrdiff_t)a.in_r0 * GW;  // row y at sg[y * GW]
 #pragma unroll
       for (int i = 0; i < E; ++i) {
         const int row = t + T * i;
         r[i] = (i < EF && row >= a.in_r0 && row < a.in_r1) ? sg[row * GW] : czero();
       }
       LF::template step1<false, NZF, PKC, false, ZX>(r, t, z, tw);
-      group_sync(g);  // the group is past its stage reads: its next rows (or its H tile) may land there
+      ok = __syncthreads_and(got_s) != 0;  // one verdict for the whole block, past its stage reads
+      if (!ok) break;
+      ++done_s;
       if constexpr (SLOT_H) {
-        if (leader) fetch_hs(it, g);
-      } else {
-        if (leader && it + (int)gridDim.x < items) fetch_s(it + gridDim.x, g);
+        if (leader) fetch_h(it);
+        ++issued_h;
+      } else if (more) {
+        if (leader) fetch_s(it + gridDim.x);
+        ++issued_s;
       }
       LF::template step2<false, LF::Q, PKC, false, ZX>(r, t, z);
-      // square lines: the inverse DFT below writes the exchange matrix in
-      // the transposed layout, i.e. only what this thread just read
-      if constexpr (!LF::SQUARE) group_sync(g);
-      // H(|ky|, |kx|) from the tile: |ky| = k below M/2 and M - k above, both
-      // affine in i at compile time
       // (injected, tests: the wait of the block's last item gives up)
-      const bool give_up_h = a.stall == 3 && it + (int)gridDim.x >= items;
-      if (STAGE_H && !bulk_wait(&bar[2], (uint32_t)(k & 1), give_up_h)) *h_late = 1;
-      if (SLOT_H && !bulk_wait(&bar[2 + g], (uint32_t)(k & 1), give_up_h)) *h_late = 1;
-      // STAGE_H: tile[hc][|ky|] (pitch HP).  SLOT_H: box b of the group's
-      // tile, [hc - g][|ky| - b (HP - HB)] (pitch HB); box 0 holds |ky| < HB,
-      // box 1 |ky| >= HP - HB, and which one a register's |ky| range lies in
-      // is known at compile time.
-      const float2* hlo = STAGE_H ? htile + hc * HP + t : stage + (size_t)g * GS + (hc - g) * HB + t;
-      const float2* hhi = STAGE_H ? htile + hc * HP + (M - t) : stage + (size_t)g * GS + (hc - g) * HB + (M - t);
-      const float* Sw = a.mis.sq ? a.mis.sq + (size_t)w * a.hs * a.hs : nullptr;
+      const bool got_h = (a.stall == 3 && !more) ? false : bulk_wait(&bar[1], (uint32_t)(k & 1));
+      // STAGE_H: tile[hc][|ky|] (pitch HP), |ky| = k below M/2 and M - k above,
+      // both affine in i at compile time.  SLOT_H: box b of the tile,
+      // [hc][|ky| - b (HP - HB)] (pitch HB); box 0 holds |ky| < HB, box 1
+      // |ky| >= HP - HB, and which one a register's |ky| range lies in is
+      // known at compile time.
+      const float2* hlo = htile + hc * (STAGE_H ? HP : HB) + t;
+      const float2* hhi = htile + hc * (STAGE_H ? HP : HB) + (M - t);
 #pragma unroll
       for (int i = 0; i < E; ++i) {
         float2 h;
@@ -327,19 +322,28 @@ struct PassBulk {
           if (i < E / 2) h = T * i + T - 1 < HB ? hlo[T * i] : hlo[B1 + T * i];
           else h = M - T * i < HB ? hhi[-T * i] : hhi[B1 - T * i];
         }
-        if (Sw) {
-          const int kk = t + T * i;
-          h = cmul(h, misalign_factor(a.mis, kk, cc, M, Sw[(size_t)min(kk, M - kk) * a.hs + c0 + hc]));
-        }
+        if constexpr (MIS) h = i < E / 2 ? cmul(h, ey[t + T * i]) : cmulc(h, ey[M - t - T * i]);
         r[i] = ADJ ? cmulc(r[i], h) : cmul(r[i], h);
       }
-      LF::template step1<true, LF::P, PKC, LF::SQUARE, ZX>(r, t, z, tw);
-      group_sync(g);
-      // SLOT_H: the group is past its H reads: its next rows may land in the slot
-      if (SLOT_H && leader && it + (int)gridDim.x < items) fetch_s(it + gridDim.x, g);
-      // no trailing barrier: the exchange buffer is next written after the
-      // barrier at the top of the next item
-      LF::template step2<true, NOI, PKC, LF::SQUARE, ZX>(r, t, z);
+      LF::template step1<true, LF::P, PKC, true, ZX>(r, t, z, tw);
+      ok = __syncthreads_and(got_h) != 0;  // the verdict on the tile, past its reads
+      if (!ok) break;
+      ++done_h;
+      if (more) {
+        if constexpr (SLOT_H) {
+          if (leader) fetch_s(it + gridDim.x);
+          ++issued_s;
+        } else {
+          if (leader) fetch_h(it + gridDim.x);
+          ++issued_h;
+        }
+      }
+      LF::template step2<true, NOI, PKC, true, ZX>(r, t, z);
+      if constexpr (MIS) {
+        const float2 ex = shift_phase(signed_bin(cc, M), a.mis.sx);
+#pragma unroll
+        for (int i = 0; i < EF; ++i) r[i] = ADJ ? cmulc(r[i], ex) : cmul(r[i], ex);
+      }
       float2* dst = a.S + (size_t)w * a.n * M + cc;
 #pragma unroll
       for (int i = 0; i < E; ++i) {
@@ -347,23 +351,10 @@ struct PassBulk {
         if (i < EF && row >= a.out_r0 && row < a.out_r1) dst[(size_t)row * M] = r[i];
       }
     }
-    // An H wait that expired in the block's last item has no later verdict
-    // to read it: every thread (the loop ends for all of them together)
-    // takes it here.
-    const bool late = __syncthreads_or(*h_late != 0) != 0;
-    if ((!ok || late) && threadIdx.x == 0) {
-      // The copies in flight land (bounded) before the block leaves: after a
-      // failed verdict at item k both groups' rows of item k, and after an
-      // expired H wait in item k - 1 that tile (no tile of item k was issued).
-      if (!ok) {
-        (void)bulk_wait(&bar[0], (uint32_t)(k & 1));
-        (void)bulk_wait(&bar[1], (uint32_t)(k & 1));
-      }
-      if (STAGE_H && late) (void)bulk_wait(&bar[2], (uint32_t)((k - 1) & 1));
-      if (SLOT_H && late) {
-        (void)bulk_wait(&bar[2], (uint32_t)((k - 1) & 1));
-        (void)bulk_wait(&bar[3], (uint32_t)((k - 1) & 1));
-      }
+    if (!ok && leader) {
+      // the copies in flight land (bounded waits) before the block leaves
+      if (issued_s > done_s) (void)bulk_wait(&bar[0], (uint32_t)(done_s & 1));
+      if (issued_h > done_h) (void)bulk_wait(&bar[1], (uint32_t)(done_h & 1));
       atomicExch(a.err, 1);
     }
   }
@@ -431,19 +422,22 @@ struct PassBulk {
     for (int w = w0; w < w1; ++w, ++k) {
       const ChanConst cc = cnext;
       if (w + 1 < w1) cnext = a.chan[w + 1];
-      okw = __syncthreads_and(bulk_wait(bar, (uint32_t)(k & 1), split_verdict(a, k))) != 0;  // one verdict for the whole block
-      if (!okw) break;
+      // a thread whose wait expires goes on to the barrier with what is there,
+      // where the whole block stops
+      const bool got = bulk_wait(bar, (uint32_t)(k & 1), split_verdict(a, k));
       float2 r[E];
 #pragma unroll
       for (int i = 0; i < E; ++i) r[i] = stage[(size_t)(ok ? l : 0) * SR + t + T * i];
       LF::template step1<true, LF::P, PKR>(r, t, z, tw);
-      __syncthreads();  // every thread is past its stage reads: the next channel may land there
+      // one verdict for the whole block; every thread is past its stage reads:
+      // the next channel may land there
+      okw = __syncthreads_and(got) != 0;
+      if (!okw) break;
       if (w + 1 < w1) fetch(w + 1);
+      // the forward DFT below writes the exchange matrix in the other layout
+      // (only what this thread reads here), and the next channel's inverse
+      // DFT again: no barrier between them
       LF::template step2<true, NOI, PKR>(r, t, z);
-      // square lines: the forward DFT below writes the exchange matrix in the
-      // transposed layout (only what this thread just read); the adjoint's
-      // forward DFT does too
-      if constexpr (!LF::SQUARE) __syncthreads();
       float2* srow = a.S + ((size_t)w * a.n + rr) * M;
       if constexpr (!ADJ) {
         float2* ck = a.ckpt + ((size_t)w * a.n + rr) * a.n;
@@ -458,7 +452,7 @@ struct PassBulk {
             r[i] = czero();
           }
         }
-        LF::template fft<false, NZF, LF::Q, false, PKR, LF::SQUARE>(r, t, z, tw);
+        LF::template fft<false, NZF, LF::Q, false, PKR, true>(r, t, z, tw);
         if (ok) {
 #pragma unroll
           for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
@@ -479,11 +473,13 @@ struct PassBulk {
           }
         }
         if constexpr (!FLAG) {
-          LF::template fft<false, NZF, LF::Q, false, PKR, LF::SQUARE>(r, t, z, tw);
+          LF::template fft<false, NZF, LF::Q, false, PKR, true>(r, t, z, tw);
           if (ok) {
 #pragma unroll
             for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
           }
+        } else {
+          __syncthreads();  // the next channel writes the exchange matrix in the same layout
         }
       }
     }
@@ -673,14 +669,18 @@ struct PassBulk {
       }
     }
     for (int w = w0; w < w1; ++w) {
-      okw = __syncthreads_and(bulk_wait(&bar[0], (uint32_t)(done_s & 1), split_verdict(a, done_s))) != 0;  // one verdict for the block
-      if (!okw) break;
-      ++done_s;
+      // a thread whose wait expires goes on to the barrier with what is there,
+      // where the whole block stops
+      const bool got_s = bulk_wait(&bar[0], (uint32_t)(done_s & 1), split_verdict(a, done_s));
       float2 r[E];
 #pragma unroll
       for (int i = 0; i < E; ++i) r[i] = stage[(size_t)lr * SR + t + T * i];
       LF::template step1<true, LF::P, PKR>(r, t, z, tw);
-      __syncthreads();  // every thread is past its stage reads: the next channel (SHARE: this channel's checkpoint) may land there
+      // one verdict for the block; every thread is past its stage reads: the
+      // next channel (SHARE: this channel's checkpoint) may land there
+      okw = __syncthreads_and(got_s) != 0;
+      if (!okw) break;
+      ++done_s;
       if constexpr (SHARE) {
         fetch_c(w);
         ++issued_c;
@@ -688,10 +688,11 @@ struct PassBulk {
         fetch_s(w + 1);
         ++issued_s;
       }
-      LF::template step2<true, NOI, PKR>(r, t, z);  // the barrier below also ends its z reads
-      okw = __syncthreads_and(bulk_wait(&bar[1], (uint32_t)(done_c & 1))) != 0;
-      if (!okw) break;
-      ++done_c;
+      // the forward DFT below writes the exchange matrix in the other layout
+      // (only what this thread reads here), and the next channel's inverse
+      // DFT again: no barrier between them
+      LF::template step2<true, NOI, PKR>(r, t, z);
+      const bool got_c = bulk_wait(&bar[1], (uint32_t)(done_c & 1));
       // the channel's constants, loaded here rather than held through the
       // inverse DFT (the registers they would take there spill)
       const ChanConst cc = a.chan[w];
@@ -710,8 +711,12 @@ struct PassBulk {
         }
       }
       if constexpr (!FIRST) {
-        LF::template step1<false, NZF, PKR, LF::SQUARE>(r, t, z, tw);
-        __syncthreads();  // every thread is past its checkpoint reads
+        LF::template step1<false, NZF, PKR, true>(r, t, z, tw);
+        // the verdict on the checkpoint rows, past their reads (the gradient
+        // sums of an expired wait are never written)
+        okw = __syncthreads_and(got_c) != 0;
+        if (!okw) break;
+        ++done_c;
         if (w + 1 < w1) {
           if constexpr (SHARE) {
             fetch_s(w + 1);
@@ -721,14 +726,16 @@ struct PassBulk {
             ++issued_c;
           }
         }
-        LF::template step2<false, LF::Q, PKR, LF::SQUARE>(r, t, z);  // next z write follows the loop-top barrier
+        LF::template step2<false, LF::Q, PKR, true>(r, t, z);
         if (ok) {
           float2* srow = a.S + ((size_t)w * a.n + rr) * M;
 #pragma unroll
           for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
         }
       } else {
-        __syncthreads();  // every thread is past its checkpoint reads
+        okw = __syncthreads_and(got_c) != 0;  // as above; also ends the exchange reads
+        if (!okw) break;
+        ++done_c;
         if (w + 1 < w1) {
           if constexpr (SHARE) {
             fetch_s(w + 1);
@@ -765,12 +772,14 @@ template <class LF, int RL, bool HALF, bool FIRST>
 __global__ void __launch_bounds__(LF::T * RL, 3) k_row_adj_staged(PassArgs a) {
   PassBulk<LF, RL, HALF>::template row_adj_staged<FIRST>(a);
 }
-// two blocks per SM for every line shape: one leaves too few warps to hide the
-// DFT's barriers and dependencies (M = 512: 8.5 ms per launch with one)
-template <class LF, int RL, bool HALF, bool ADJ>
-__global__ void __launch_bounds__(LF::T * Pass<LF>::COLL, 2)
+// Column pass: four blocks of 8 lines per SM for every line shape (M = 400: 20
+// warps at up to 102 registers, M = 512: 16 at up to 128).
+template <class LF>
+constexpr int col_bulk_min_blocks() { return LF::T >= 16 ? 4 : 8; }
+template <class LF, int RL, bool HALF, bool ADJ, bool MIS>
+__global__ void __launch_bounds__(PassBulk<LF, RL, HALF>::GT, col_bulk_min_blocks<LF>())
     k_col_bulk(PassArgs a, const __grid_constant__ CUtensorMap smap, const __grid_constant__ CUtensorMap hmap) {
-  PassBulk<LF, RL, HALF>::template col<ADJ>(a, &smap, &hmap);
+  PassBulk<LF, RL, HALF>::template col<ADJ, MIS>(a, &smap, &hmap);
 }
 // the row passes: as many resident blocks as their shared memory allows
 template <class LF, int RL>
@@ -806,24 +815,25 @@ struct PassBulkLaunch {
   static bool half(const PassArgs& a) { return 2 * a.n <= LF::M; }
   template <bool H>
   static cudaError_t col_h(const PassArgs& a, bool adj, size_t sm, cudaStream_t s) {
-    const int items = a.nw * (LF::M / PB::COLL);
+    const int items = a.nw * (LF::M / PB::GW);
     if (items == 0) return cudaSuccess;
     int n_slots = 0;
-    auto kern = adj ? k_col_bulk<LF, RL, H, true> : k_col_bulk<LF, RL, H, false>;
-    cudaError_t e = slots(kern, PB::CT, sm, &n_slots);
+    auto kern = a.displaced ? (adj ? k_col_bulk<LF, RL, H, true, true> : k_col_bulk<LF, RL, H, false, true>)
+                            : (adj ? k_col_bulk<LF, RL, H, true, false> : k_col_bulk<LF, RL, H, false, false>);
+    cudaError_t e = slots(kern, PB::GT, sm, &n_slots);
     if (e != cudaSuccess) return e;
-    kern<<<std::min(items, n_slots), PB::CT, sm, s>>>(a, *static_cast<const CUtensorMap*>(a.tmap),
+    kern<<<std::min(items, n_slots), PB::GT, sm, s>>>(a, *static_cast<const CUtensorMap*>(a.tmap),
                                                      *static_cast<const CUtensorMap*>(a.hmap));
     return cudaGetLastError();
   }
   // The tensor copies need maps whose boxes hold the input rows (at most 256)
-  // and the H tile, and M a multiple of 16 (whole mirrored pairs of 8-column
-  // groups); otherwise the plain kernel runs.
+  // and the H tile, and M a multiple of 8 (whole 8-column groups); otherwise
+  // the plain kernel runs.
   static cudaError_t col(const PassArgs& a, bool adj, cudaStream_t s) {
-    const size_t sm = PB::col_smem(a.n);
+    const size_t sm = PB::col_smem(a.n, a.displaced);
     if (!a.tmap || !a.hmap || a.tmap_rows != a.in_r1 - a.in_r0 || a.tmap_rows > 256 ||
-        LF::M % 16 != 0 ||
-        sm > 227 * 1024)
+        (a.displaced && a.mis.sq) ||  // the length change is not in the table
+        LF::M % PB::GW != 0 || sm > 227 * 1024)
       return PassLaunch<LF>::col(a, adj, false, s);
     return half(a) ? col_h<true>(a, adj, sm, s) : col_h<false>(a, adj, sm, s);
   }
