@@ -144,7 +144,8 @@ struct dos_ctx {
   double* d_loss = nullptr;
   unsigned* loss_ticket = nullptr;  // channels done in the running loss kernel (zero between launches)
   double* h_loss = nullptr;  // pinned
-  int chunk = 1, n_chunks = 1;
+  // channels per block of the adjoint row pass, plain and prefetching
+  int chunk_plain = 1, chunk_bulk = 1;
   // multi-pass passes that run their bulk-async prefetching kernels
   // (DOS_PATH_MULTIPASS_BULK: all three; the autotuner may mix them per kind)
   unsigned bulk = 0;
@@ -250,6 +251,8 @@ struct dos_ctx {
     if (h_err) cudaFreeHost(h_err);
     h_err = nullptr;
   }
+  int adj_chunk() const { return (bulk & kBulkRowAdj) ? chunk_bulk : chunk_plain; }
+  int chunks_of(int chunk) const { return (nw + chunk - 1) / chunk; }
   float2* hq_slot(int gap) const { return Hq + (size_t)gap_slot[gap] * nw * hs * hs; }
   dos::PassArgs base() const {
     dos::PassArgs a;
@@ -265,8 +268,8 @@ struct dos_ctx {
     a.fov = fov;
     a.of = of;
     a.hs = hs;
-    a.chunk = chunk;
-    a.n_chunks = n_chunks;
+    a.chunk = adj_chunk();
+    a.n_chunks = chunks_of(a.chunk);
     a.err = d_err;
     a.tmap = have_tmap ? &tmap_S : nullptr;
     a.tmap_rows = n;
@@ -417,17 +420,19 @@ int build(dos_ctx* x, const dos_config* c) {
     x->gap_slot.push_back(s);
   }
   x->n_slots = (int)slots.size();
-  // channel chunks of the adjoint row pass: about 8 blocks per SM in flight
+  // channel chunks of the plain adjoint row pass: about 8 blocks per SM in
+  // flight; the prefetching one has its own (whole waves of its resident blocks)
   const int row_blocks = (x->n + x->ops->row_lines - 1) / x->ops->row_lines;
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
   const int want_chunks = std::max(1, (8 * sms) / std::max(1, row_blocks));
-  x->chunk = std::max(1, (x->nw + want_chunks - 1) / want_chunks);
-  x->n_chunks = (x->nw + x->chunk - 1) / x->chunk;
+  x->chunk_plain = std::max(1, (x->nw + want_chunks - 1) / want_chunks);
+  x->chunk_bulk = x->ops->bulk_adj_chunk(x->n, x->nw, x->chunk_plain);
+  if (x->chunk_bulk < 1) x->chunk_bulk = x->chunk_plain;
 
   const size_t n2 = (size_t)x->n * x->n;
   // cluster-resident configurations that fit this design
-  size_t partial_count = (size_t)x->K * x->n_chunks * n2;
+  size_t partial_count = (size_t)x->K * std::max(x->chunks_of(x->chunk_plain), x->chunks_of(x->chunk_bulk)) * n2;
   if (2 * x->n <= x->m) {
     const dos::FusedOps* list[16];
     const int k = dos::fused_ops_for_m(x->m, list, 16);
@@ -654,7 +659,7 @@ dos::PassArgs range_args(const dos_ctx* c, int w0, int w1) {
   a.o = c->o + (size_t)w0 * c->fov * c->fov;
   a.chan = c->chan + w0;
   a.nw = w1 - w0;
-  a.n_chunks = (a.nw + c->chunk - 1) / c->chunk;
+  a.n_chunks = (a.nw + a.chunk - 1) / a.chunk;
   a.tmap_w0 = w0;
   return a;
 }
@@ -768,7 +773,7 @@ std::vector<Launch> backward_launches(dos_ctx* c, const float* d_h, const float*
                  "adjoint column pass"});
     a.h = d_h + (size_t)(l - 1) * n2;
     a.ckpt = (l == 1 && c->ckpt1_is_v1) ? c->v1 + (size_t)w0 * n2 : c->ckpt + ((size_t)(l - 1) * c->nw + w0) * n2;
-    a.partial = c->partial + ((size_t)(l - 1) * c->n_chunks + w0 / c->chunk) * n2;
+    a.partial = c->partial + ((size_t)(l - 1) * c->chunks_of(a.chunk) + w0 / a.chunk) * n2;
     const bool brow = (c->bulk & kBulkRowAdj) != 0;
     const bool first = l == 1;
     a.stall = c->take_stall(kBulkRowAdj);
@@ -894,7 +899,7 @@ int run_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dLd
   const int rc = run_launches(c, backward_launches(c, d_h, d_dLdI, 0, c->nw));
   if (rc) return rc;
   DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
-            dos::launch_grad_reduce(c->partial, d_dLdh, c->n_chunks, (size_t)c->K * n2, n2, c->stream),
+            dos::launch_grad_reduce(c->partial, d_dLdh, c->chunks_of(c->adj_chunk()), (size_t)c->K * n2, n2, c->stream),
             "gradient reduction");
   ++c->launches;
   return DOS_OK;

@@ -79,7 +79,7 @@ struct PassArgs {
   int n, m, nw, fov, of, hs;
   int in_r0, in_r1;       // column pass: rows that may be non-zero on input
   int out_r0, out_r1;     // column pass: rows stored on output
-  int chunk;              // channels per block of the adjoint row pass
+  int chunk;              // channels per block of the adjoint row pass (the bulk forward ones set their own)
   int n_chunks;
   bool displaced;         // column pass: the gap carries a displacement that Hq does not hold (mis)
   Misalign mis;           // its lateral shift; and, with mis.sq, its length change (plain kernel only)
@@ -113,6 +113,7 @@ struct PassOps {
   cudaError_t (*bulk_row_fwd)(const PassArgs&, bool save, cudaStream_t);
   cudaError_t (*bulk_row_adj)(const PassArgs&, bool first, cudaStream_t);
   cudaError_t (*bulk_row_first)(const PassArgs&, cudaStream_t);  // t(h) * field (fin) -> row spectra
+  int (*bulk_adj_chunk)(int n, int nw, int most);  // channels per block of bulk_row_adj (0: unknown)
   // boxes of the bulk column pass's tensor copies: spectra {col_group, rows, 1},
   // transfer table {h_box_cols, h_box_rows, 1} (h_box_cols 0: no staged H tile)
   int col_group, h_box_cols, h_box_rows;

@@ -793,6 +793,34 @@ __global__ void __launch_bounds__(LF::T * RL, row_bulk_min_blocks<LF, RL>()) k_r
   PassBulk<LF, RL, HALF>::row_first_staged(a);
 }
 
+// Channels per block of a row pass.  A launch of rb row blocks x c chunks runs
+// in waves of `slots` resident blocks, each as long as one block's channels
+// plus about one channel's time to start (twiddles, thickness row, the first
+// copy's latency) and to finish: the split with the smallest waves x (channels
+// + 1), and of equals the one with the fewest waves.  (Chunks made for about
+// eight blocks per SM whatever the kernel's residency left a last wave with 20
+// blocks of 456 at 4096 channels of 200 x 200, and three channels per block at
+// 256.)  most: the largest chunk allowed.
+inline int balanced_chunk(int nw, int rb, int slots, int most) {
+  int best = std::max(1, std::min(nw, most));
+  double cost = 1e30;
+  for (int waves = 1; waves <= 64; ++waves) {
+    const int c = std::max(1, std::min(nw, waves * slots / std::max(1, rb)));
+    const int chunk = (nw + c - 1) / c, cc = (nw + chunk - 1) / chunk;
+    if (chunk > most) continue;
+    const double t = (double)(((long)rb * cc + slots - 1) / slots) * (chunk + 1.0);
+    if (t < 0.999 * cost) cost = t, best = chunk;
+    if (c == nw) break;
+  }
+  return best;
+}
+// Most channels per block.  The adjoint row pass sums its chunk's channels in
+// FP32 registers (before balanced_chunk: 45 at 4096 channels, so no more terms
+// than then); and in both passes long chunks spread the blocks that run
+// together over the whole spectra buffer: forward 0.95 -> 0.99 ms at 4096
+// channels with 171 per block.
+constexpr int kRowChunk = 48;
+
 // Launchers.  The column pass runs one persistent block per resident slot
 // (blocks per SM from the occupancy calculator x SMs); the row passes run
 // (row blocks) x (channel chunks) blocks, each looping over its chunk.
@@ -837,12 +865,24 @@ struct PassBulkLaunch {
       return PassLaunch<LF>::col(a, adj, false, s);
     return half(a) ? col_h<true>(a, adj, sm, s) : col_h<false>(a, adj, sm, s);
   }
+  // Launch of a forward row kernel over all channels: the channels split into
+  // chunks (grid.y) that fill whole waves of the resident slots.
+  template <typename K>
+  static cudaError_t launch_rows(K kernel, size_t sm, const PassArgs& a, cudaStream_t s) {
+    int n_slots = 0;
+    cudaError_t e = slots(kernel, PB::RT, sm, &n_slots);
+    if (e != cudaSuccess) return e;
+    PassArgs b = a;
+    const int rb = (a.n + RL - 1) / RL;
+    b.chunk = balanced_chunk(a.nw, rb, n_slots, kRowChunk);
+    kernel<<<dim3(rb, (a.nw + b.chunk - 1) / b.chunk), PB::RT, sm, s>>>(b);
+    return cudaGetLastError();
+  }
   template <bool H>
   static cudaError_t row_fwd_h(const PassArgs& a, bool save, cudaStream_t s) {
-    const dim3 g((a.n + RL - 1) / RL, a.n_chunks);
     const size_t sm = PB::row_smem();
-    return save ? launch_k(k_row_bulk<LF, RL, H, false, true>, g, PB::RT, sm, a, s)
-                : launch_k(k_row_bulk<LF, RL, H, false, false>, g, PB::RT, sm, a, s);
+    return save ? launch_rows(k_row_bulk<LF, RL, H, false, true>, sm, a, s)
+                : launch_rows(k_row_bulk<LF, RL, H, false, false>, sm, a, s);
   }
   static cudaError_t row_fwd(const PassArgs& a, bool save, cudaStream_t s) {
     return half(a) ? row_fwd_h<true>(a, save, s) : row_fwd_h<false>(a, save, s);
@@ -852,9 +892,8 @@ struct PassBulkLaunch {
   static cudaError_t row_first(const PassArgs& a, cudaStream_t s) {
     const size_t sm = PB::first_smem(a.n);
     if (a.n % 2 != 0 || sm > 227 * 1024) return PassLaunch<LF>::row_first(a, s);
-    const dim3 g((a.n + RL - 1) / RL, a.n_chunks);
-    return half(a) ? launch_k(k_row_first_staged<LF, RL, true>, g, PB::RT, sm, a, s)
-                   : launch_k(k_row_first_staged<LF, RL, false>, g, PB::RT, sm, a, s);
+    return half(a) ? launch_rows(k_row_first_staged<LF, RL, true>, sm, a, s)
+                   : launch_rows(k_row_first_staged<LF, RL, false>, sm, a, s);
   }
   // rows per block of the staged adjoint row pass
   static constexpr int RLA = RL >= 16 ? RL / 2 : RL;
@@ -876,6 +915,28 @@ struct PassBulkLaunch {
   static cudaError_t row_adj(const PassArgs& a, bool first, cudaStream_t s) {
     return half(a) ? row_adj_h<true>(a, first, s) : row_adj_h<false>(a, first, s);
   }
+  // channels per block of row_adj for n x n layers and nw channels, at most
+  // kRowChunk or `most` where that is larger (the
+  // gradient partials hold one n x n plane per chunk)
+  template <bool H>
+  static int adj_chunk_h(int n, int nw, int most) {
+    int n_slots = 0, rows = RL;
+    cudaError_t e;
+    if (n % 2 == 0 && PBA::adj_staged_smem(n) <= 227 * 1024) {
+      rows = RLA;
+      e = slots(k_row_adj_staged<LF, RLA, H, false>, PBA::RT, PBA::adj_staged_smem(n), &n_slots);
+    } else {
+      e = slots(k_row_bulk<LF, RL, H, true, false>, PB::RT, PB::row_smem(), &n_slots);
+    }
+    if (e != cudaSuccess) {
+      (void)cudaGetLastError();
+      return 0;
+    }
+    return balanced_chunk(nw, (n + rows - 1) / rows, n_slots, std::max(most, kRowChunk));
+  }
+  static int adj_chunk(int n, int nw, int most) {
+    return 2 * n <= LF::M ? adj_chunk_h<true>(n, nw, most) : adj_chunk_h<false>(n, nw, most);
+  }
 };
 
 // The launchers of one padded size, plain and bulk-prefetching.
@@ -887,7 +948,7 @@ const PassOps* pass_ops_table() {
                             Pass<LF>::ROWL, Pass<LF>::COLL, &PL::col,    &PL::row_fwd,
                             &PL::row_out, &PL::row_seed,  &PL::row_adj,  &PL::row_in,
                             &PL::row_back, &PL::row_first, &PBL::col, &PBL::row_fwd,
-                            &PBL::row_adj, &PBL::row_first, PassBulk<LF, RL>::GW,
+                            &PBL::row_adj, &PBL::row_first, &PBL::adj_chunk, PassBulk<LF, RL>::GW,
                             PassBulk<LF, RL>::STAGE_H ? PassBulk<LF, RL>::HP : PassBulk<LF, RL>::HB,
                             PassBulk<LF, RL>::STAGE_H ? PassBulk<LF, RL>::HW : PassBulk<LF, RL>::GW};
   return &o;
