@@ -459,7 +459,7 @@ int build(dos_ctx* x, const dos_config* c) {
     x->gp.rp1 = pad(2 * x->m, 256);
     x->gp.rp2 = pad(2 * x->n, 256);
     x->gchunks = (x->nw + x->gp.nwc - 1) / x->gp.nwc;
-    partial_count = std::max(partial_count, (size_t)x->gchunks * x->K * n2);
+    partial_count = std::max(partial_count, (size_t)x->gchunks * dos::gemm_adj_slices(x->gp) * x->K * n2);
   }
   int rc;
   if (gemm) {
@@ -467,14 +467,25 @@ int build(dos_ctx* x, const dos_config* c) {
     const size_t nwc = (size_t)g.nwc;
     // the data operand holds whole 256-row tiles (the GEMM reads them whole)
     const size_t cm = (nwc * g.m + 255) / 256 * 256, cn = (nwc * g.n + 255) / 256 * 256;
-    const size_t xsz = std::max({cm * g.kp1, cm * g.kp2, cn * g.kp1, cn * g.kp2});
-    g.F.k = g.G.k = g.X.k = g.Y.k = g.parts;
-    for (int q = 0; q < 3; ++q) g.F.p[q] = g.G.p[q] = g.X.p[q] = g.Y.p[q] = nullptr;
+    dos::Parts* ops[4] = {&g.X1, &g.Y1, &g.X2, &g.Y2};
+    const size_t sizes[4] = {cn * g.kp1, cm * g.kp1, cm * g.kp2, cn * g.kp2};
+    g.F.k = g.G.k = g.parts;
     for (int q = 0; q < g.parts; ++q) {
       if ((rc = x->alloc(&g.F.p[q], (size_t)g.rp1 * g.kp1, "DFT matrix"))) return rc;
       if ((rc = x->alloc(&g.G.p[q], (size_t)g.rp2 * g.kp2, "IDFT matrix"))) return rc;
-      if ((rc = x->alloc(&g.X.p[q], xsz, "GEMM operand"))) return rc;
-      if ((rc = x->alloc(&g.Y.p[q], xsz, "GEMM operand"))) return rc;
+    }
+    // one block for all of them, whole 256-row tiles each
+    const size_t all = sizes[0] + sizes[1] + sizes[2] + sizes[3];
+    __nv_bfloat16* block = nullptr;
+    if ((rc = x->alloc(&block, all * g.parts, "GEMM operands"))) return rc;
+    if (g.kp1 != 2 * x->n || g.kp2 != 2 * x->m)  // rows with padding entries
+      DOS_CUDA(cudaMemsetAsync(block, 0, all * g.parts * sizeof(*block), x->stream), "GEMM operands");
+    for (int i = 0; i < 4; ++i) {
+      ops[i]->k = g.parts;
+      for (int q = 0; q < 3; ++q) {
+        ops[i]->p[q] = q < g.parts ? block : nullptr;
+        if (q < g.parts) block += sizes[i];
+      }
     }
     if ((rc = x->alloc(&g.fld, nwc * n2, "GEMM field"))) return rc;
   }
@@ -577,8 +588,7 @@ int gemm_forward(dos_ctx* c, const float* d_h, float* d_I) {
   for (int w0 = 0; w0 < c->nw; w0 += g.nwc) {
     const int nc = std::min(g.nwc, c->nw - w0);
     DOS_TIMED(c, DOS_KERNEL_GEMM_FIELD,
-              dos::gemm_prep_field(g, nc, nullptr, nullptr, nullptr, nullptr, 2, c->oa, c->ap, c->stream),
-              "GEMM aperture field");
+              dos::gemm_prep_aperture(g, nc, c->oa, c->ap, c->stream), "GEMM aperture field");
     for (int gap = 0; gap <= c->K; ++gap) {
       const bool last = gap == c->K;
       dos::Misalign mg = c->gap_mis(gap);
@@ -591,8 +601,8 @@ int gemm_forward(dos_ctx* c, const float* d_h, float* d_I) {
                 "GEMM propagation");
       if (!last) {
         DOS_TIMED(c, DOS_KERNEL_GEMM_FIELD,
-                  dos::gemm_prep_field(g, nc, g.fld, c->ckpt + ((size_t)gap * c->nw + w0) * n2, d_h + (size_t)gap * n2,
-                                       c->chan + w0, 1, 0, 0, c->stream),
+                  dos::gemm_prep_layer(g, nc, c->ckpt + ((size_t)gap * c->nw + w0) * n2, d_h + (size_t)gap * n2,
+                                       c->chan + w0, c->stream),
                   "GEMM layer modulation");
         ++c->launches;
       }
@@ -607,14 +617,13 @@ int gemm_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dL
   const size_t n2 = (size_t)c->n * c->n, hs2 = (size_t)c->hs * c->hs, f2 = (size_t)c->fov * c->fov;
   c->launches = 0;
   int chunk = 0;
+  const int slices = dos::gemm_adj_slices(g);
   for (int w0 = 0; w0 < c->nw; w0 += g.nwc, ++chunk) {
     const int nc = std::min(g.nwc, c->nw - w0);
     DOS_TIMED(c, DOS_KERNEL_GEMM_FIELD,
-              dos::gemm_seed(g, nc, c->o + (size_t)w0 * f2, d_dLdI + (size_t)w0 * f2, c->of, c->fov, c->stream),
+              dos::gemm_prep_seed(g, nc, c->o + (size_t)w0 * f2, d_dLdI + (size_t)w0 * f2, c->of, c->fov, c->stream),
               "GEMM adjoint seed");
-    DOS_TIMED(c, DOS_KERNEL_GEMM_FIELD,
-              dos::gemm_prep_field(g, nc, g.fld, nullptr, nullptr, nullptr, 0, 0, 0, c->stream), "GEMM field");
-    c->launches += 2;
+    c->launches += 1;
     for (int l = c->K; l >= 1; --l) {
       dos::Misalign mg = c->gap_mis(l);
       if (mg.sq) mg.sq += (size_t)w0 * hs2;
@@ -623,20 +632,15 @@ int gemm_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dL
                                     c->fov, mg, &c->launches, c->stream),
                 "GEMM adjoint propagation");
       DOS_TIMED(c, DOS_KERNEL_GEMM_FIELD,
-                dos::gemm_adj_layer(g, nc, c->ckpt + ((size_t)(l - 1) * c->nw + w0) * n2, n2,
-                                    d_h + (size_t)(l - 1) * n2, c->chan + w0,
-                                    c->partial + ((size_t)chunk * c->K + (l - 1)) * n2, c->stream),
+                dos::gemm_adj_layer(g, nc, c->ckpt + ((size_t)(l - 1) * c->nw + w0) * n2, d_h + (size_t)(l - 1) * n2,
+                                    c->chan + w0, c->partial + ((size_t)chunk * slices * c->K + (l - 1)) * n2,
+                                    (size_t)c->K * n2, l == 1, c->stream),
                 "GEMM adjoint layer");
       c->launches += 1;
-      if (l > 1) {
-        DOS_TIMED(c, DOS_KERNEL_GEMM_FIELD,
-                  dos::gemm_prep_field(g, nc, g.fld, nullptr, nullptr, nullptr, 0, 0, 0, c->stream), "GEMM field");
-        ++c->launches;
-      }
     }
   }
   DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
-            dos::launch_grad_reduce(c->partial, d_dLdh, c->gchunks, (size_t)c->K * n2, (size_t)c->K * n2, c->stream),
+            dos::launch_grad_reduce(c->partial, d_dLdh, c->gchunks * slices, (size_t)c->K * n2, (size_t)c->K * n2, c->stream),
             "gradient reduction");
   ++c->launches;
   return gemm_check(c);

@@ -431,84 +431,178 @@ cudaError_t launch_build_dft(GemmPlan& p, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------ conversion kernels
-// field (complex [w][y][x]) -> X rows (w, y): [Re(u), Im(u), 0 ...] of length kp.
-// mode 0: u = v;  mode 1: checkpoint v, u = t(h) v (forward layer);  mode 2: aperture.
-__global__ void k_prep_field(const float2* __restrict__ v, float2* __restrict__ ckpt, const float* __restrict__ h,
-                             const ChanConst* __restrict__ chan, Parts X, int n, int kp, int mode, int a_off,
-                             int a_w) {
-  const int wy = blockIdx.x;  // w * n + y
-  const int w = wy / n, y = wy % n;
-  for (int c = threadIdx.x; c < kp; c += blockDim.x) {
-    float val = 0.f;
-    if (c < 2 * n) {
-      const int x = c < n ? c : c - n;
-      float2 u;
-      if (mode == 2) {
-        const bool in = y >= a_off && y < a_off + a_w && x >= a_off && x < a_off + a_w;
-        u = make_float2(in ? 1.f : 0.f, 0.f);
-      } else {
-        const float2 vv = v[(size_t)wy * n + x];
-        if (mode == 1) {
-          if (c < n) ckpt[(size_t)wy * n + x] = vv;
-          u = cmul(transmission(h[(size_t)y * n + x], chan[w]), vv);
-        } else {
-          u = vv;
-        }
-      }
-      val = c < n ? u.x : u.y;
+// What becomes the operand rows (w, y) = [Re(u), Im(u)] of a propagation.
+enum {
+  PREP_LAYER = 1,     // checkpoint the field v, u = t(h) v (forward layer)
+  PREP_APERTURE = 2,  // u = the square aperture
+  PREP_SEED = 3       // u = 2 dL/dI o on the FOV, zero elsewhere (adjoint seed)
+};
+struct PrepArgs {
+  const float2* v;        // [nwc][n][n] (LAYER)
+  float2* ckpt;           // [nwc][n][n] (LAYER)
+  const float* h;         // [n][n] (LAYER)
+  const ChanConst* chan;  // [nwc] (LAYER)
+  const float2* o;        // [nwc][fov][fov] (SEED)
+  const float* dLdI;      // [nwc][fov][fov] (SEED)
+  int a_off, a_w;         // APERTURE: first pixel and side
+  int of, fov;            // SEED
+};
+
+// value of pixel (y, x) of channel w; LAYER also stores its checkpoint
+template <int MODE>
+__device__ __forceinline__ float2 prep_value(const PrepArgs& g, int n, int w, int y, int x) {
+  if constexpr (MODE == PREP_APERTURE) {
+    const bool in = y >= g.a_off && y < g.a_off + g.a_w && x >= g.a_off && x < g.a_off + g.a_w;
+    return make_float2(in ? 1.f : 0.f, 0.f);
+  } else if constexpr (MODE == PREP_SEED) {
+    const int fy = y - g.of, fx = x - g.of;
+    if (fy < 0 || fy >= g.fov || fx < 0 || fx >= g.fov) return make_float2(0.f, 0.f);
+    const size_t q = ((size_t)w * g.fov + fy) * g.fov + fx;
+    return cscale(g.o[q], 2.0f * g.dLdI[q]);
+  } else {
+    const size_t at = ((size_t)w * n + y) * n + x;
+    const float2 vv = g.v[at];
+    g.ckpt[at] = vv;
+    return cmul(transmission(g.h[(size_t)y * n + x], g.chan[w]), vv);
+  }
+}
+
+// One thread per pixel (any n).
+template <int MODE>
+__global__ void k_prep_field(PrepArgs g, Parts X, int n, int kp) {
+  const int wy = blockIdx.x, w = wy / n, y = wy % n;
+  for (int x = threadIdx.x; x < n; x += blockDim.x) {
+    const float2 u = prep_value<MODE>(g, n, w, y, x);
+    split_store(X, gemm_tiled((size_t)wy, x, kp), u.x);
+    split_store(X, gemm_tiled((size_t)wy, n + x, kp), u.y);
+  }
+}
+
+// One thread per 8 pixels of a row (n % 8 == 0): 16-byte accesses on every
+// array.  A warp takes 8 rows x 4 neighbouring groups, so that an operand store
+// covers whole 128-byte core matrices and a field access 256 bytes of each row.
+// Bound by memory (24 bytes a pixel with the checkpoint).  All field kernels of
+// a 128-channel, 8-layer, 256 x 256 step: 1784 us with one thread per operand
+// entry (each value formed twice, 2-byte stores scattered over the tiles, a
+// serial channel loop per pixel in the adjoint) -> 813 us.
+struct Px8 {
+  int wy, w, y, x0;  // operand row, channel, field row, first pixel
+};
+__device__ __forceinline__ bool px8(size_t i, int n, int rows, Px8& p) {
+  const int groups = n / 8;
+  const size_t g = i >> 3;
+  p.wy = (int)(g / groups) * 8 + (int)(i & 7);
+  p.x0 = (int)(g % groups) * 8;
+  p.w = p.wy / n;
+  p.y = p.wy - p.w * n;
+  return p.wy < rows;
+}
+template <int MODE>
+__global__ void __launch_bounds__(256) k_prep_field8(PrepArgs g, Parts X, int n, int kp, int rows) {
+  Px8 p;
+  if (!px8((size_t)blockIdx.x * blockDim.x + threadIdx.x, n, rows, p)) return;
+  float re[8], im[8];
+  if constexpr (MODE == PREP_LAYER) {
+    const size_t at = (size_t)p.wy * n + p.x0;
+    const float4* v4 = reinterpret_cast<const float4*>(g.v + at);
+    const float* hp = g.h + (size_t)p.y * n + p.x0;
+    float4 v[4];
+    float hv[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = v4[q];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) hv[e] = __ldg(hp + e);  // the caller's array: any 4-byte alignment
+    const ChanConst cc = g.chan[p.w];
+    float4* c4 = reinterpret_cast<float4*>(g.ckpt + at);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      c4[q] = v[q];
+      const float2 u0 = cmul(transmission(hv[2 * q], cc), make_float2(v[q].x, v[q].y));
+      const float2 u1 = cmul(transmission(hv[2 * q + 1], cc), make_float2(v[q].z, v[q].w));
+      re[2 * q] = u0.x, im[2 * q] = u0.y, re[2 * q + 1] = u1.x, im[2 * q + 1] = u1.y;
     }
-    split_store(X, gemm_tiled((size_t)wy, c, kp), val);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float2 u = prep_value<MODE>(g, n, p.w, p.y, p.x0 + e);
+      re[e] = u.x, im[e] = u.y;
+    }
   }
-}
-
-// zero the K entries [k_from, kp) of operand rows [0, rows) (the padding of
-// K past the data, which the epilogues do not write)
-__global__ void k_zero_kpad(Parts X, size_t rows, int k_from, int kp) {
-  const int wk = kp - k_from;
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows * (size_t)wk) return;
-  const size_t r = i / wk;
-  const int k = k_from + (int)(i % wk);
-  const size_t at = gemm_tiled(r, k, kp);
-  const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
-  for (int q = 0; q < X.k; ++q) X.p[q][at] = z;
-}
-
-// adjoint seed on the FOV: 2 dL/dI o, zero elsewhere
-__global__ void k_field_seed(float2* __restrict__ field, const float2* __restrict__ o, const float* __restrict__ dLdI,
-                             int n, int of, int fov, size_t total) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const size_t w = i / ((size_t)n * n);
-  const int y = (int)((i / n) % n), x = (int)(i % n);
-  const int fy = y - of, fx = x - of;
-  float2 g = make_float2(0.f, 0.f);
-  if (fy >= 0 && fy < fov && fx >= 0 && fx < fov) {
-    const size_t q = (w * fov + fy) * fov + fx;
-    g = cscale(o[q], 2.0f * dLdI[q]);
-  }
-  field[i] = g;
+  split_store8(X, gemm_tiled((size_t)p.wy, p.x0, kp), re);
+  split_store8(X, gemm_tiled((size_t)p.wy, n + p.x0, kp), im);
 }
 
 // adjoint layer: per pixel, over the chunk's channels in order:
-//   partial += Re(conj(grad_u) c t v);  grad_v = conj(t) grad_u (in place)
-__global__ void k_field_adj(float2* __restrict__ field, const float2* __restrict__ ckpt, size_t ckpt_stride,
-                            const float* __restrict__ h, const ChanConst* __restrict__ chan, float* __restrict__ partial,
-                            int nwc, int n) {
-  const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t n2 = (size_t)n * n;
+//   partial += Re(conj(grad_u) c t v);  grad_v = conj(t) grad_u -> operand rows
+//   (FIRST: not for the first layer, where the adjoint ends)
+template <bool FIRST>
+__global__ void k_field_adj(const float2* __restrict__ field, const float2* __restrict__ ckpt,
+                            const float* __restrict__ h, const ChanConst* __restrict__ chan,
+                            float* __restrict__ partial, Parts X, int nwc, int n, int kp) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n2 = n * n;
   if (p >= n2) return;
+  const int y = p / n, x = p - y * n;
   const float hv = h[p];
   float acc = 0.f;
   for (int w = 0; w < nwc; ++w) {
     const ChanConst cc = chan[w];
-    const float2 au = field[w * n2 + p];
+    const float2 au = field[(size_t)w * n2 + p];
     const float2 tt = transmission(hv, cc);
-    const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, ckpt[(size_t)w * ckpt_stride + p]));
+    const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, ckpt[(size_t)w * n2 + p]));
     acc = fmaf(au.x, cu.x, fmaf(au.y, cu.y, acc));
-    field[w * n2 + p] = cmulc(au, tt);
+    if constexpr (!FIRST) {
+      const float2 u = cmulc(au, tt);
+      split_store(X, gemm_tiled((size_t)w * n + y, x, kp), u.x);
+      split_store(X, gemm_tiled((size_t)w * n + y, n + x, kp), u.y);
+    }
   }
   partial[p] = acc;
+}
+
+// The same with one thread per 8 pixels of a row (n % 8 == 0, mapping as
+// k_prep_field8) and the chunk's channels in gridDim.y slices, each with a
+// partial plane of its own (part_stride apart): enough threads to fill the
+// chip, and FP32 sums of fewer terms.
+template <bool FIRST>
+__global__ void __launch_bounds__(128) k_field_adj8(const float2* __restrict__ field, const float2* __restrict__ ckpt,
+                                                    const float* __restrict__ h, const ChanConst* __restrict__ chan,
+                                                    float* __restrict__ partial, size_t part_stride, Parts X, int nwc,
+                                                    int n, int kp) {
+  Px8 p;
+  if (!px8((size_t)blockIdx.x * blockDim.x + threadIdx.x, n, n, p)) return;  // rows of one channel: w = 0
+  const int per = (nwc + gridDim.y - 1) / gridDim.y;
+  const int w0 = blockIdx.y * per, w1 = min(nwc, w0 + per);
+  const size_t n2 = (size_t)n * n, at = (size_t)p.y * n + p.x0;
+  float hv[8], acc[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) acc[e] = 0.f, hv[e] = __ldg(h + at + e);  // h: the caller's, any 4-byte alignment
+  for (int w = w0; w < w1; ++w) {
+    const ChanConst cc = chan[w];
+    const float4* f4 = reinterpret_cast<const float4*>(field + (size_t)w * n2 + at);
+    const float4* c4 = reinterpret_cast<const float4*>(ckpt + (size_t)w * n2 + at);
+    float4 f[4], c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f[q] = f4[q], c[q] = c4[q];
+    float re[8], im[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float2 au = (e & 1) ? make_float2(f[e / 2].z, f[e / 2].w) : make_float2(f[e / 2].x, f[e / 2].y);
+      const float2 v = (e & 1) ? make_float2(c[e / 2].z, c[e / 2].w) : make_float2(c[e / 2].x, c[e / 2].y);
+      const float2 tt = transmission(hv[e], cc);
+      const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, v));
+      acc[e] = fmaf(au.x, cu.x, fmaf(au.y, cu.y, acc[e]));
+      const float2 u = cmulc(au, tt);
+      re[e] = u.x, im[e] = u.y;
+    }
+    if constexpr (!FIRST) {
+      split_store8(X, gemm_tiled((size_t)w * n + p.y, p.x0, kp), re);
+      split_store8(X, gemm_tiled((size_t)w * n + p.y, n + p.x0, kp), im);
+    }
+  }
+  float4* out = reinterpret_cast<float4*>(partial + blockIdx.y * part_stride + at);
+  out[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  out[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
 }
 
 // ------------------------------------------------------------ one propagation
@@ -529,75 +623,102 @@ static void set_terms(GemmArgs& g, const Parts& A, const Parts& B) {
   }
 }
 
-static cudaError_t zero_kpad(const Parts& X, size_t rows, int k_from, int kp, int* launches, cudaStream_t s) {
-  if (k_from >= kp) return cudaSuccess;
-  const size_t total = rows * (size_t)(kp - k_from);
-  k_zero_kpad<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(X, rows, k_from, kp);
-  ++*launches;
-  return cudaGetLastError();
-}
-
-// X rows (w, y) of the chunk hold the field; computes the propagated field
-// (into fld) or, with o non-null, the output plane.  Operands alternate
-// between the X and Y buffers: X1 (field) -> Y (after the row DFT) -> X (after
-// the column DFT and H) -> Y (after the column IDFT) -> field.
+// X1 rows (w, y) of the chunk hold the field; computes the propagated field
+// (into fld) or, with o non-null, the output plane.  Operands: X1 (field) -> Y1
+// (after the row DFT) -> X2 (after the column DFT and H) -> Y2 (after the
+// column IDFT) -> field.  Each has its own buffer, so that the K entries that
+// pad its rows to whole 64s, zeroed once at create, stay zero.
 cudaError_t gemm_propagate(GemmPlan& p, int nwc, const float2* Hq, int hs, bool adj, float2* o, float* I, int of,
                            int fov, const Misalign& mis, int* launches, cudaStream_t s) {
   const int n = p.n, m = p.m;
-  auto pad256 = [](int v) { return (v + 255) / 256 * 256; };
+  auto pad = [](int v, int q) { return (v + q - 1) / q * q; };
   const int c1 = nwc * n, c2 = nwc * m;
   cudaError_t e;
   GemmArgs g;
   std::memset(&g, 0, sizeof(g));
   g.err = p.err;
-  // row DFT: D = F X1^T -> Y rows (w, kx), K = p n + y
-  if ((e = zero_kpad(p.Y, (size_t)pad256(c2), 2 * n, p.kp1, launches, s)) != cudaSuccess) return e;
-  set_terms(g, p.F, p.X);
-  g.rows = p.rp1; g.cols = c1; g.K = p.kp1; g.w_is_b = 0;
-  g.mode = GEMM_OUT_ROWS; g.vrows = 2 * m; g.vcols = c1; g.nk = m; g.nj = n; g.xo = p.Y; g.kpo = p.kp1;
+  // row DFT: D = F X1^T -> Y1 rows (w, kx), K = p n + y
+  set_terms(g, p.F, p.X1);
+  g.rows = pad(2 * m, GTM); g.cols = c1; g.K = p.kp1; g.w_is_b = 0;
+  g.mode = GEMM_OUT_ROWS; g.vrows = 2 * m; g.vcols = c1; g.nk = m; g.nj = n; g.xo = p.Y1; g.kpo = p.kp1;
   if ((e = launch_tc_gemm(g, s)) != cudaSuccess) return e;
-  ++*launches;
-  // column DFT and H: D = Y F^T -> X rows (w, kx), K = ky | m + ky
-  if ((e = zero_kpad(p.X, (size_t)pad256(c2), 2 * m, p.kp2, launches, s)) != cudaSuccess) return e;
-  set_terms(g, p.Y, p.F);
-  g.rows = pad256(c2); g.cols = 2 * m; g.K = p.kp1; g.w_is_b = 1;
-  g.mode = GEMM_OUT_SPECTRUM; g.vrows = c2; g.vcols = 2 * m; g.xo = p.X; g.kpo = p.kp2;
+  // column DFT and H: D = Y1 F^T -> X2 rows (w, kx), K = ky | m + ky
+  set_terms(g, p.Y1, p.F);
+  g.rows = pad(c2, GTM); g.cols = 2 * m; g.K = p.kp1; g.w_is_b = 1;
+  g.mode = GEMM_OUT_SPECTRUM; g.vrows = c2; g.vcols = 2 * m; g.xo = p.X2; g.kpo = p.kp2;
   g.Hq = Hq; g.hs = hs; g.m = m; g.adj = adj ? 1 : 0; g.mis = mis;
   if ((e = launch_tc_gemm(g, s)) != cudaSuccess) return e;
-  ++*launches;
-  // column IDFT: D = G X^T -> Y rows (w, y), K = p m + kx
-  if ((e = zero_kpad(p.Y, (size_t)pad256(c1), 2 * m, p.kp2, launches, s)) != cudaSuccess) return e;
-  set_terms(g, p.G, p.X);
-  g.rows = p.rp2; g.cols = c2; g.K = p.kp2; g.w_is_b = 0;
-  g.mode = GEMM_OUT_ROWS; g.vrows = 2 * n; g.vcols = c2; g.nk = n; g.nj = m; g.xo = p.Y; g.kpo = p.kp2;
+  // column IDFT: D = G X2^T -> Y2 rows (w, y), K = p m + kx
+  set_terms(g, p.G, p.X2);
+  g.rows = pad(2 * n, GTM); g.cols = c2; g.K = p.kp2; g.w_is_b = 0;
+  g.mode = GEMM_OUT_ROWS; g.vrows = 2 * n; g.vcols = c2; g.nk = n; g.nj = m; g.xo = p.Y2; g.kpo = p.kp2;
   if ((e = launch_tc_gemm(g, s)) != cudaSuccess) return e;
-  ++*launches;
-  // row IDFT: D = Y G^T -> field (or the output plane)
-  set_terms(g, p.Y, p.G);
-  g.rows = pad256(c1); g.cols = 2 * n; g.K = p.kp2; g.w_is_b = 1;
+  // row IDFT: D = Y2 G^T -> field (or the output plane)
+  set_terms(g, p.Y2, p.G);
+  g.rows = pad(c1, GTM); g.cols = 2 * n; g.K = p.kp2; g.w_is_b = 1;
   g.mode = GEMM_OUT_FIELD; g.vrows = c1; g.vcols = 2 * n; g.fld = p.fld; g.o = o; g.I = I; g.n = n; g.of = of;
   g.fov = fov;
   if ((e = launch_tc_gemm(g, s)) != cudaSuccess) return e;
-  ++*launches;
+  *launches += 4;
   return cudaSuccess;
 }
 
-cudaError_t gemm_prep_field(GemmPlan& p, int nwc, const float2* v, float2* ckpt, const float* h,
-                            const ChanConst* chan, int mode, int a_off, int a_w, cudaStream_t s) {
-  k_prep_field<<<nwc * p.n, 128, 0, s>>>(v, ckpt, h, chan, p.X, p.n, p.kp1, mode, a_off, a_w);
+template <int MODE>
+static cudaError_t launch_prep(GemmPlan& p, int nwc, const PrepArgs& g, cudaStream_t s) {
+  if (p.n % 8 == 0) {
+    const int rows = nwc * p.n;
+    const size_t threads = (size_t)rows * (p.n / 8);
+    k_prep_field8<MODE><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(g, p.X1, p.n, p.kp1, rows);
+  } else {
+    k_prep_field<MODE><<<nwc * p.n, 128, 0, s>>>(g, p.X1, p.n, p.kp1);
+  }
   return cudaGetLastError();
 }
 
-cudaError_t gemm_seed(GemmPlan& p, int nwc, const float2* o, const float* dLdI, int of, int fov, cudaStream_t s) {
-  const size_t total = (size_t)nwc * p.n * p.n;
-  k_field_seed<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(p.fld, o, dLdI, p.n, of, fov, total);
-  return cudaGetLastError();
+cudaError_t gemm_prep_aperture(GemmPlan& p, int nwc, int a_off, int a_w, cudaStream_t s) {
+  PrepArgs g = {};
+  g.a_off = a_off;
+  g.a_w = a_w;
+  return launch_prep<PREP_APERTURE>(p, nwc, g, s);
 }
 
-cudaError_t gemm_adj_layer(GemmPlan& p, int nwc, const float2* ckpt, size_t ckpt_stride, const float* h,
-                           const ChanConst* chan, float* partial, cudaStream_t s) {
-  const size_t n2 = (size_t)p.n * p.n;
-  k_field_adj<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(p.fld, ckpt, ckpt_stride, h, chan, partial, nwc, p.n);
+cudaError_t gemm_prep_layer(GemmPlan& p, int nwc, float2* ckpt, const float* h, const ChanConst* chan,
+                            cudaStream_t s) {
+  PrepArgs g = {};
+  g.v = p.fld;
+  g.ckpt = ckpt;
+  g.h = h;
+  g.chan = chan;
+  return launch_prep<PREP_LAYER>(p, nwc, g, s);
+}
+
+cudaError_t gemm_prep_seed(GemmPlan& p, int nwc, const float2* o, const float* dLdI, int of, int fov, cudaStream_t s) {
+  PrepArgs g = {};
+  g.o = o;
+  g.dLdI = dLdI;
+  g.of = of;
+  g.fov = fov;
+  return launch_prep<PREP_SEED>(p, nwc, g, s);
+}
+
+// about 128 K threads, in whole channels
+int gemm_adj_slices(const GemmPlan& p) {
+  if (p.n % 8 != 0) return 1;
+  return std::max(1, std::min(p.nwc, (1 << 20) / (p.n * p.n)));
+}
+
+cudaError_t gemm_adj_layer(GemmPlan& p, int nwc, const float2* ckpt, const float* h, const ChanConst* chan,
+                           float* partial, size_t part_stride, bool first, cudaStream_t s) {
+  const int n2 = p.n * p.n;
+  if (p.n % 8 == 0) {
+    const dim3 grid((n2 / 8 + 127) / 128, gemm_adj_slices(p));
+    if (first) k_field_adj8<true><<<grid, 128, 0, s>>>(p.fld, ckpt, h, chan, partial, part_stride, p.X1, nwc, p.n, p.kp1);
+    else k_field_adj8<false><<<grid, 128, 0, s>>>(p.fld, ckpt, h, chan, partial, part_stride, p.X1, nwc, p.n, p.kp1);
+  } else {
+    const int blocks = (n2 + 255) / 256;
+    if (first) k_field_adj<true><<<blocks, 256, 0, s>>>(p.fld, ckpt, h, chan, partial, p.X1, nwc, p.n, p.kp1);
+    else k_field_adj<false><<<blocks, 256, 0, s>>>(p.fld, ckpt, h, chan, partial, p.X1, nwc, p.n, p.kp1);
+  }
   return cudaGetLastError();
 }
 

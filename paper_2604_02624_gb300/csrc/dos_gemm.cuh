@@ -95,26 +95,29 @@ struct GemmPlan {
   int parts;                // bf16 parts per operand: 2 (three products) or 3 (six)
   Parts F;                  // [rp1][kp1] each
   Parts G;                  // [rp2][kp2] each
-  Parts X;                  // data operand (product input), whole 256-row tiles
-  Parts Y;                  // the other data operand buffer (products alternate X -> Y -> X -> Y)
+  // data operands, whole 256-row tiles: X1 (w, y) and Y1 (w, kx) with pitch kp1,
+  // X2 (w, kx) and Y2 (w, y) with pitch kp2; their padding entries are zero
+  Parts X1, Y1, X2, Y2;
   float2* fld;              // FP32 working field [nwc][n][n]
   int* err;
 };
 
 cudaError_t launch_build_dft(GemmPlan& p, cudaStream_t s);
 
-// One propagation (forward H or conj H) of the chunk's field held in X rows
+// One propagation (forward H or conj H) of the chunk's field held in X1 rows
 // (w, y); the result goes to p.fld, or to o / I on the FOV when o is given.
 // Adds the number of kernels it launched to *launches.
 cudaError_t gemm_propagate(GemmPlan& p, int nwc, const float2* Hq, int hs, bool adj, float2* o, float* I, int of,
                            int fov, const Misalign& mis, int* launches, cudaStream_t s);
-// field -> X rows: mode 0 copy, mode 1 checkpoint + Eq. 1 modulation, mode 2 aperture.
-cudaError_t gemm_prep_field(GemmPlan& p, int nwc, const float2* v, float2* ckpt, const float* h,
-                            const ChanConst* chan, int mode, int a_off, int a_w, cudaStream_t s);
-// p.fld = 2 dL/dI o on the FOV, zero elsewhere
-cudaError_t gemm_seed(GemmPlan& p, int nwc, const float2* o, const float* dLdI, int of, int fov, cudaStream_t s);
-// gradient partial of one layer over the chunk, p.fld <- conj(t) p.fld
-cudaError_t gemm_adj_layer(GemmPlan& p, int nwc, const float2* ckpt, size_t ckpt_stride, const float* h,
-                           const ChanConst* chan, float* partial, cudaStream_t s);
+// X1 rows of the next propagation: the square aperture; the field p.fld,
+// checkpointed and modulated by Eq. 1; the adjoint seed 2 dL/dI o on the FOV.
+cudaError_t gemm_prep_aperture(GemmPlan& p, int nwc, int a_off, int a_w, cudaStream_t s);
+cudaError_t gemm_prep_layer(GemmPlan& p, int nwc, float2* ckpt, const float* h, const ChanConst* chan, cudaStream_t s);
+cudaError_t gemm_prep_seed(GemmPlan& p, int nwc, const float2* o, const float* dLdI, int of, int fov, cudaStream_t s);
+// gradient partials of one layer over the chunk (gemm_adj_slices planes,
+// part_stride apart), X1 rows <- conj(t) p.fld (not for the first layer)
+int gemm_adj_slices(const GemmPlan& p);
+cudaError_t gemm_adj_layer(GemmPlan& p, int nwc, const float2* ckpt, const float* h, const ChanConst* chan,
+                           float* partial, size_t part_stride, bool first, cudaStream_t s);
 
 }  // namespace dos
