@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
+  pdl_wait();
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = sm.tmem;
@@ -387,8 +388,7 @@ static cudaError_t launch_mode(const GemmArgs& g, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int tiles = (g.rows / GTM) * ((g.cols + GTN - 1) / GTN);
-  k_tc_gemm<MODE><<<std::min(tiles, sms), kGemmThreads, sm, s>>>(g);
-  return cudaGetLastError();
+  return launch_next(k_tc_gemm<MODE>, dim3(std::min(tiles, sms)), kGemmThreads, sm, s, g);
 }
 
 cudaError_t launch_tc_gemm(const GemmArgs& g, cudaStream_t s) {
@@ -470,6 +470,7 @@ __device__ __forceinline__ float2 prep_value(const PrepArgs& g, int n, int w, in
 // One thread per pixel (any n).
 template <int MODE>
 __global__ void k_prep_field(PrepArgs g, Parts X, int n, int kp) {
+  pdl_wait();
   const int wy = blockIdx.x, w = wy / n, y = wy % n;
   for (int x = threadIdx.x; x < n; x += blockDim.x) {
     const float2 u = prep_value<MODE>(g, n, w, y, x);
@@ -499,6 +500,7 @@ __device__ __forceinline__ bool px8(size_t i, int n, int rows, Px8& p) {
 }
 template <int MODE>
 __global__ void __launch_bounds__(256) k_prep_field8(PrepArgs g, Parts X, int n, int kp, int rows) {
+  pdl_wait();
   Px8 p;
   if (!px8((size_t)blockIdx.x * blockDim.x + threadIdx.x, n, rows, p)) return;
   float re[8], im[8];
@@ -539,6 +541,7 @@ template <bool FIRST>
 __global__ void k_field_adj(const float2* __restrict__ field, const float2* __restrict__ ckpt,
                             const float* __restrict__ h, const ChanConst* __restrict__ chan,
                             float* __restrict__ partial, Parts X, int nwc, int n, int kp) {
+  pdl_wait();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int n2 = n * n;
   if (p >= n2) return;
@@ -569,6 +572,7 @@ __global__ void __launch_bounds__(128) k_field_adj8(const float2* __restrict__ f
                                                     const float* __restrict__ h, const ChanConst* __restrict__ chan,
                                                     float* __restrict__ partial, size_t part_stride, Parts X, int nwc,
                                                     int n, int kp) {
+  pdl_wait();
   Px8 p;
   if (!px8((size_t)blockIdx.x * blockDim.x + threadIdx.x, n, n, p)) return;  // rows of one channel: w = 0
   const int per = (nwc + gridDim.y - 1) / gridDim.y;
@@ -668,11 +672,10 @@ static cudaError_t launch_prep(GemmPlan& p, int nwc, const PrepArgs& g, cudaStre
   if (p.n % 8 == 0) {
     const int rows = nwc * p.n;
     const size_t threads = (size_t)rows * (p.n / 8);
-    k_prep_field8<MODE><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(g, p.X1, p.n, p.kp1, rows);
-  } else {
-    k_prep_field<MODE><<<nwc * p.n, 128, 0, s>>>(g, p.X1, p.n, p.kp1);
+    return launch_next(k_prep_field8<MODE>, dim3((unsigned)((threads + 255) / 256)), 256, 0, s, g, p.X1, p.n, p.kp1,
+                       rows);
   }
-  return cudaGetLastError();
+  return launch_next(k_prep_field<MODE>, dim3(nwc * p.n), 128, 0, s, g, p.X1, p.n, p.kp1);
 }
 
 cudaError_t gemm_prep_aperture(GemmPlan& p, int nwc, int a_off, int a_w, cudaStream_t s) {
@@ -712,14 +715,11 @@ cudaError_t gemm_adj_layer(GemmPlan& p, int nwc, const float2* ckpt, const float
   const int n2 = p.n * p.n;
   if (p.n % 8 == 0) {
     const dim3 grid((n2 / 8 + 127) / 128, gemm_adj_slices(p));
-    if (first) k_field_adj8<true><<<grid, 128, 0, s>>>(p.fld, ckpt, h, chan, partial, part_stride, p.X1, nwc, p.n, p.kp1);
-    else k_field_adj8<false><<<grid, 128, 0, s>>>(p.fld, ckpt, h, chan, partial, part_stride, p.X1, nwc, p.n, p.kp1);
-  } else {
-    const int blocks = (n2 + 255) / 256;
-    if (first) k_field_adj<true><<<blocks, 256, 0, s>>>(p.fld, ckpt, h, chan, partial, p.X1, nwc, p.n, p.kp1);
-    else k_field_adj<false><<<blocks, 256, 0, s>>>(p.fld, ckpt, h, chan, partial, p.X1, nwc, p.n, p.kp1);
+    return launch_next(first ? k_field_adj8<true> : k_field_adj8<false>, grid, 128, 0, s, p.fld, ckpt, h, chan, partial,
+                       part_stride, p.X1, nwc, p.n, p.kp1);
   }
-  return cudaGetLastError();
+  return launch_next(first ? k_field_adj<true> : k_field_adj<false>, dim3((n2 + 255) / 256), 256, 0, s, p.fld, ckpt, h,
+                     chan, partial, p.X1, nwc, p.n, p.kp1);
 }
 
 }  // namespace dos

@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   __shared__ double tot[3];
   __shared__ float sg_sh;
   __shared__ bool last;
+  pdl_wait();
   const int w = blockIdx.x, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int fd = fov / b, det2 = fd * fd;
   const bool keep = det2 <= kLossKeep;
@@ -194,8 +195,8 @@ cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, 
   const float scale = (float)(2.0 / norm);  // dL/dD = 2 (D - T) / norm
   const int det2 = (fov / bin) * (fov / bin);
   const size_t sm = det2 <= kLossKeep ? sizeof(float) * det2 : 0;
-  k_loss<<<nw, kRedThreads, sm, s>>>(o, T, st, fov, bin, dLdI, scale, norm, mode, psnr, d_loss, ticket);
-  return cudaGetLastError();
+  return launch_next(k_loss, dim3(nw), kRedThreads, sm, s, o, T, st, fov, bin, dLdI, scale, norm, mode, psnr, d_loss,
+                     ticket);
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_loss_final(const LossStats* __restrict__ st, int nw,
@@ -242,6 +243,7 @@ __global__ void __launch_bounds__(kGradPx * kGradSlices) k_grad_reduce(const flo
                                                                        float* __restrict__ grad, int n_parts,
                                                                        size_t count, size_t n2) {
   __shared__ float2 sh[kGradSlices][kGradPx];
+  pdl_wait();
   const int lane = threadIdx.x % kGradPx, slice = threadIdx.x / kGradPx;
   const size_t g = (size_t)blockIdx.x * kGradPx + lane;
   const int per = (n_parts + kGradSlices - 1) / kGradSlices;
@@ -276,8 +278,7 @@ __global__ void __launch_bounds__(kGradPx * kGradSlices) k_grad_reduce(const flo
 cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2,
                                cudaStream_t s) {
   const unsigned blocks = (unsigned)((count + kGradPx - 1) / kGradPx);
-  k_grad_reduce<<<blocks, kGradPx * kGradSlices, 0, s>>>(partial, grad, n_parts, count, n2);
-  return cudaGetLastError();
+  return launch_next(k_grad_reduce, dim3(blocks), kGradPx * kGradSlices, 0, s, partial, grad, n_parts, count, n2);
 }
 
 }  // namespace dos

@@ -76,8 +76,11 @@ struct Pass {
   static constexpr size_t smem_bytes(int lines) { return sizeof(float2) * (LF::TWS + (size_t)lines * ZL); }
   static constexpr size_t row_smem_bytes(int lines) { return sizeof(float2) * (LF::TWS + (size_t)lines * RZL); }
 
+  // the start of every kernel: the twiddles (made at create) do not depend on
+  // the grid before this one
   __device__ static __forceinline__ void load_tw(float2* tw, const float2* g) {
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = g[i];
+    pdl_wait();
     __syncthreads();
   }
 
@@ -422,8 +425,7 @@ static cudaError_t launch_k(K kernel, dim3 grid, int threads, size_t smem, const
   if (grid.x == 0 || grid.y == 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kernel<<<grid, threads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_next(kernel, grid, threads, smem, s, a);
 }
 
 // Each launcher picks the halved (pruned) kernels when the design allows it.

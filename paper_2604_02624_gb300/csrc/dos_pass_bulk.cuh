@@ -237,6 +237,7 @@ struct PassBulk {
     if constexpr (MIS) {
       for (int i = threadIdx.x; i <= M / 2; i += blockDim.x) ey[i] = shift_phase(i, a.mis.sy);
     }
+    pdl_wait();
     __syncthreads();
     auto tensor_copy = [](float2* dst, const CUtensorMap* map, int x, int y, int zc, uint64_t* b) {
       asm volatile(
@@ -389,6 +390,7 @@ struct PassBulk {
     const uint32_t bytes = (uint32_t)nrows * M * 8u;
     if (threadIdx.x == 0) bulk_bar_init(bar);
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
+    pdl_wait();
     __syncthreads();
     // thread 0 copies the block's rows of channel w, one bulk copy (M * 8 bytes) per row
     auto fetch = [&](int w) {
@@ -530,6 +532,7 @@ struct PassBulk {
     const uint32_t bytes = (uint32_t)nrows * a.n * 8u;
     if (threadIdx.x == 0) bulk_bar_init(bar);
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
+    pdl_wait();
     __syncthreads();
     auto fetch = [&](int w) {
       if (threadIdx.x != 0) return;
@@ -628,6 +631,7 @@ struct PassBulk {
       bulk_bar_init(&bar[1]);
     }
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
+    pdl_wait();
     __syncthreads();
     // thread 0 copies the block's rows of channel w: spectra (M * 8 bytes a
     // row) into the stage, checkpoint (N * 8 bytes a row) into ck
@@ -850,9 +854,8 @@ struct PassBulkLaunch {
                             : (adj ? k_col_bulk<LF, RL, H, true, false> : k_col_bulk<LF, RL, H, false, false>);
     cudaError_t e = slots(kern, PB::GT, sm, &n_slots);
     if (e != cudaSuccess) return e;
-    kern<<<std::min(items, n_slots), PB::GT, sm, s>>>(a, *static_cast<const CUtensorMap*>(a.tmap),
-                                                     *static_cast<const CUtensorMap*>(a.hmap));
-    return cudaGetLastError();
+    return launch_next(kern, dim3(std::min(items, n_slots)), PB::GT, sm, s, a,
+                       *static_cast<const CUtensorMap*>(a.tmap), *static_cast<const CUtensorMap*>(a.hmap));
   }
   // The tensor copies need maps whose boxes hold the input rows (at most 256)
   // and the H tile, and M a multiple of 8 (whole 8-column groups); otherwise
@@ -875,8 +878,7 @@ struct PassBulkLaunch {
     PassArgs b = a;
     const int rb = (a.n + RL - 1) / RL;
     b.chunk = balanced_chunk(a.nw, rb, n_slots, kRowChunk);
-    kernel<<<dim3(rb, (a.nw + b.chunk - 1) / b.chunk), PB::RT, sm, s>>>(b);
-    return cudaGetLastError();
+    return launch_next(kernel, dim3(rb, (a.nw + b.chunk - 1) / b.chunk), PB::RT, sm, s, b);
   }
   template <bool H>
   static cudaError_t row_fwd_h(const PassArgs& a, bool save, cudaStream_t s) {

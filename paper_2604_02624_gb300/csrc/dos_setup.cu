@@ -97,6 +97,7 @@ __device__ __forceinline__ float2 longer(float2 h, float sq, float sq_lo, float2
 __global__ void __launch_bounds__(256) k_longer_table(float4* __restrict__ out, const float4* __restrict__ Hq,
                                                       const float2* __restrict__ sq, const float2* __restrict__ sq_lo,
                                                       float2 dz, size_t pairs) {
+  pdl_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= pairs) return;
   const float4 h = Hq[i];
@@ -110,10 +111,9 @@ __global__ void __launch_bounds__(256) k_longer_table(float4* __restrict__ out, 
 cudaError_t launch_longer_table(float2* out, const float2* Hq, const float* sq, const float* sq_lo, float2 dz,
                                 size_t count, cudaStream_t s) {
   const size_t pairs = count / 2;
-  k_longer_table<<<(unsigned)((pairs + 255) / 256), 256, 0, s>>>(
-      reinterpret_cast<float4*>(out), reinterpret_cast<const float4*>(Hq), reinterpret_cast<const float2*>(sq),
-      reinterpret_cast<const float2*>(sq_lo), dz, pairs);
-  return cudaGetLastError();
+  return launch_next(k_longer_table, dim3((unsigned)((pairs + 255) / 256)), 256, 0, s,
+                     reinterpret_cast<float4*>(out), reinterpret_cast<const float4*>(Hq),
+                     reinterpret_cast<const float2*>(sq), reinterpret_cast<const float2*>(sq_lo), dz, pairs);
 }
 
 // Arow[k] = sum_{x = offset}^{offset + width - 1} exp(-2 pi j k x / m)
