@@ -142,6 +142,7 @@ struct dos_ctx {
   float* h_fwd = nullptr;
   dos::LossStats* stats = nullptr;
   double* d_loss = nullptr;
+  unsigned* col_work = nullptr;     // items drawn in the running column pass (zero between launches)
   unsigned* loss_ticket = nullptr;  // channels done in the running loss kernel (zero between launches)
   double* h_loss = nullptr;  // pinned
   // channels per block of the adjoint row pass, plain and prefetching
@@ -271,6 +272,7 @@ struct dos_ctx {
     a.chunk = adj_chunk();
     a.n_chunks = chunks_of(a.chunk);
     a.err = d_err;
+    a.work = col_work;
     a.tmap = have_tmap ? &tmap_S : nullptr;
     a.tmap_rows = n;
     a.hmap = have_tmap ? &tmap_H : nullptr;
@@ -511,6 +513,8 @@ int build(dos_ctx* x, const dos_config* c) {
   if ((rc = x->alloc(&x->h_fwd, (size_t)x->K * n2, "saved thickness"))) return rc;
   if ((rc = x->alloc(&x->stats, (size_t)x->nw, "loss statistics"))) return rc;
   if ((rc = x->alloc(&x->d_loss, 1, "loss"))) return rc;
+  if ((rc = x->alloc(&x->col_work, 1, "column item counter"))) return rc;
+  DOS_CUDA(cudaMemsetAsync(x->col_work, 0, sizeof(unsigned), x->stream), "column item counter");
   if ((rc = x->alloc(&x->loss_ticket, 1, "loss ticket"))) return rc;
   DOS_CUDA(cudaMemsetAsync(x->loss_ticket, 0, sizeof(unsigned), x->stream), "loss ticket");
   if ((rc = x->alloc(&x->dLdI_step, (size_t)x->nw * x->fov * x->fov, "step seed"))) return rc;
@@ -564,6 +568,7 @@ int flag_after_sync(dos_ctx* c) {
   if (*c->h_err) {
     *c->h_err = 0;
     DOS_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream), "error flag");
+    DOS_CUDA(cudaMemsetAsync(c->col_work, 0, sizeof(unsigned), c->stream), "column item counter");
     return fail(DOS_ERR_TIMEOUT, "a bounded wait gave up (mbarrier wait for a tensor-core commit or a bulk copy "
                                  "expired); results of the call are invalid");
   }

@@ -114,6 +114,7 @@ struct PassArgs {
   int n_chunks;
   bool displaced;         // column pass: the gap carries a displacement that Hq does not hold (mis)
   Misalign mis;           // its lateral shift; and, with mis.sq, its length change (plain kernel only)
+  unsigned* work;         // item counter of the bulk column pass, 0 between launches
   int* err;               // set to 1 by a bulk-copy pass whose bounded wait expired
   int stall;              // fault injection (tests): 1 = the bulk pass expects bytes that are never
                           // copied; 2 = its copies land but odd threads give up their first wait;

@@ -186,13 +186,13 @@ struct PassBulk {
   static_assert(ZX % 2 == 0 && ZLB % 16 == 2, "16-byte aligned rows, conflict-free line stride");
   static_assert(LF::ALT, "the two line DFTs of an item alternate their exchange layouts");
   // dynamic shared memory (from a 128-byte aligned base):
-  //   stage[rows][8] | H tile[8][M/2+2] | exchange[8][ZLB] | tw[TWS] | barrier[2] | ey[M/2+1] (MIS)
+  //   stage[rows][8] | H tile[8][M/2+2] | exchange[8][ZLB] | tw[TWS] | barrier[2] | next item | ey[M/2+1] (MIS)
   // (the H tile starts on a 128-byte boundary, as tensor copies need)
   static constexpr int HTILE_PAD = (HTILE + 15) / 16 * 16;
   static size_t col_smem(int n, bool mis) {
     return 128 + sizeof(float2) * ((size_t)col_stage(n) + (size_t)HTILE_PAD + (size_t)GW * ZLB + LF::TWS + 1 +
                                    (mis ? M / 2 + 1 : 0)) +
-           2 * sizeof(uint64_t);
+           3 * sizeof(uint64_t);
   }
 
   // MIS: displaced layers.  The table of the copies already holds the gap's
@@ -212,6 +212,7 @@ struct PassBulk {
     float2* zb = stage + (size_t)col_stage(a.n) + HTILE_PAD;
     float2* tw = tw_align(zb + (size_t)GW * ZLB);
     uint64_t* bar = reinterpret_cast<uint64_t*>(tw + LF::TWS);  // [0] input rows, [1] H tile
+    int* next_item = reinterpret_cast<int*>(bar + 2);           // thread 0's, read after the first barrier
     const int lc = threadIdx.x % GW, t = threadIdx.x / GW;
     const bool leader = threadIdx.x == 0;  // issues the copies
     float2* z = zb + lc * ZLB;
@@ -233,7 +234,7 @@ struct PassBulk {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(hmap)) : "memory");
     }
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
-    float2* ey = reinterpret_cast<float2*>(bar + 2);
+    float2* ey = reinterpret_cast<float2*>(bar + 3);
     if constexpr (MIS) {
       for (int i = threadIdx.x; i <= M / 2; i += blockDim.x) ey[i] = shift_phase(i, a.mis.sy);
     }
@@ -267,20 +268,33 @@ struct PassBulk {
     };
     bool ok = true;
     int k = 0, issued_s = 0, issued_h = 0, done_s = 0, done_h = 0;  // copies per barrier (thread 0's view)
-    if ((int)blockIdx.x < items) {
-      if (leader) fetch_s(blockIdx.x);
-      issued_s = 1;
-      if constexpr (STAGE_H) {
-        if (leader) fetch_h(blockIdx.x);
-        issued_h = 1;
-      }
+    // Items are taken in order by whichever block is free: the first gridDim by
+    // block index, the others from a counter.  (Blocks that stepped through
+    // the items by gridDim finished far apart: SMs differ in how far they are
+    // from the memory they read, and 16 of 20 warps were resident on average.
+    // 4096 x 200 launch 1.50 -> 1.34 ms, 256 x 200 103 -> 94 us, 2048 x 256
+    // 1.19 -> 1.10 ms.)
+    // Thread 0 draws two items ahead, so that the counter's answer is there
+    // when the next copy is issued.  Every block draws until its first number
+    // past the end, items draws in all: whoever drew the last one leaves the
+    // counter at 0.
+    unsigned drawn = 0;  // thread 0: the counter's answer for the item after the current one
+    if (leader) {
+      fetch_s(blockIdx.x);
+      if constexpr (STAGE_H) fetch_h(blockIdx.x);
+      drawn = atomicAdd(a.work, 1u);
     }
-    for (int it = blockIdx.x; it < items; it += gridDim.x, ++k) {
+    issued_s = 1;
+    issued_h = STAGE_H ? 1 : 0;
+    for (int it = blockIdx.x; it < items; ++k) {
       int w, c0;
       place(it, w, c0);
       const int cc = c0 + lc;  // this line's column
       const int hc = min(cc, M - cc) - table_row(c0);  // |kx|'s row of the H tile
-      const bool more = it + (int)gridDim.x < items;
+      if (leader) {
+        *next_item = (int)min(drawn + gridDim.x, (unsigned)items);
+        if (drawn == (unsigned)items - 1u) *a.work = 0u;
+      }
       // this item's input rows; a thread whose wait expires goes on to the
       // barrier with what is there, where the whole block stops
       const bool got_s = bulk_wait(&bar[0], (uint32_t)(k & 1), split_verdict(a, k));
@@ -295,13 +309,16 @@ struct PassBulk {
       ok = __syncthreads_and(got_s) != 0;  // one verdict for the whole block, past its stage reads
       if (!ok) break;
       ++done_s;
+      const int next = *next_item;
+      const bool more = next < items;
       if constexpr (SLOT_H) {
         if (leader) fetch_h(it);
         ++issued_h;
       } else if (more) {
-        if (leader) fetch_s(it + gridDim.x);
+        if (leader) fetch_s(next);
         ++issued_s;
       }
+      if (leader && more) drawn = atomicAdd(a.work, 1u);
       LF::template step2<false, LF::Q, PKC, false, ZX>(r, t, z);
       // (injected, tests: the wait of the block's last item gives up)
       const bool got_h = (a.stall == 3 && !more) ? false : bulk_wait(&bar[1], (uint32_t)(k & 1));
@@ -332,10 +349,10 @@ struct PassBulk {
       ++done_h;
       if (more) {
         if constexpr (SLOT_H) {
-          if (leader) fetch_s(it + gridDim.x);
+          if (leader) fetch_s(next);
           ++issued_s;
         } else {
-          if (leader) fetch_h(it + gridDim.x);
+          if (leader) fetch_h(next);
           ++issued_h;
         }
       }
@@ -351,8 +368,10 @@ struct PassBulk {
         const int row = t + T * i;
         if (i < EF && row >= a.out_r0 && row < a.out_r1) dst[(size_t)row * M] = r[i];
       }
+      it = next;
     }
     if (!ok && leader) {
+      // (the counter is left where it is: the host zeroes it with the flag)
       // the copies in flight land (bounded waits) before the block leaves
       if (issued_s > done_s) (void)bulk_wait(&bar[0], (uint32_t)(done_s & 1));
       if (issued_h > done_h) (void)bulk_wait(&bar[1], (uint32_t)(done_h & 1));
