@@ -550,12 +550,8 @@ __global__ void k_field_adj(const float2* __restrict__ field, const float2* __re
   float acc = 0.f;
   for (int w = 0; w < nwc; ++w) {
     const ChanConst cc = chan[w];
-    const float2 au = field[(size_t)w * n2 + p];
-    const float2 tt = transmission(hv, cc);
-    const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, ckpt[(size_t)w * n2 + p]));
-    acc = fmaf(au.x, cu.x, fmaf(au.y, cu.y, acc));
+    const float2 u = adjoint_pixel(field[(size_t)w * n2 + p], transmission(hv, cc), ckpt[(size_t)w * n2 + p], cc, acc);
     if constexpr (!FIRST) {
-      const float2 u = cmulc(au, tt);
       split_store(X, gemm_tiled((size_t)w * n + y, x, kp), u.x);
       split_store(X, gemm_tiled((size_t)w * n + y, n + x, kp), u.y);
     }
@@ -593,10 +589,7 @@ __global__ void __launch_bounds__(128) k_field_adj8(const float2* __restrict__ f
     for (int e = 0; e < 8; ++e) {
       const float2 au = (e & 1) ? make_float2(f[e / 2].z, f[e / 2].w) : make_float2(f[e / 2].x, f[e / 2].y);
       const float2 v = (e & 1) ? make_float2(c[e / 2].z, c[e / 2].w) : make_float2(c[e / 2].x, c[e / 2].y);
-      const float2 tt = transmission(hv[e], cc);
-      const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, v));
-      acc[e] = fmaf(au.x, cu.x, fmaf(au.y, cu.y, acc[e]));
-      const float2 u = cmulc(au, tt);
+      const float2 u = adjoint_pixel(au, transmission(hv[e], cc), v, cc, acc[e]);
       re[e] = u.x, im[e] = u.y;
     }
     if constexpr (!FIRST) {

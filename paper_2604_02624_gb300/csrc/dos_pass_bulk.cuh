@@ -484,11 +484,7 @@ struct PassBulk {
         for (int i = 0; i < E; ++i) {
           const int x = t + T * i;
           if (i < EF && x < a.n) {
-            const float2 au = r[i];
-            const float2 tt = transmission(__ldg(hrow + x), cc);
-            const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, ck[x]));
-            g[i] = fmaf(au.x, cu.x, fmaf(au.y, cu.y, g[i]));
-            r[i] = cmulc(au, tt);
+            r[i] = adjoint_pixel(r[i], transmission(__ldg(hrow + x), cc), ck[x], cc, g[i]);
           } else {
             r[i] = czero();
           }
@@ -724,11 +720,7 @@ struct PassBulk {
       for (int i = 0; i < E; ++i) {
         const int x = t + T * i;
         if (i < EF && x < a.n) {
-          const float2 au = r[i];
-          const float2 tt = transmission(hv[i], cc);
-          const float2 cu = cmul(make_float2(cc.c_re, cc.c_im), cmul(tt, ck[x]));
-          g[i] = fmaf(au.x, cu.x, fmaf(au.y, cu.y, g[i]));
-          r[i] = cmulc(au, tt);
+          r[i] = adjoint_pixel(r[i], transmission(hv[i], cc), ck[x], cc, g[i]);
         } else {
           r[i] = czero();
         }
