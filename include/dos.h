@@ -284,6 +284,9 @@ DOS_API int dos_quantize_thickness(const float *d_h, float *d_hq, size_t count, 
  * Returns DOS_ERR_TIMEOUT when a kernel queued since the previous check gave
  * up a bounded wait (bulk-copy or tensor-core completion); the loss and every
  * result of that work are then invalid.  The flag is cleared by the report.
+ * On the DFT-GEMM paths dos_forward and dos_backward also report, in the same
+ * way and before they queue anything, an expired wait of an earlier call that
+ * the GPU has finished by then.
  */
 DOS_API int dos_read_loss(dos_ctx *ctx, double *h_loss);
 

@@ -153,6 +153,8 @@ struct dos_ctx {
 
   int* d_err = nullptr;    // set by a kernel whose bounded wait expired
   int* h_err = nullptr;    // pinned copy
+  cudaEvent_t ev_err = nullptr;  // after the copy that a GEMM-path call queued
+  bool err_pending = false;      // that copy has not been looked at
   // DOS_INJECT_WAIT_TIMEOUT (tests): the next bulk pass stalls.  1: its copies
   // never arrive, so every block's first wait expires; 2: the copies land, but
   // the odd threads of every block report their first wait as expired; 3 (a
@@ -240,6 +242,8 @@ struct dos_ctx {
     if (gexec) cudaGraphExecDestroy(gexec);
     if (ev_in) cudaEventDestroy(ev_in);
     if (ev_out) cudaEventDestroy(ev_out);
+    if (ev_err) cudaEventDestroy(ev_err);
+    ev_err = nullptr;
     if (gstream) cudaStreamDestroy(gstream);
     gexec = nullptr;
     gstream = nullptr;
@@ -565,6 +569,7 @@ int build(dos_ctx* x, const dos_config* c) {
 // The error flag set by a kernel whose bounded wait expired (tensor-core
 // commit or bulk-copy completion), read after the stream has drained.
 int flag_after_sync(dos_ctx* c) {
+  c->err_pending = false;
   if (*c->h_err) {
     *c->h_err = 0;
     DOS_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream), "error flag");
@@ -584,9 +589,39 @@ int err_check(dos_ctx* c) {
   return flag_after_sync(c);
 }
 
-int gemm_check(dos_ctx* c) { return err_check(c); }
+// The GEMM path's calls do not wait for the GPU: each queues a copy of the
+// error flag behind its kernels (err_post), and the next call on the context
+// that finds the copy done reports it (err_poll), as dos_read_loss does after
+// its own synchronisation.  (A stream synchronisation at the end of every call
+// left the GPU idle while the host prepared the next one.)
+int err_post(dos_ctx* c) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DOS_CUDA(cudaStreamIsCapturing(c->stream, &cs), "capture status");
+  if (cs != cudaStreamCaptureStatusNone) return DOS_OK;  // read by the next call that copies it
+  if (!c->ev_err) DOS_CUDA(cudaEventCreateWithFlags(&c->ev_err, cudaEventDisableTiming), "error event");
+  DOS_CUDA(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "error flag");
+  DOS_CUDA(cudaEventRecord(c->ev_err, c->stream), "error event");
+  c->err_pending = true;
+  return DOS_OK;
+}
+
+int err_poll(dos_ctx* c) {
+  if (!c->err_pending) return DOS_OK;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DOS_CUDA(cudaStreamIsCapturing(c->stream, &cs), "capture status");
+  if (cs != cudaStreamCaptureStatusNone) return DOS_OK;
+  const cudaError_t e = cudaEventQuery(c->ev_err);
+  if (e == cudaErrorNotReady) {
+    (void)cudaGetLastError();
+    return DOS_OK;
+  }
+  DOS_CUDA(e, "error event");
+  return flag_after_sync(c);
+}
 
 int gemm_forward(dos_ctx* c, const float* d_h, float* d_I) {
+  const int late = err_poll(c);
+  if (late) return late;
   dos::GemmPlan& g = c->gp;
   const size_t n2 = (size_t)c->n * c->n, hs2 = (size_t)c->hs * c->hs, f2 = (size_t)c->fov * c->fov;
   c->launches = 0;
@@ -614,10 +649,12 @@ int gemm_forward(dos_ctx* c, const float* d_h, float* d_I) {
     }
     c->launches += 1;
   }
-  return gemm_check(c);
+  return err_post(c);
 }
 
 int gemm_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dLdh) {
+  const int late = err_poll(c);
+  if (late) return late;
   dos::GemmPlan& g = c->gp;
   const size_t n2 = (size_t)c->n * c->n, hs2 = (size_t)c->hs * c->hs, f2 = (size_t)c->fov * c->fov;
   c->launches = 0;
@@ -648,7 +685,7 @@ int gemm_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dL
             dos::launch_grad_reduce(c->partial, d_dLdh, c->gchunks * slices, (size_t)c->K * n2, (size_t)c->K * n2, c->stream),
             "gradient reduction");
   ++c->launches;
-  return gemm_check(c);
+  return err_post(c);
 }
 
 // ------------------------------------------------------------ launch sequences
