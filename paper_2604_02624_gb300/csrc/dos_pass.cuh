@@ -154,7 +154,7 @@ struct Pass {
         const int row = t + T * i;
         r[i] = (i < EF && ok && row >= a.in_r0 && row < a.in_r1) ? src[(size_t)row * M] : czero();
       }
-      LF::template fft<false, NZF, LF::Q, true, PKC>(r, t, z, tw);
+      LF::template fft<false, NZF, LF::Q, false, PKC>(r, t, z, tw);
     }
     const float2* Hw = a.Hq + (size_t)w * a.hs * a.hs;
     const float* Sw = MIS && a.mis.sq ? a.mis.sq + (size_t)w * a.hs * a.hs : nullptr;
@@ -169,7 +169,8 @@ struct Pass {
                          : cmul(shift_phase(signed_bin(k, M), a.mis.sy), shift_phase(signed_bin(cc, M), a.mis.sx)));
       r[i] = ADJ ? cmulc(r[i], hv) : cmul(r[i], hv);
     }
-    LF::template fft<true, LF::P, NOI, true, PKC>(r, t, z, tw);
+    // (the other exchange layout: only what this thread read is overwritten)
+    LF::template fft<true, LF::P, NOI, false, PKC, true>(r, t, z, tw);
     float2* dst = a.S + (size_t)w * a.n * M + cc;
 #pragma unroll
     for (int i = 0; i < E; ++i) {
@@ -208,7 +209,7 @@ struct Pass {
     float2 r[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) r[i] = srow[t + T * i];
-    LF::template fft<true, LF::P, NOI, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<true, LF::P, NOI, false, PKR>(r, t, rc.z, rc.tw);
     const ChanConst cc = a.chan[w];
     const float* hrow = a.h + (size_t)rr * a.n;
     float2* ck = a.ckpt + ((size_t)w * a.n + rr) * a.n;
@@ -223,7 +224,7 @@ struct Pass {
         r[i] = czero();
       }
     }
-    LF::template fft<false, NZF, LF::Q, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<false, NZF, LF::Q, false, PKR, true>(r, t, rc.z, rc.tw);
     if (ok) {
 #pragma unroll
       for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
@@ -249,7 +250,7 @@ struct Pass {
       const int x = t + T * i;
       r[i] = (i < EF && x < a.n) ? cmul(transmission(hrow[x], cc), vrow[x]) : czero();
     }
-    LF::template fft<false, NZF, LF::Q, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<false, NZF, LF::Q, false, PKR>(r, t, rc.z, rc.tw);
     if (ok) {
       float2* srow = a.S + ((size_t)w * a.n + row) * M;
 #pragma unroll
@@ -272,7 +273,7 @@ struct Pass {
     float2 r[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) r[i] = srow[t + T * i];
-    LF::template fft<true, LF::P, NOI, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<true, LF::P, NOI, false, PKR>(r, t, rc.z, rc.tw);
     if (ok) {
       float2* orow = a.o + ((size_t)w * a.fov + fr) * a.fov;
       float* irow = a.I ? a.I + ((size_t)w * a.fov + fr) * a.fov : nullptr;
@@ -304,7 +305,7 @@ struct Pass {
       const int x = t + T * i - a.of;
       r[i] = (i < EF && ok && x >= 0 && x < a.fov) ? cscale(orow[x], 2.0f * grow[x]) : czero();
     }
-    LF::template fft<false, NZF, LF::Q, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<false, NZF, LF::Q, false, PKR>(r, t, rc.z, rc.tw);
     if (ok) {
       float2* srow = a.S + ((size_t)w * a.n + a.of + fr) * M;
 #pragma unroll
@@ -335,7 +336,7 @@ struct Pass {
       float2 r[E];
 #pragma unroll
       for (int i = 0; i < E; ++i) r[i] = srow[t + T * i];
-      LF::template fft<true, LF::P, NOI, true, PKA>(r, t, rc.z, rc.tw);
+      LF::template fft<true, LF::P, NOI, false, PKA>(r, t, rc.z, rc.tw);
       const ChanConst cc = a.chan[w];
 #pragma unroll
       for (int i = 0; i < E; ++i) {
@@ -347,11 +348,15 @@ struct Pass {
         }
       }
       if constexpr (!FIRST) {
-        LF::template fft<false, NZF, LF::Q, true, PKA>(r, t, rc.z, rc.tw);
+        // alternating exchange layouts: no barrier between the two DFTs, nor
+        // between this one and the next channel's
+        LF::template fft<false, NZF, LF::Q, false, PKA, true>(r, t, rc.z, rc.tw);
         if (ok) {
 #pragma unroll
           for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
         }
+      } else {
+        __syncthreads();  // the next channel writes the same layout
       }
     }
     if (ok) {
@@ -379,7 +384,7 @@ struct Pass {
       const int x = t + T * i;
       r[i] = (i < EF && x < a.n) ? frow[x] : czero();
     }
-    LF::template fft<false, NZF, LF::Q, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<false, NZF, LF::Q, false, PKR>(r, t, rc.z, rc.tw);
     if (ok) {
       float2* srow = a.S + ((size_t)w * a.n + row) * M;
 #pragma unroll
@@ -399,7 +404,7 @@ struct Pass {
     float2 r[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) r[i] = srow[t + T * i];
-    LF::template fft<true, LF::P, NOI, true, PKR>(r, t, rc.z, rc.tw);
+    LF::template fft<true, LF::P, NOI, false, PKR>(r, t, rc.z, rc.tw);
     if (ok) {
       float2* frow = a.fout + ((size_t)w * a.n + row) * a.n;
 #pragma unroll
