@@ -121,25 +121,33 @@ __device__ __forceinline__ void split_store8(const Parts& P, size_t at, const fl
   if (P.k > 2) *reinterpret_cast<uint4*>(P.p[2] + at) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
 }
 
+// Accumulator columns an epilogue warp takes at a time.  The spectrum epilogue
+// takes 16, so that the transfer-function values of the next ones can be on
+// their way (in registers) while it works on the current ones: with K = 512 a
+// tile's MMAs take about as long as its epilogue, which then bounds the launch.
+// With the field epilogue's 16-byte stores: 540 -> 498 us per propagation (128
+// channels, 256 x 256, two parts).
+template <int MODE>
+constexpr int epi_cols() { return MODE == GEMM_OUT_SPECTRUM ? 16 : 32; }
+
 // Transfer-function values of accumulator row r = (w, kx), columns cb ..
-// cb+31 = sixteen ky (spectrum epilogue): loaded before the accumulator is,
-// so that the table's latency overlaps the tensor-memory load
-__device__ __forceinline__ void spectrum_h(const GemmArgs& g, int r, int cb, float2 (&hv)[16]) {
+// cb + 15 = eight ky (spectrum epilogue)
+__device__ __forceinline__ void spectrum_h(const GemmArgs& g, int r, int cb, float2 (&hv)[8]) {
   const int m = g.m, w = r / m, kx = r - w * m;
   const int bx = min(kx, m - kx);
   const float2* Hw = g.Hq + (size_t)w * g.hs * g.hs;
   const int ky0 = cb >> 1;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < 8; ++q) {
     const int ky = ky0 + q;
     hv[q] = ky < m ? __ldg(Hw + (size_t)min(ky, m - ky) * g.hs + bx) : make_float2(0.f, 0.f);
   }
 }
 
-// accumulator row r, columns cb .. cb+31 (values v) -> the destination of MODE
-// (hv: the spectrum epilogue's transfer-function values, from spectrum_h)
+// accumulator row r, columns cb .. cb + epi_cols - 1 (values v) -> the
+// destination of MODE (hv: the spectrum epilogue's transfer-function values)
 template <int MODE>
-__device__ __forceinline__ void epilogue(const GemmArgs& g, int r, int cb, const float* v, const float2 (&hv)[16]) {
+__device__ __forceinline__ void epilogue(const GemmArgs& g, int r, int cb, const float* v, const float2 (&hv)[8]) {
   if constexpr (MODE == GEMM_OUT_ROWS) {
     const int k = r >> 1, p = r & 1;
     if (g.nj % 8 == 0) {
@@ -160,37 +168,36 @@ __device__ __forceinline__ void epilogue(const GemmArgs& g, int r, int cb, const
       }
     }
   } else if constexpr (MODE == GEMM_OUT_SPECTRUM) {
-    // row r = (w, kx); columns 2ky + {0, 1}: sixteen spectrum values
+    // row r = (w, kx); columns 2ky + {0, 1}: eight spectrum values
     const int m = g.m, w = r / m, kx = r - w * m;
     const int bx = min(kx, m - kx);
     const float* Sw = g.mis.sq ? g.mis.sq + (size_t)w * g.hs * g.hs : nullptr;
-    const int ky0 = cb >> 1;  // multiple of 16
-    if (ky0 >= m) return;
-    float re[16], im[16];
+    const int ky0 = cb >> 1;  // multiple of 8
+    if (ky0 >= m) return;     // m is a multiple of 8 for every compiled size: whole groups of 8
+    float re[8], im[8];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
+    for (int q = 0; q < 8; ++q) {
       const int ky = ky0 + q;
-      float2 val = make_float2(0.f, 0.f);
-      if (ky < m) {
-        float2 h = hv[q];
-        if (Sw) h = cmul(h, misalign_factor(g.mis, ky, kx, m, Sw[(size_t)min(ky, m - ky) * g.hs + bx]));
-        const float2 b = make_float2(v[2 * q], v[2 * q + 1]);
-        val = g.adj ? cmulc(b, h) : cmul(b, h);
-      }
+      float2 h = hv[q];
+      if (Sw) h = cmul(h, misalign_factor(g.mis, ky, kx, m, Sw[(size_t)min(ky, m - ky) * g.hs + bx]));
+      const float2 b = make_float2(v[2 * q], v[2 * q + 1]);
+      const float2 val = g.adj ? cmulc(b, h) : cmul(b, h);
       re[q] = val.x;
       im[q] = val.y;
     }
-    // m is a multiple of 8 for every compiled size: whole groups of 8
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (ky0 + 8 * q >= m) break;
-      split_store8(g.xo, gemm_tiled((size_t)r, ky0 + 8 * q, g.kpo), re + 8 * q);
-      split_store8(g.xo, gemm_tiled((size_t)r, m + ky0 + 8 * q, g.kpo), im + 8 * q);
-    }
+    split_store8(g.xo, gemm_tiled((size_t)r, ky0, g.kpo), re);
+    split_store8(g.xo, gemm_tiled((size_t)r, m + ky0, g.kpo), im);
   } else {
     // row r = (w, y); columns 2x + {0, 1}: sixteen field values
     const int n = g.n, w = r / n, y = r - w * n;
     const int x0 = cb >> 1;
+    if (!g.o && n % 2 == 0) {
+      float4* row = reinterpret_cast<float4*>(g.fld + (size_t)r * n + x0);  // two values a store
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (x0 + 2 * q < n) row[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      return;
+    }
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const int x = x0 + q;
@@ -208,6 +215,29 @@ __device__ __forceinline__ void epilogue(const GemmArgs& g, int r, int cb, const
       }
     }
   }
+}
+
+// CW columns of this warp's 32 accumulator rows, one row per lane
+template <int CW>
+__device__ __forceinline__ void tmem_load(uint32_t addr, uint32_t (&u)[CW]) {
+  static_assert(CW == 16 || CW == 32, "compiled widths");
+  if constexpr (CW == 32) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+          "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]),
+          "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]),
+          "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
+        : "r"(addr));
+  } else {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+          "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+        : "r"(addr));
+  }
+  asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
 template <int MODE>
@@ -333,36 +363,37 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
     // ---------------------------------------------------------------- epilogue
     const int q = warp & 3;                 // TMEM lane quarter
     const int part = (warp - 2) >> 2;       // column quarter
+    constexpr int CW = epi_cols<MODE>();
     int tc = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tc) {
       const int b = tc & 1;
-      if (!mbar_wait(smem_addr(&sm.acc_full[b]), (uint32_t)((tc >> 1) & 1), abort)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
       int mt, nt;
       tile_of(t, mt, nt);
       const int r = mt * GTM + q * 32 + lane;  // accumulator row of this thread
+      const int cbeg = part * (GTN / 4), cend = cbeg + GTN / 4;
+      float2 hv[8];
+      if constexpr (MODE == GEMM_OUT_SPECTRUM) {
+        if (r < g.vrows) spectrum_h(g, r, nt * GTN + cbeg, hv);  // before the wait for the accumulator
+      }
+      if (!mbar_wait(smem_addr(&sm.acc_full[b]), (uint32_t)((tc >> 1) & 1), abort)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll 1
-      for (int c0 = part * (GTN / 4); c0 < (part + 1) * (GTN / 4); c0 += 32) {
-        float2 hv[16];
+      for (int c0 = cbeg; c0 < cend; c0 += CW) {
+        uint32_t u[CW];
+        tmem_load<CW>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * GTN + c0), u);
+        float2 hn[8];
         if constexpr (MODE == GEMM_OUT_SPECTRUM) {
-          if (r < g.vrows) spectrum_h(g, r, nt * GTN + c0, hv);
+          if (c0 + CW < cend && r < g.vrows) spectrum_h(g, r, nt * GTN + c0 + CW, hn);
         }
-        uint32_t u[32];
-        const uint32_t addr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * GTN + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
-              "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]),
-              "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]),
-              "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
-            : "r"(addr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;");
         if (r < g.vrows) {
-          float v[32];
+          float v[CW];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(u[j]);
+          for (int j = 0; j < CW; ++j) v[j] = __uint_as_float(u[j]);
           epilogue<MODE>(g, r, nt * GTN + c0, v, hv);
+        }
+        if constexpr (MODE == GEMM_OUT_SPECTRUM) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) hv[j] = hn[j];
         }
       }
       // this warp is done with the accumulator
