@@ -140,6 +140,7 @@ struct dos_ctx {
   // [K][N][N] thickness of the last forward that saved checkpoints: dos_backward
   // rebuilds t(h) from it, so the caller passes h once per step
   float* h_fwd = nullptr;
+  bool in_step = false;  // a step is being captured: its gradient reduction keeps the thickness
   dos::LossStats* stats = nullptr;
   double* d_loss = nullptr;
   unsigned* col_work = nullptr;     // items drawn in the running column pass (zero between launches)
@@ -619,6 +620,9 @@ int err_poll(dos_ctx* c) {
   return flag_after_sync(c);
 }
 
+// The thickness that a step's last kernel copies to h_fwd (null: nothing to copy)
+const float* keep_h(const dos_ctx* c, const float* d_h) { return c->in_step && d_h != c->h_fwd ? d_h : nullptr; }
+
 int gemm_forward(dos_ctx* c, const float* d_h, float* d_I) {
   const int late = err_poll(c);
   if (late) return late;
@@ -682,7 +686,8 @@ int gemm_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dL
     }
   }
   DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
-            dos::launch_grad_reduce(c->partial, d_dLdh, c->gchunks * slices, (size_t)c->K * n2, (size_t)c->K * n2, c->stream),
+            dos::launch_grad_reduce(c->partial, d_dLdh, c->gchunks * slices, (size_t)c->K * n2, (size_t)c->K * n2, keep_h(c, d_h), c->h_fwd,
+                                    c->stream),
             "gradient reduction");
   ++c->launches;
   return err_post(c);
@@ -710,11 +715,41 @@ dos::PassArgs range_args(const dos_ctx* c, int w0, int w1) {
   return a;
 }
 
+// Displaced gaps whose length changes: the launches that build the tables of
+// gaps [g0, g1] for nw channels from w0, up to kLongerTables of one slot at a
+// time.
+void build_tables(dos_ctx* c, int g0, int g1, int w0, int nw, int kind, std::vector<Launch>& L) {
+  const size_t hs2 = (size_t)c->hs * c->hs;
+  for (int slot = 0; slot < c->n_slots; ++slot) {
+    dos::LongerTables t = {};
+    const float2* hq = c->Hq + ((size_t)slot * c->nw + w0) * hs2;
+    const float *sq = c->sq + (size_t)w0 * hs2, *sq_lo = c->sq_lo + (size_t)w0 * hs2;
+    const size_t count = (size_t)nw * hs2;
+    auto flush = [&]() {
+      if (t.n == 0) return;
+      L.push_back({kind,
+                   [t, hq, sq, sq_lo, count](cudaStream_t s) {
+                     return dos::launch_longer_tables(t, hq, sq, sq_lo, count, s);
+                   },
+                   "displaced gaps' transfer tables"});
+      t.n = 0;
+    };
+    for (int g = g0; g <= g1; ++g) {
+      const dos::Misalign m = c->gap_mis(g);
+      if (c->gap_slot[g] != slot || m.dz == 0.f) continue;
+      t.out[t.n] = c->hmis + ((size_t)(g % c->mis_tables) * c->nw + w0) * hs2;
+      t.dz[t.n++] = m.dz2;
+      if (t.n == dos::kLongerTables) flush();
+    }
+    flush();
+  }
+}
+
 // The transfer table of gap g for the column passes over a's channels (from
 // w0) and, with displaced layers, what the table does not hold.  A gap whose
-// length changes gets a table of its own; its launch goes to L (kind) first
-// when `build` is set or the table in place is another one.
-void use_gap(dos_ctx* c, dos::PassArgs& a, int g, int w0, bool build, int kind, std::vector<Launch>& L) {
+// length changes has a table of its own; where only one is kept, or the ones in
+// place are another displacement's, its launch goes to L (kind) first.
+void use_gap(dos_ctx* c, dos::PassArgs& a, int g, int w0, int kind, std::vector<Launch>& L) {
   const size_t hs2 = (size_t)c->hs * c->hs;
   a.Hq = c->hq_slot(g) + (size_t)w0 * hs2;
   a.hmap = c->have_tmap ? &c->tmap_H : nullptr;
@@ -725,24 +760,14 @@ void use_gap(dos_ctx* c, dos::PassArgs& a, int g, int w0, bool build, int kind, 
     a.mis.sq = nullptr;
     return;
   }
-  const float *sq = c->sq + (size_t)w0 * hs2, *sq_lo = c->sq_lo + (size_t)w0 * hs2;
   if (c->mis_tables == 0) {
-    a.mis.sq = sq;
+    a.mis.sq = c->sq + (size_t)w0 * hs2;
     a.displaced = true;
     return;
   }
+  if (c->mis_tables == 1 || c->mis_built != c->mis_gen) build_tables(c, g, g, w0, a.nw, kind, L);
   const int slot = g % c->mis_tables;
-  float2* table = c->hmis + ((size_t)slot * c->nw + w0) * hs2;
-  if (build || c->mis_tables == 1 || c->mis_built != c->mis_gen) {
-    const float2 *hq = a.Hq, dz = a.mis.dz2;
-    const size_t count = (size_t)a.nw * hs2;
-    L.push_back({kind,
-                 [table, hq, sq, sq_lo, dz, count](cudaStream_t s) {
-                   return dos::launch_longer_table(table, hq, sq, sq_lo, dz, count, s);
-                 },
-                 "displaced gap's transfer table"});
-  }
-  a.Hq = table;
+  a.Hq = c->hmis + ((size_t)slot * c->nw + w0) * hs2;
   a.hmap = c->have_tmap ? &c->tmap_Hm : nullptr;
   a.hmap_z0 = slot * c->nw + w0;
   a.mis.sq = nullptr;
@@ -755,9 +780,13 @@ std::vector<Launch> forward_launches(dos_ctx* c, const float* d_h, float* d_I, i
   const size_t n2 = (size_t)c->n * c->n;
   std::vector<Launch> L;
   dos::PassArgs a = range_args(c, w0, w1);
+  if (c->mis_on && c->mis_tables > 1) {
+    build_tables(c, 0, c->K, w0, a.nw, DOS_KERNEL_COLUMN_FORWARD, L);
+    c->mis_built = c->mis_gen;
+  }
   if (!c->ckpt1_is_v1) {
     // the aperture field has the separable spectrum Arow[ky] Arow[kx]
-    use_gap(c, a, 0, w0, true, DOS_KERNEL_COLUMN_FORWARD, L);
+    use_gap(c, a, 0, w0, DOS_KERNEL_COLUMN_FORWARD, L);
     a.out_r0 = 0;
     a.out_r1 = c->n;
     L.push_back({DOS_KERNEL_COLUMN_FORWARD, [op, a](cudaStream_t s) { return op->col(a, false, true, s); },
@@ -779,7 +808,7 @@ std::vector<Launch> forward_launches(dos_ctx* c, const float* d_h, float* d_I, i
                    [op, a, brow, sv](cudaStream_t s) { return brow ? op->bulk_row_fwd(a, sv, s) : op->row_fwd(a, sv, s); },
                    "forward row pass"});
     }
-    use_gap(c, a, l, w0, true, DOS_KERNEL_COLUMN_FORWARD, L);
+    use_gap(c, a, l, w0, DOS_KERNEL_COLUMN_FORWARD, L);
     a.in_r0 = 0;
     a.in_r1 = c->n;
     a.out_r0 = l == c->K ? c->of : 0;
@@ -805,7 +834,7 @@ std::vector<Launch> backward_launches(dos_ctx* c, const float* d_h, const float*
   a.dLdI = d_dLdI + (size_t)w0 * c->fov * c->fov;
   L.push_back({DOS_KERNEL_ROW_SEED, [op, a](cudaStream_t s) { return op->row_seed(a, s); }, "adjoint seed row pass"});
   for (int l = c->K; l >= 1; --l) {
-    use_gap(c, a, l, w0, false, DOS_KERNEL_COLUMN_ADJOINT, L);
+    use_gap(c, a, l, w0, DOS_KERNEL_COLUMN_ADJOINT, L);
     a.in_r0 = l == c->K ? c->of : 0;
     a.in_r1 = l == c->K ? c->of + c->fov : c->n;
     a.tmap = !c->have_tmap ? nullptr : l == c->K ? &c->tmap_F : &c->tmap_S;
@@ -851,7 +880,7 @@ int run_launches(dos_ctx* c, const std::vector<Launch>& L) {
 int run_forward(dos_ctx* c, const float* d_h, float* d_I, int save) {
   const size_t n2 = (size_t)c->n * c->n;
   c->launches = 0;
-  if (save && d_h != c->h_fwd)
+  if (save && d_h != c->h_fwd && !c->in_step)
     DOS_CUDA(cudaMemcpyAsync(c->h_fwd, d_h, sizeof(float) * c->K * n2, cudaMemcpyDeviceToDevice, c->stream),
              "saved thickness");
   if (c->path == DOS_PATH_DFT_GEMM || c->path == DOS_PATH_DFT_GEMM_X3) return gemm_forward(c, d_h, d_I);
@@ -895,7 +924,7 @@ int run_forward(dos_ctx* c, const float* d_h, float* d_I, int save) {
   // first gap depends on layer 1's displacement)
   c->ckpt1_is_v1 = c->v1 && !c->mis_on;
   const int rc = run_launches(c, forward_launches(c, d_h, d_I, save, 0, c->nw));
-  c->mis_built = (!rc && c->mis_on && c->mis_tables > 1) ? c->mis_gen : -1;
+  if (rc) c->mis_built = -1;
   return rc;
 }
 
@@ -937,7 +966,7 @@ int run_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dLd
               "fused adjoint sweep");
     DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
               dos::launch_grad_reduce(c->partial, d_dLdh, std::min(c->n_clusters, c->nw), (size_t)c->K * n2,
-                                      (size_t)c->K * n2, c->stream),
+                                      (size_t)c->K * n2, keep_h(c, d_h), c->h_fwd, c->stream),
               "gradient reduction");
     c->launches = 2;
     return DOS_OK;
@@ -945,7 +974,8 @@ int run_backward(dos_ctx* c, const float* d_h, const float* d_dLdI, float* d_dLd
   const int rc = run_launches(c, backward_launches(c, d_h, d_dLdI, 0, c->nw));
   if (rc) return rc;
   DOS_TIMED(c, DOS_KERNEL_GRAD_REDUCE,
-            dos::launch_grad_reduce(c->partial, d_dLdh, c->chunks_of(c->adj_chunk()), (size_t)c->K * n2, n2, c->stream),
+            dos::launch_grad_reduce(c->partial, d_dLdh, c->chunks_of(c->adj_chunk()), (size_t)c->K * n2, n2, keep_h(c, d_h),
+                                    c->h_fwd, c->stream),
             "gradient reduction");
   ++c->launches;
   return DOS_OK;
@@ -1360,6 +1390,7 @@ DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dL
     c->inject_stall = 0;
     cudaStream_t user = c->stream;
     c->stream = c->gstream;
+    c->in_step = true;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
@@ -1375,6 +1406,7 @@ DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dL
       cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
       if (e == cudaSuccess) e = e2;
     }
+    c->in_step = false;
     c->stream = user;
     c->timer.on = timing;
     c->inject_stall = inject;
@@ -1436,7 +1468,8 @@ DOS_API int dos_propagate(dos_ctx* c, int gap, const float* d_in, float* d_out, 
   dos::PassArgs a = range_args(c, 0, c->nw);
   a.fin = reinterpret_cast<const float2*>(d_in);
   a.fout = reinterpret_cast<float2*>(d_out);
-  use_gap(c, a, gap, 0, true, DOS_KERNEL_COLUMN_FORWARD, L);
+  c->mis_built = -1;  // the gap's table is built here
+  use_gap(c, a, gap, 0, DOS_KERNEL_COLUMN_FORWARD, L);
   a.in_r0 = 0;
   a.in_r1 = c->n;
   a.out_r0 = 0;

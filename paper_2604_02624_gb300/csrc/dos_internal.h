@@ -164,10 +164,17 @@ cudaError_t launch_arow(float2* arow, int m, int offset, int width, cudaStream_t
 // sq_lo: what the rounding of sq left (null: not wanted)
 cudaError_t launch_sqtable(float* sq, float* sq_lo, const double* d_lambda, int nw, double n_medium, double pitch, int m, int hs,
                            cudaStream_t s);
-// out = Hq * H(dz) over the count quadrant entries of the channels (from the
-// signed roots, FP32 value and remainder): the table of a gap that is dz longer
-cudaError_t launch_longer_table(float2* out, const float2* Hq, const float* sq, const float* sq_lo, float2 dz,
-                                size_t count, cudaStream_t s);
+// out[i] = Hq * H(dz[i]) over the count quadrant entries of the channels (from
+// the signed roots, FP32 value and remainder): the tables of gaps that are
+// dz[i] longer than Hq's
+constexpr int kLongerTables = 8;
+struct LongerTables {
+  float2* out[kLongerTables];
+  float2 dz[kLongerTables];
+  int n;
+};
+cudaError_t launch_longer_tables(const LongerTables& t, const float2* Hq, const float* sq, const float* sq_lo,
+                                 size_t count, cudaStream_t s);
 cudaError_t launch_twiddles(float2* tw, int P, int Q, int TWP, int m, cudaStream_t s);
 cudaError_t launch_chan(ChanConst* chan, const double* d_lambda, const double* d_nidx,
                         const double* d_kappa, int nw, double n_medium, double h_base,
@@ -190,9 +197,10 @@ cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, 
 // pixels per channel (PSNR mean)
 cudaError_t launch_loss_final(const LossStats* st, int nw, int det2, double norm, int mode,
                               double* d_loss, float* d_psnr, cudaStream_t s);
-// partial: [count / n2][n_parts][n2] -> grad [count] (n2 = count: flat parts)
-cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2,
-                               cudaStream_t s);
+// partial: [count / n2][n_parts][n2] -> grad [count] (n2 = count: flat parts);
+// h not null: also copies h [count] to h_keep
+cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2, const float* h,
+                               float* h_keep, cudaStream_t s);
 
 // Evaluation variants (dos_eval.cu).
 cudaError_t launch_quantize(const float* h, float* q, size_t count, double h_max, int bits, cudaStream_t s);

@@ -225,11 +225,15 @@ cudaError_t launch_loss_final(const LossStats* st, int nw, int fov2, double norm
 // exact rounding errors of its additions, Knuth's two-sum), about 48 bits, and
 // rounded to FP32 once at the end like the FP64 sum before it: GB300 adds and
 // converts FP64 at a small fraction of its FP32 rate, which bound the kernel.
-// A block takes 32 pixels x 8 slices of the parts, eight loads of a slice in
-// flight, so that small layers with many parts still fill the chip.
-// 5 layers of 200 x 200: 92 parts 86 -> 22 us, 86 parts 81 -> 26 us; 3 layers of
-// 64 x 64, 293 parts 57 -> 12 us.
-constexpr int kGradPx = 32, kGradSlices = 8;
+// A block's 256 threads take 32 pixels x 8 slices of the parts, eight loads of a
+// slice in flight, so that small layers with many parts still fill the chip; or
+// 256 pixels each with all of them where the parts are few and the pixels many
+// (below 64 parts a slice is shorter than one unrolled step).
+// 5 layers of 200 x 200: 92 parts 86 -> 22 us, 86 parts 81 -> 26 us, 18 parts with
+// eight slices 18 us, with one 9 us; 3 layers of 64 x 64, 293 parts 57 -> 12 us.
+// A step's thickness is copied here too (h not null), which saves the step a
+// copy of its own.
+constexpr int kGradThreads = 256;
 
 // (s, e) += x with s + e kept exact up to the rounding of e
 __device__ __forceinline__ void pair_add(float& s, float& e, float x) {
@@ -239,14 +243,17 @@ __device__ __forceinline__ void pair_add(float& s, float& e, float x) {
   s = t;
 }
 
-__global__ void __launch_bounds__(kGradPx * kGradSlices) k_grad_reduce(const float* __restrict__ partial,
-                                                                       float* __restrict__ grad, int n_parts,
-                                                                       size_t count, size_t n2) {
-  __shared__ float2 sh[kGradSlices][kGradPx];
+template <int SLICES>
+__global__ void __launch_bounds__(kGradThreads) k_grad_reduce(const float* __restrict__ partial,
+                                                              float* __restrict__ grad, int n_parts, size_t count,
+                                                              size_t n2, const float* __restrict__ h,
+                                                              float* __restrict__ h_keep) {
+  constexpr int PX = kGradThreads / SLICES;
+  __shared__ float2 sh[SLICES][PX];
   pdl_wait();
-  const int lane = threadIdx.x % kGradPx, slice = threadIdx.x / kGradPx;
-  const size_t g = (size_t)blockIdx.x * kGradPx + lane;
-  const int per = (n_parts + kGradSlices - 1) / kGradSlices;
+  const int lane = threadIdx.x % PX, slice = threadIdx.x / PX;
+  const size_t g = (size_t)blockIdx.x * PX + lane;
+  const int per = (n_parts + SLICES - 1) / SLICES;
   const int c0 = min(slice * per, n_parts), c1 = min(c0 + per, n_parts);
   float s = 0.f, e = 0.f;
   if (g < count) {
@@ -262,23 +269,28 @@ __global__ void __launch_bounds__(kGradPx * kGradSlices) k_grad_reduce(const flo
     }
     for (; c < c1; ++c, p += n2) pair_add(s, e, __ldcs(p));
   }
-  sh[slice][lane] = make_float2(s, e);
-  __syncthreads();
+  if constexpr (SLICES > 1) {
+    sh[slice][lane] = make_float2(s, e);
+    __syncthreads();
+  }
   if (slice != 0 || g >= count) return;
 #pragma unroll
-  for (int q = 1; q < kGradSlices; ++q) {
+  for (int q = 1; q < SLICES; ++q) {
     const float2 v = sh[q][lane];
     pair_add(s, e, v.x);
     e = __fadd_rn(e, v.y);
   }
+  if (h) h_keep[g] = h[g];
   // an infinite sum has no rounding error to add (inf - inf)
   grad[g] = isinf(s) ? s : s + e;
 }
 
-cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2,
-                               cudaStream_t s) {
-  const unsigned blocks = (unsigned)((count + kGradPx - 1) / kGradPx);
-  return launch_next(k_grad_reduce, dim3(blocks), kGradPx * kGradSlices, 0, s, partial, grad, n_parts, count, n2);
+cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2, const float* h,
+                               float* h_keep, cudaStream_t s) {
+  const bool one = n_parts < 64 && count >= (size_t)64 * kGradThreads;
+  const size_t px = one ? kGradThreads : kGradThreads / 8;
+  return launch_next(one ? k_grad_reduce<1> : k_grad_reduce<8>, dim3((unsigned)((count + px - 1) / px)), kGradThreads, 0,
+                     s, partial, grad, n_parts, count, n2, h, h_keep);
 }
 
 }  // namespace dos

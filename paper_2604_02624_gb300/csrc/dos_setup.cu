@@ -77,14 +77,16 @@ cudaError_t launch_sqtable(float* sq, float* sq_lo, const double* d_lambda, int 
   return cudaGetLastError();
 }
 
-// Transfer table of a gap lengthened by dz: Hq times exp(2 pi j dz sqrt(q)), or
+// Transfer tables of gaps lengthened by dz: Hq times exp(2 pi j dz sqrt(q)), or
 // exp(-2 pi dz sqrt(-q)) for evanescent bins, from the signed roots.  One pass
-// over the quadrant, 24 bytes an entry, bound by memory.  A column pass reads
-// every quadrant entry at four bins, and formed the factor there: a sine, a
-// cosine and a gathered root for each.  256 channels, M = 400, both column
-// passes of a gap: 524 -> 230 us, and 55 us for its table.  Root and length as
-// FP32 pairs: a root rounded to FP32 turns the phase by up to 2e-7 of a
-// wavelength per wavelength of dz.
+// over the quadrant for up to eight gaps of one table slot, 16 bytes read and 8
+// written a gap for each entry, bound by memory (a launch per gap, 24 bytes an
+// entry each, took 55 us a gap at 256 channels, M = 400: 330 us for six; now
+// 185 us).  A column pass reads every quadrant entry at four bins, and
+// formed the factor there: a sine, a cosine and a gathered root for each; both
+// column passes of a gap then took 524 us, 230 us with the table.
+// Root and length as FP32 pairs: a root rounded to FP32 turns the phase by up to
+// 2e-7 of a wavelength per wavelength of dz.
 __device__ __forceinline__ float2 longer(float2 h, float sq, float sq_lo, float2 dz) {
   float amp = 1.0f, ph = 0.0f;
   if (sq >= 0.0f) ph = fmaf(dz.x, sq_lo, cycles(sq, dz));
@@ -94,26 +96,29 @@ __device__ __forceinline__ float2 longer(float2 h, float sq, float sq_lo, float2
   const float re = amp * cs, im = amp * sn;
   return make_float2(fmaf(h.x, re, -h.y * im), fmaf(h.x, im, h.y * re));
 }
-__global__ void __launch_bounds__(256) k_longer_table(float4* __restrict__ out, const float4* __restrict__ Hq,
-                                                      const float2* __restrict__ sq, const float2* __restrict__ sq_lo,
-                                                      float2 dz, size_t pairs) {
+__global__ void __launch_bounds__(256) k_longer_tables(LongerTables t, const float4* __restrict__ Hq,
+                                                       const float2* __restrict__ sq,
+                                                       const float2* __restrict__ sq_lo, size_t pairs) {
   pdl_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= pairs) return;
   const float4 h = Hq[i];
   const float2 r = sq[i], l = sq_lo[i];
-  const float2 a = longer(make_float2(h.x, h.y), r.x, l.x, dz), b = longer(make_float2(h.z, h.w), r.y, l.y, dz);
-  out[i] = make_float4(a.x, a.y, b.x, b.y);
+  for (int g = 0; g < t.n; ++g) {
+    const float2 dz = t.dz[g];
+    const float2 a = longer(make_float2(h.x, h.y), r.x, l.x, dz), b = longer(make_float2(h.z, h.w), r.y, l.y, dz);
+    reinterpret_cast<float4*>(t.out[g])[i] = make_float4(a.x, a.y, b.x, b.y);
+  }
 }
 
 // count is even (a channel's quadrant has hs^2 entries, hs = M/2 + 2 even) and
 // the tables start 16-byte aligned
-cudaError_t launch_longer_table(float2* out, const float2* Hq, const float* sq, const float* sq_lo, float2 dz,
-                                size_t count, cudaStream_t s) {
+cudaError_t launch_longer_tables(const LongerTables& t, const float2* Hq, const float* sq, const float* sq_lo,
+                                 size_t count, cudaStream_t s) {
   const size_t pairs = count / 2;
-  return launch_next(k_longer_table, dim3((unsigned)((pairs + 255) / 256)), 256, 0, s,
-                     reinterpret_cast<float4*>(out), reinterpret_cast<const float4*>(Hq),
-                     reinterpret_cast<const float2*>(sq), reinterpret_cast<const float2*>(sq_lo), dz, pairs);
+  return launch_next(k_longer_tables, dim3((unsigned)((pairs + 255) / 256)), 256, 0, s, t,
+                     reinterpret_cast<const float4*>(Hq), reinterpret_cast<const float2*>(sq),
+                     reinterpret_cast<const float2*>(sq_lo), pairs);
 }
 
 // Arow[k] = sum_{x = offset}^{offset + width - 1} exp(-2 pi j k x / m)
