@@ -80,6 +80,11 @@ struct Fused {
 
   // H(|ky|, |kx|) for the thread's frequencies k = t + T*i of column cc:
   // |k| = k below M/2 and M - k above, both affine in i at compile time.
+  // MIS: displaced layers (kernels of their own: the displacement's phase per
+  // element would more than double the column phase's code, which a short sweep
+  // fetches cold: 4 channels of 64 x 64, forward and adjoint sweep 29 -> 25 us
+  // of the 31 us step before).
+  template <bool MIS>
   __device__ static __forceinline__ void load_h(float2 (&hreg)[E], const float2* __restrict__ Hw, int hs, int t,
                                                 int cc, const float* __restrict__ Sw, const Misalign& mg) {
     const int bc = min(cc, M - cc);
@@ -88,7 +93,7 @@ struct Fused {
 #pragma unroll
     for (int i = 0; i < E; ++i)
       hreg[i] = i < EH ? __ldg(lo + (size_t)T * i * hs) : __ldg(hi - (size_t)T * i * hs);
-    if (Sw) {
+    if constexpr (MIS) {
       const float* slo = Sw + (size_t)t * hs + bc;
       const float* shi = Sw + (size_t)(M - t) * hs + bc;
 #pragma unroll
@@ -130,7 +135,7 @@ struct Fused {
   // ------------------------------------------------------------- column phase
   // Columns [rank*MC, rank*MC + MC) of the plane; rows [in_r0, in_r1) are read
   // (others are zero), rows [out_r0, out_r1) are written back.
-  template <bool ADJ, bool APERTURE>
+  template <bool ADJ, bool APERTURE, bool MIS>
   __device__ static void col_phase(const cg::cluster_group& cl, const Sm& s, const float2* __restrict__ Hw,
                                    const float2* __restrict__ arow, int n, int hs, int in_r0, int in_r1,
                                    int out_r0, int out_r1, const float* __restrict__ Sw, const Misalign& mg) {
@@ -167,7 +172,7 @@ struct Fused {
       const int cc = ok ? c : c0;
       float2 r[E];
       float2 hreg[E];
-      if constexpr (kPrefetchH) load_h(hreg, Hw, hs, t, cc, Sw, mg);
+      if constexpr (kPrefetchH) load_h<MIS>(hreg, Hw, hs, t, cc, Sw, mg);
       if constexpr (APERTURE) {
         const float2 ac = arow[cc];
 #pragma unroll
@@ -178,7 +183,7 @@ struct Fused {
         if (cb + LINES < MC) fetch(cb + LINES, rnext);
         LF::template fft<false, PH, LF::Q, true, FPK>(r, t, z, s.tw);
       }
-      if constexpr (!kPrefetchH) load_h(hreg, Hw, hs, t, cc, Sw, mg);
+      if constexpr (!kPrefetchH) load_h<MIS>(hreg, Hw, hs, t, cc, Sw, mg);
 #pragma unroll
       for (int i = 0; i < E; ++i) r[i] = ADJ ? cmulc(r[i], hreg[i]) : cmul(r[i], hreg[i]);
       LF::template fft<true, LF::P, QH, true, FPK>(r, t, z, s.tw);
@@ -410,21 +415,22 @@ struct Fused {
   }
 
   // --------------------------------------------------------------- sweeps
+  template <bool MIS>
   __device__ static void forward(const FusedArgs& a) {
     cg::cluster_group cl = cg::this_cluster();
     const Sm s = carve(a);
     const int cid = blockIdx.x / C;
     const int ncl = gridDim.x / C;
     for (int w = cid; w < a.nw; w += ncl) {
-      if (!a.v1) {  // gap 0 from the aperture (the table is not used with displaced layers)
-        col_phase<false, true>(cl, s, table(a, 0, w), a.arow, a.n, a.hs, 0, 0, 0, a.n, sqt(a, w), mis(a, 0));
+      if constexpr (MIS) {  // gap 0 from the aperture (aligned layers start from the table v1)
+        col_phase<false, true, MIS>(cl, s, table(a, 0, w), a.arow, a.n, a.hs, 0, 0, 0, a.n, sqt(a, w), mis(a, 0));
         cl.sync();
       }
       for (int layer = 0; layer < a.K; ++layer) {
         row_fwd_phase(cl, s, a, layer, w);
         cl.sync();
         const bool lastgap = layer == a.K - 1;
-        col_phase<false, false>(cl, s, table(a, layer + 1, w), a.arow, a.n, a.hs, 0, a.n,
+        col_phase<false, false, MIS>(cl, s, table(a, layer + 1, w), a.arow, a.n, a.hs, 0, a.n,
                                 lastgap ? a.of : 0, lastgap ? a.of + a.fov : a.n, sqt(a, w), mis(a, layer + 1));
         cl.sync();
       }
@@ -433,6 +439,7 @@ struct Fused {
     }
   }
 
+  template <bool MIS>
   __device__ static void adjoint(const FusedArgs& a) {
     cg::cluster_group cl = cg::this_cluster();
     const Sm s = carve(a);
@@ -444,7 +451,7 @@ struct Fused {
       cl.sync();
       for (int layer = a.K - 1; layer >= 0; --layer) {
         const bool lastgap = layer == a.K - 1;
-        col_phase<true, false>(cl, s, table(a, layer + 1, w), a.arow, a.n, a.hs,
+        col_phase<true, false, MIS>(cl, s, table(a, layer + 1, w), a.arow, a.n, a.hs,
                                lastgap ? a.of : 0, lastgap ? a.of + a.fov : a.n, 0, a.n, sqt(a, w), mis(a, layer + 1));
         cl.sync();
         row_adj_phase(cl, s, a, layer, w, part, w == cid);
@@ -454,13 +461,13 @@ struct Fused {
   }
 };
 
-template <class LF, int C, int LINES>
+template <class LF, int C, int LINES, bool MIS>
 __global__ void __launch_bounds__(LINES * LF::T, 1) k_fused_fwd(FusedArgs a) {
-  Fused<LF, C, LINES>::forward(a);
+  Fused<LF, C, LINES>::template forward<MIS>(a);
 }
-template <class LF, int C, int LINES>
+template <class LF, int C, int LINES, bool MIS>
 __global__ void __launch_bounds__(LINES * LF::T, 1) k_fused_adj(FusedArgs a) {
-  Fused<LF, C, LINES>::adjoint(a);
+  Fused<LF, C, LINES>::template adjoint<MIS>(a);
 }
 
 // Host side of one fused configuration.
@@ -500,14 +507,14 @@ struct FusedLaunch {
   static int max_clusters(int n) {
     const size_t sm = smem(n);
     if (sm > 227 * 1024) return 0;
-    if (prep(k_fused_fwd<LF, C, LINES>, sm) != cudaSuccess) {
+    if (prep(k_fused_fwd<LF, C, LINES, false>, sm) != cudaSuccess) {
       (void)cudaGetLastError();
       return 0;
     }
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg = config(1, sm, nullptr, at);
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, k_fused_fwd<LF, C, LINES>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nc, k_fused_fwd<LF, C, LINES, false>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       return 0;
     }
@@ -517,14 +524,10 @@ struct FusedLaunch {
     const size_t sm = smem(a.n);
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg = config(n_clusters, sm, s, at);
-    cudaError_t e;
-    if (adjoint) {
-      e = prep(k_fused_adj<LF, C, LINES>, sm);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_fused_adj<LF, C, LINES>, a);
-    } else {
-      e = prep(k_fused_fwd<LF, C, LINES>, sm);
-      if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_fused_fwd<LF, C, LINES>, a);
-    }
+    auto kernel = a.sq ? (adjoint ? k_fused_adj<LF, C, LINES, true> : k_fused_fwd<LF, C, LINES, true>)
+                       : (adjoint ? k_fused_adj<LF, C, LINES, false> : k_fused_fwd<LF, C, LINES, false>);
+    cudaError_t e = prep(kernel, sm);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kernel, a);
     return e;
   }
   static const FusedOps* ops() {

@@ -27,11 +27,12 @@ namespace dos {
 // sin and cos of 2 pi f for |f| <= 1/2 (a thickness phase in cycles), FP32.
 // 4 f = k + r with k the nearest integer (the low bits of 4 f + 1.5 2^23, whose
 // ulp is 1) and |r| <= 1/2 exact; sin and cos of r pi/2 are polynomials in r^2
-// fitted here for the least largest error (3.2e-9 and 5e-11 before rounding),
-// pi/2 held in two parts, and k turns them by quarters.  Non-finite f gives NaN.
+// fitted here for the least largest error (3.2e-9 and 4e-10 before rounding;
+// the sine's pi/2 is held in two parts, the cosine fitted around its rounded
+// first coefficient, so that neither is biased), and k turns them by quarters.  Non-finite f gives NaN.
 // Rounded results, |r| <= 1/2: sine within 4.4e-8 of the exact value (root mean
 // square 1.15e-8; the nearest FP32 numbers: 3.0e-8 and 1.13e-8), cosine within
-// 5.8e-8 (1.81e-8; 3.0e-8 and 1.72e-8).
+// 5.2e-8 (1.79e-8; 3.0e-8 and 1.72e-8).
 // The library's sincospif does the same work on any argument, with conversions
 // and roundings on the quarter-rate unit.  With it, and one complex product
 // more in the adjoint pixel, 4096 x 200 forward / adjoint row launches took 0.942
@@ -45,8 +46,8 @@ __device__ __forceinline__ void sincos_turns(float f, float* s, float* c) {
   p = __fmaf_rn(u, p, -0.6459635f);
   p = __fmaf_rn(u, p, -4.8539483e-8f);
   p = __fmaf_rn(r, 1.5707963705f, r * p);
-  float q = __fmaf_rn(u, 0.0009040216f, -0.020860288f);
-  q = __fmaf_rn(u, q, 0.25366924f);
+  float q = __fmaf_rn(u, 0.0008929509f, -0.02085506f);
+  q = __fmaf_rn(u, q, 0.25366852f);
   q = __fmaf_rn(u, q, -1.2337005f);
   q = __fmaf_rn(u, q, 1.0f);
   const int k = __float_as_int(b);
