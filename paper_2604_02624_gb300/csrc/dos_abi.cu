@@ -13,6 +13,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -135,6 +136,7 @@ struct dos_ctx {
   float2* v1 = nullptr;
   bool ckpt1_is_v1 = false;  // the last multi-pass forward started from v1
   int step_launches = 0;     // kernels in the captured step graph
+  bool step_from_v1 = false; // its forward started from v1
   dos::ChanConst* chan = nullptr;
   float* partial = nullptr;
   // [K][N][N] thickness of the last forward that saved checkpoints: dos_backward
@@ -178,6 +180,12 @@ struct dos_ctx {
   std::vector<int> fcand_clusters;
   const dos::FusedOps* fops = nullptr;
   int n_clusters = 0;
+  // Implementations (choices of the autotuner) of the stream calls and of the
+  // captured step, and the one that the last forward ran, whose fields and
+  // flags dos_backward continues from.  bulk / path / fops / n_clusters are
+  // those of the choice in use (use_choice).
+  static constexpr int kFixed = 1 << 30;  // the GEMM paths: nothing to choose
+  int call_choice = kFixed, step_choice = kFixed, fwd_choice = kFixed;
   std::string describe;
   // graph of one design step (dos_step)
   cudaStream_t gstream = nullptr;
@@ -1029,29 +1037,54 @@ void set_choice(dos_ctx* x, int idx) {
   }
 }
 
+// Switches the context to a choice unless it has none (the GEMM paths).
+void use_choice(dos_ctx* x, int idx) {
+  if (idx != dos_ctx::kFixed) set_choice(x, idx);
+}
+
+// The context's choices, and the one in use: the stream calls'.
+void keep_choices(dos_ctx* x, int call, int step) {
+  x->call_choice = x->fwd_choice = call;
+  x->step_choice = step;
+  set_choice(x, call);
+}
+
 std::string choice_detail(const dos_ctx* x, int idx) {
   std::ostringstream d;
   d << "path=" << choice_name(x, idx);
   if (idx >= 0)
     d << " threads=" << x->fops->threads << " clusters=" << x->n_clusters << " smem=" << x->fops->smem(x->n);
+  if (x->step_choice != idx) d << " step=" << choice_name(x, x->step_choice);
   return d.str();
 }
+
+// The step replays a graph, so its choice is the one whose kernels take the
+// least time.  The stream calls also cost the host their launches, and their
+// callers do host work of their own between them (an objective in PyTorch is
+// ten and more operations of some 5 us): their choice is the one with the
+// shortest pass beside kCallerMs of that, the longer of the GPU's time and the
+// host's.  It differs where a whole pass takes less than that: 6 channels of
+// 200 x 200, 12 calls and 55 us on the GPU with the multi-pass kernels, 4 and 78 us
+// cluster-resident; under autograd (host-bound) 446 against 406 us a pass.
+constexpr float kCallerMs = 0.06f;
 
 // time forward(save) + backward of the current choice on zero thickness / zero
 // seed; with kind_ms, one more forward + backward with per-launch events gives
 // the time of every kernel kind
-int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, float* ms_out,
+int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, float* ms_out, float* host_ms_out,
                 double* kind_ms = nullptr) {
   int rc;
   if ((rc = run_forward(x, h0, nullptr, 1)) || (rc = run_backward(x, h0, g0, d0))) return rc;
   cudaEvent_t a, b;
   DOS_CUDA(cudaEventCreate(&a), "tune event");
   DOS_CUDA(cudaEventCreate(&b), "tune event");
-  float best = 1e30f;
+  float best = 1e30f, host = 1e30f;
   for (int rep = 0; rep < 2; ++rep) {
+    const auto t0 = std::chrono::steady_clock::now();
     cudaEventRecord(a, x->stream);
     if ((rc = run_forward(x, h0, nullptr, 1)) || (rc = run_backward(x, h0, g0, d0))) break;
     cudaEventRecord(b, x->stream);
+    host = std::min(host, std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count());
     cudaError_t e = cudaEventSynchronize(b);
     float t = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&t, a, b);
@@ -1084,6 +1117,7 @@ int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, float* 
   }
   if (!rc) rc = err_check(x);
   *ms_out = best;
+  *host_ms_out = host;
   return rc;
 }
 
@@ -1099,12 +1133,12 @@ int choose_path(dos_ctx* x, int requested) {
     return DOS_OK;
   }
   if (requested == DOS_PATH_MULTIPASS) {
-    set_choice(x, kPlain);
+    keep_choices(x, kPlain, kPlain);
     x->describe = "path=multipass (requested)";
     return DOS_OK;
   }
   if (requested == DOS_PATH_MULTIPASS_BULK) {
-    set_choice(x, kBulk);
+    keep_choices(x, kBulk, kBulk);
     x->describe = "path=multipass:bulk (requested)";
     return DOS_OK;
   }
@@ -1119,7 +1153,7 @@ int choose_path(dos_ctx* x, int requested) {
   }
   for (int i = 0; i < (int)x->fcands.size(); ++i) cands.push_back(i);
   if (cands.size() == 1) {
-    set_choice(x, cands[0]);
+    keep_choices(x, cands[0], cands[0]);
     x->describe = choice_detail(x, cands[0]) + " (only candidate)";
     return DOS_OK;
   }
@@ -1137,7 +1171,7 @@ int choose_path(dos_ctx* x, int requested) {
   const char* force = std::getenv("DOS_FORCE_CONFIG");
   int named = 0;
   if (force && *force && by_name(force, &named)) {
-    set_choice(x, named);
+    keep_choices(x, named, named);
     x->describe = choice_detail(x, named) + " (DOS_FORCE_CONFIG)";
     return DOS_OK;
   }
@@ -1149,9 +1183,13 @@ int choose_path(dos_ctx* x, int requested) {
     std::string line;
     while (std::getline(in, line)) {
       if (line.compare(0, key.size() + 1, key + "\t") != 0) continue;
+      // the stream calls' choice, and after a tab the step's where it differs
       const std::string v = line.substr(key.size() + 1);
-      if (by_name(v, &named)) {
-        set_choice(x, named);
+      const size_t tab = v.find('\t');
+      int step = 0;
+      if (by_name(v.substr(0, tab), &named) &&
+          (tab == std::string::npos ? (step = named, true) : by_name(v.substr(tab + 1), &step))) {
+        keep_choices(x, named, step);
         x->describe = choice_detail(x, named) + " (tuning cache)";
         return DOS_OK;
       }
@@ -1166,8 +1204,8 @@ int choose_path(dos_ctx* x, int requested) {
   if (e == cudaSuccess) e = cudaMemsetAsync(g0, 0, sizeof(float) * (size_t)x->nw * x->fov * x->fov, x->stream);
   int rc = DOS_OK;
   if (e != cudaSuccess) rc = fail(DOS_ERR_CUDA, std::string("autotune buffers: ") + cudaGetErrorString(e));
-  int best = cands[0];
-  float best_ms = 1e30f;
+  int best = cands[0], best_call = cands[0];
+  float best_ms = 1e30f, best_call_ms = 1e30f;
   std::ostringstream d;
   d << "tuned (fwd+bwd ms):";
   // per-kind times of the plain and the bulk-prefetching multi-pass kernels;
@@ -1176,8 +1214,8 @@ int choose_path(dos_ctx* x, int requested) {
   for (size_t k = 0; rc == DOS_OK && k < cands.size(); ++k) {
     const int idx = cands[k];
     set_choice(x, idx);
-    float ms = 0.f;
-    rc = time_choice(x, h0, g0, d0, &ms, idx == kPlain ? kind_plain : idx == kBulk ? kind_bulk : nullptr);
+    float ms = 0.f, host_ms = 0.f;
+    rc = time_choice(x, h0, g0, d0, &ms, &host_ms, idx == kPlain ? kind_plain : idx == kBulk ? kind_bulk : nullptr);
     if (rc) break;
     if (idx == kBulk && requested == DOS_PATH_AUTO) {
       unsigned mix = 0;
@@ -1195,16 +1233,23 @@ int choose_path(dos_ctx* x, int requested) {
       best_ms = ms;
       best = idx;
     }
+    const float call_ms = std::max(ms, host_ms + kCallerMs);
+    if (call_ms < best_call_ms || (call_ms == best_call_ms && best == idx)) {
+      best_call_ms = call_ms;
+      best_call = idx;
+    }
   }
   cudaFree(h0);
   cudaFree(g0);
   cudaFree(d0);
   if (rc) return rc;
-  set_choice(x, best);
-  x->describe = choice_detail(x, best) + " | " + d.str();
+  keep_choices(x, best_call, best);
+  x->describe = choice_detail(x, best_call) + " | " + d.str();
   if (cache && *cache) {
     std::ofstream out(cache, std::ios::app);
-    out << key << "\t" << choice_name(x, best) << "\n";
+    out << key << "\t" << choice_name(x, best_call);
+    if (best != best_call) out << "\t" << choice_name(x, best);
+    out << "\n";
   }
   return DOS_OK;
 }
@@ -1264,6 +1309,7 @@ DOS_API int dos_forward(dos_ctx* c, const float* d_h, float* d_I, int save_for_b
   if (rc) return rc;
   if (!d_h) return fail(DOS_ERR_ARG, "d_h is NULL");
   c->have_fwd = c->have_ckpt = c->have_loss = false;
+  use_choice(c, c->fwd_choice = c->call_choice);
   if ((rc = run_forward(c, d_h, d_I, save_for_backward))) return rc;
   c->have_fwd = true;
   c->have_ckpt = save_for_backward != 0;
@@ -1302,7 +1348,7 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
     const size_t count = (size_t)c->nw * c->hs * c->hs;
     if ((rc = c->alloc(&c->sq, count, "root table"))) return rc;
     // the column passes' tables: where they do not fit, the plain kernel does without
-    if ((c->path == DOS_PATH_MULTIPASS || c->path == DOS_PATH_MULTIPASS_BULK) &&
+    if ((c->call_choice < 0 || c->step_choice < 0) &&  // the multi-pass choices
         c->alloc(&c->sq_lo, count, "root table") == DOS_OK) {
       for (int tables : {c->K + 1, 1}) {
         if (c->alloc(&c->hmis, tables * count, "displaced transfer tables") != DOS_OK) continue;
@@ -1365,7 +1411,10 @@ DOS_API int dos_backward(dos_ctx* c, const float* d_dLdI, float* d_dLdh) {
   if (rc) return rc;
   if (!c->have_ckpt) return fail(DOS_ERR_STATE, "dos_backward needs dos_forward(save_for_backward=1) first");
   if (!d_dLdI || !d_dLdh) return fail(DOS_ERR_ARG, "d_dLdI and d_dLdh are required");
-  return run_backward(c, c->h_fwd, d_dLdI, d_dLdh);
+  use_choice(c, c->fwd_choice);
+  rc = run_backward(c, c->h_fwd, d_dLdI, d_dLdh);
+  use_choice(c, c->call_choice);
+  return rc;
 }
 
 DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dLdh, float* d_I, float* d_psnr,
@@ -1391,6 +1440,7 @@ DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dL
     cudaStream_t user = c->stream;
     c->stream = c->gstream;
     c->in_step = true;
+    use_choice(c, c->step_choice);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
@@ -1403,10 +1453,12 @@ DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dL
                              c->d_loss, c->loss_ticket, c->gstream);
       if (!rc && e == cudaSuccess) rc = run_backward(c, d_h, c->dLdI_step, d_dLdh);
       if (!rc) c->step_launches = fwd_launches + 1 + c->launches;
+      c->step_from_v1 = c->ckpt1_is_v1;
       cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
       if (e == cudaSuccess) e = e2;
     }
     c->in_step = false;
+    use_choice(c, c->call_choice);
     c->stream = user;
     c->timer.on = timing;
     c->inject_stall = inject;
@@ -1426,6 +1478,8 @@ DOS_API int dos_step(dos_ctx* c, const float* d_h, const float* d_T, float* d_dL
   DOS_CUDA(cudaEventRecord(c->ev_out, c->gstream), "step order");
   DOS_CUDA(cudaStreamWaitEvent(c->stream, c->ev_out, 0), "step order");
   c->launches = c->step_launches;
+  c->fwd_choice = c->step_choice;
+  c->ckpt1_is_v1 = c->step_from_v1;
   c->have_fwd = c->have_ckpt = c->have_loss = true;
   if (h_loss) return dos_read_loss(c, h_loss);
   return DOS_OK;
@@ -1449,8 +1503,7 @@ DOS_API int dos_layer_field(dos_ctx* c, int layer, float* d_v) {
   if (layer < 1 || layer > c->K) return fail(DOS_ERR_ARG, "layer must be in [1, n_layers]");
   if (!d_v) return fail(DOS_ERR_ARG, "d_v is NULL");
   const size_t n2 = (size_t)c->n * c->n;
-  const bool table = layer == 1 && c->ckpt1_is_v1 &&
-                     (c->path == DOS_PATH_MULTIPASS || c->path == DOS_PATH_MULTIPASS_BULK || c->path == DOS_PATH_FUSED);
+  const bool table = layer == 1 && c->ckpt1_is_v1;  // never on the GEMM paths
   DOS_CUDA(cudaMemcpyAsync(d_v, table ? c->v1 : c->ckpt + (size_t)(layer - 1) * c->nw * n2,
                            sizeof(float2) * c->nw * n2, cudaMemcpyDeviceToDevice, c->stream),
            "copy layer field");
@@ -1476,7 +1529,9 @@ DOS_API int dos_propagate(dos_ctx* c, int gap, const float* d_in, float* d_out, 
   a.out_r1 = c->n;
   for (const Launch& l : L) DOS_CUDA(l.go(c->stream), l.what);
   DOS_CUDA(op->row_in(a, c->stream), "propagate row pass");
-  if (c->bulk & kBulkCol) DOS_CUDA(op->bulk_col(a, adjoint != 0, c->stream), "propagate column pass");
+  // the prefetching column kernel where either of the context's choices runs it
+  const unsigned bulk = c->call_choice < 0 ? choice_mask(c->call_choice) : c->step_choice < 0 ? choice_mask(c->step_choice) : 0;
+  if (bulk & kBulkCol) DOS_CUDA(op->bulk_col(a, adjoint != 0, c->stream), "propagate column pass");
   else DOS_CUDA(op->col(a, adjoint != 0, false, c->stream), "propagate column pass");
   DOS_CUDA(op->row_back(a, c->stream), "propagate back row pass");
   c->launches = 3 + (int)L.size();
