@@ -14,7 +14,7 @@
 
 namespace dos {
 
-constexpr int kRedThreads = 256;
+constexpr int kRedThreads = 256;  // threads of a reducing block (k_loss also has a smaller one)
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
   sh[threadIdx.x] = v;
@@ -40,15 +40,16 @@ __device__ __forceinline__ float detector(const float2* ow, int fov, int b, int 
   return s;
 }
 
-// Fixed-order FP64 total of the block's kRedThreads FP32 partials, by one
-// warp: lane l adds eight of them, a shuffle tree the 32 lanes.  The total is
+// Fixed-order FP64 total of the block's NT FP32 partials, by one warp: lane l
+// adds NT / 32 of them, a shuffle tree the 32 lanes.  The total is
 // valid in lane 0.  (An FP64 addition occupies the SM's FP64 pipe for many
 // cycles: one warp issues 13 of them here where a block-wide tree in shared
 // memory issues them from every warp and takes eight barriers per sum.)
+template <int NT>
 __device__ __forceinline__ double warp_total(const float* part, int lane) {
   double v = 0.0;
 #pragma unroll
-  for (int i = 0; i < kRedThreads / 32; ++i) v += (double)part[lane + 32 * i];
+  for (int i = 0; i < NT / 32; ++i) v += (double)part[lane + 32 * i];
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
   return v;
@@ -75,6 +76,10 @@ __device__ __forceinline__ float ten_log10(double x) {
 // between the two loops (16 KB: five blocks and more per SM); above it the
 // second loop forms them again.
 constexpr int kLossKeep = 4096;
+// Up to this many detector pixels a channel gets a block of 128 threads, so that
+// twice as many channels are in flight (a thread then adds at most ten terms,
+// as one of 256 does at 50 x 50).
+constexpr int kLossSmall = 1280;
 
 // One block per channel: sum (D-T)^2, sigma = sum D T / sum D^2, sum (sigma D
 // - T)^2, the PSNR (psnr not null) and (dLdI not null) dL/dI of the channel's
@@ -87,15 +92,16 @@ constexpr int kLossKeep = 4096;
 // division and one logarithm per channel, each in a block of its own (the
 // total kernel took them all in one block), and the detector sums formed once.
 // 4096 channels of 50 x 50: 157 -> 64 us; 2048 channels of 32 x 32 on
-// 4 x 4-pixel detectors 88 -> 37 us; 4 channels of 32 x 32 20 -> 11 us
+// 4 x 4-pixel detectors 88 -> 31 us (37 us with blocks of 256 threads); 4 channels of 32 x 32 20 -> 11 us
 // (with the total and the PSNR, both launches before).
-__global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__ o, const float* __restrict__ T,
+template <int NT>
+__global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const float* __restrict__ T,
                                                       LossStats* __restrict__ st, int fov, int b,
                                                       float* __restrict__ dLdI, float scale, double norm, int mode,
                                                       float* __restrict__ psnr, double* __restrict__ d_loss,
                                                       unsigned* __restrict__ ticket) {
   extern __shared__ float dsh[];  // [det2] detector values, when det2 <= kLossKeep
-  __shared__ float part[3][kRedThreads];
+  __shared__ float part[3][NT];
   __shared__ double tot[3];
   __shared__ float sg_sh;
   __shared__ bool last;
@@ -106,7 +112,7 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   const float2* ow = o + (size_t)w * fov * fov;
   const float* tw = T + (size_t)w * det2;
   float fse = 0.f, fit = 0.f, fii = 0.f;
-  for (int p = threadIdx.x; p < det2; p += kRedThreads) {
+  for (int p = threadIdx.x; p < det2; p += NT) {
     const float I = detector(ow, fov, b, p);
     const float t = tw[p];
     const float d = I - t;
@@ -120,7 +126,7 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   part[2][threadIdx.x] = fii;
   __syncthreads();
   if (warp < 3) {
-    const double v = warp_total(part[warp], lane);
+    const double v = warp_total<NT>(part[warp], lane);
     if (lane == 0) tot[warp] = v;
   }
   __syncthreads();
@@ -134,7 +140,7 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   const bool scaled = mode == DOS_LOSS_MSE_SCALED;
   float* gw = dLdI ? dLdI + (size_t)w * fov * fov : nullptr;
   float fsc = 0.f;
-  for (int p = threadIdx.x; p < det2; p += kRedThreads) {
+  for (int p = threadIdx.x; p < det2; p += NT) {
     const float I = keep ? dsh[p] : detector(ow, fov, b, p);
     const float t = tw[p];
     const float d = fmaf(sg, I, -t);
@@ -143,7 +149,7 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   }
   if (gw && b > 1) {
     const int fov2 = fov * fov;
-    for (int q = threadIdx.x; q < fov2; q += kRedThreads) {
+    for (int q = threadIdx.x; q < fov2; q += NT) {
       const int p = ((q / fov) / b) * fd + (q % fov) / b;  // detector pixel covering q
       const float I = keep ? dsh[p] : detector(ow, fov, b, p);
       const float t = tw[p];
@@ -153,7 +159,7 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   part[0][threadIdx.x] = fsc;
   __syncthreads();
   if (warp == 0) {
-    const double ssc = warp_total(part[0], lane);
+    const double ssc = warp_total<NT>(part[0], lane);
     if (lane == 0) {
       LossStats s;
       s.sse = tot[0];
@@ -170,17 +176,17 @@ __global__ void __launch_bounds__(kRedThreads) k_loss(const float2* __restrict__
   if (!last) return;
   // every channel's record is in place: the total, in a fixed order (each
   // thread a stride of the channels, the threads in order of one tree)
-  __shared__ double acc[kRedThreads];
+  __shared__ double acc[NT];
   __threadfence();
   double v = 0.0;
-  for (int c = threadIdx.x; c < (int)gridDim.x; c += kRedThreads)
+  for (int c = threadIdx.x; c < (int)gridDim.x; c += NT)
     v += __ldcg(scaled ? &st[c].sse_sc : &st[c].sse);
   acc[threadIdx.x] = v;
   __syncthreads();
   if (warp == 0) {
     v = 0.0;
 #pragma unroll
-    for (int i = 0; i < kRedThreads / 32; ++i) v += acc[lane + 32 * i];
+    for (int i = 0; i < NT / 32; ++i) v += acc[lane + 32 * i];
 #pragma unroll
     for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
     if (lane == 0) {
@@ -195,7 +201,8 @@ cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, 
   const float scale = (float)(2.0 / norm);  // dL/dD = 2 (D - T) / norm
   const int det2 = (fov / bin) * (fov / bin);
   const size_t sm = det2 <= kLossKeep ? sizeof(float) * det2 : 0;
-  return launch_next(k_loss, dim3(nw), kRedThreads, sm, s, o, T, st, fov, bin, dLdI, scale, norm, mode, psnr, d_loss,
+  const bool small = det2 <= kLossSmall;
+  return launch_next(small ? k_loss<128> : k_loss<kRedThreads>, dim3(nw), small ? 128 : kRedThreads, sm, s, o, T, st, fov, bin, dLdI, scale, norm, mode, psnr, d_loss,
                      ticket);
 }
 

@@ -418,11 +418,17 @@ struct Pass {
 };
 
 // ------------------------------------------------------------------ kernels
-// The forward row pass of lines with up to 20 elements per thread fits three
-// blocks per SM in 64 registers per thread without spills (measured faster than
-// two; the column pass is faster with its own register allocation).
+// Resident blocks per SM that the row kernels' register counts are held to
+// (they would drift just past): three of the 320-thread blocks of M = 400 (64
+// registers; the column pass is faster with its own register allocation), four
+// of the 256-thread ones of M = 256 (64 registers without spills: a 96-channel
+// 101 x 101 design is then one wave), three at M = 512 for the kernels of one
+// DFT (85 registers: 2048 x 256 seed pass 167 -> 140 us, propagation 64 x 256 172
+// -> 167 us) but the output pass, which that made slower (134 -> 149 us).
 template <class LF>
-constexpr int pass_min_blocks() { return LF::E <= 20 ? 3 : 1; }
+constexpr int pass_min_blocks() { return LF::M == 256 ? 4 : LF::E <= 20 ? 3 : 1; }
+template <class LF>
+constexpr int single_min_blocks() { return LF::M == 512 ? 3 : pass_min_blocks<LF>(); }
 // column pass: the halved kernel fits three blocks per SM without spills
 template <class LF, bool HALF>
 constexpr int col_min_blocks() { return HALF && LF::M == 400 ? 3 : 0; }
@@ -436,17 +442,15 @@ __global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, pass_min_blocks<LF>())
   Pass<LF, HALF>::template row_fwd<SAVE>(a);
 }
 template <class LF, bool HALF>
-__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, pass_min_blocks<LF>()) k_row_first(PassArgs a) {
+__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, single_min_blocks<LF>()) k_row_first(PassArgs a) {
   Pass<LF, HALF>::row_first(a);
 }
-// the output and seed passes: three blocks per SM where the lines are short
-// (the register count would otherwise drift past 64 and leave two)
 template <class LF, bool HALF>
 __global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, pass_min_blocks<LF>()) k_row_out(PassArgs a) {
   Pass<LF, HALF>::row_out(a);
 }
 template <class LF, bool HALF>
-__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, pass_min_blocks<LF>()) k_row_seed(PassArgs a) {
+__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, single_min_blocks<LF>()) k_row_seed(PassArgs a) {
   Pass<LF, HALF>::row_seed(a);
 }
 template <class LF, bool HALF, bool FIRST>
@@ -454,11 +458,11 @@ __global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, col_min_blocks<LF, HAL
   Pass<LF, HALF>::template row_adj<FIRST>(a);
 }
 template <class LF, bool HALF>
-__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL) k_row_in(PassArgs a) {
+__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, single_min_blocks<LF>()) k_row_in(PassArgs a) {
   Pass<LF, HALF>::row_in(a);
 }
 template <class LF, bool HALF>
-__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL) k_row_back(PassArgs a) {
+__global__ void __launch_bounds__(LF::T * Pass<LF>::ROWL, single_min_blocks<LF>()) k_row_back(PassArgs a) {
   Pass<LF, HALF>::row_back(a);
 }
 

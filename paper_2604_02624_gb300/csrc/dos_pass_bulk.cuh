@@ -790,7 +790,7 @@ __global__ void __launch_bounds__(LF::T * RL, 3) k_row_adj_staged(PassArgs a) {
 // Column pass: four blocks of 8 lines per SM for every line shape (M = 400: 20
 // warps at up to 102 registers, M = 512: 16 at up to 128).
 template <class LF>
-constexpr int col_bulk_min_blocks() { return LF::T >= 16 ? 4 : 8; }
+constexpr int col_bulk_min_blocks() { return LF::M == 256 ? 6 : LF::T >= 16 ? 4 : 8; }
 template <class LF, int RL, bool HALF, bool ADJ, bool MIS>
 __global__ void __launch_bounds__(PassBulk<LF, RL, HALF>::GT, col_bulk_min_blocks<LF>())
     k_col_bulk(PassArgs a, const __grid_constant__ CUtensorMap smap, const __grid_constant__ CUtensorMap hmap) {
