@@ -24,7 +24,8 @@
 
 namespace dos {
 
-// sin and cos of 2 pi f for |f| <= 1/2 (a thickness phase in cycles), FP32.
+// sin and cos of 2 pi f for |f| <= 1/2 and a little over (a reduced phase in
+// cycles), FP32.
 // 4 f = k + r with k the nearest integer (the low bits of 4 f + 1.5 2^23, whose
 // ulp is 1) and |r| <= 1/2 exact; sin and cos of r pi/2 are polynomials in r^2
 // fitted here for the least largest error (3.2e-9 and 4e-10 before rounding;

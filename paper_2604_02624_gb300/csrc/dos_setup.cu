@@ -11,6 +11,7 @@
 //  * the line-FFT twiddles exp(-2 pi j q k / M);
 //  * per-channel constants of the transmission of Eq. 1-2.
 #include "dos_internal.h"
+#include "dos_pass.cuh"
 
 #include "../../include/dos.h"
 
@@ -88,12 +89,13 @@ cudaError_t launch_sqtable(float* sq, float* sq_lo, const double* d_lambda, int 
 // Root and length as FP32 pairs: a root rounded to FP32 turns the phase by up to
 // 2e-7 of a wavelength per wavelength of dz.
 __device__ __forceinline__ float2 longer(float2 h, float sq, float sq_lo, float2 dz) {
-  float amp = 1.0f, ph = 0.0f;
-  if (sq >= 0.0f) ph = fmaf(dz.x, sq_lo, cycles(sq, dz));
-  else amp = expf(6.283185307179586f * dz.x * sq);
-  float sn, cs;
-  sincospif(2.0f * ph, &sn, &cs);
-  const float re = amp * cs, im = amp * sn;
+  float re, im;
+  if (sq >= 0.0f) {
+    sincos_turns(fmaf(dz.x, sq_lo, cycles(sq, dz)), &im, &re);
+  } else {
+    re = expf(6.283185307179586f * dz.x * sq);
+    im = 0.0f;
+  }
   return make_float2(fmaf(h.x, re, -h.y * im), fmaf(h.x, im, h.y * re));
 }
 __global__ void __launch_bounds__(256) k_longer_tables(LongerTables t, const float4* __restrict__ Hq,
