@@ -1060,13 +1060,17 @@ std::string choice_detail(const dos_ctx* x, int idx) {
 
 // The step replays a graph, so its choice is the one whose kernels take the
 // least time.  The stream calls also cost the host their launches, and their
-// callers do host work of their own between them (an objective in PyTorch is
-// ten and more operations of some 5 us): their choice is the one with the
-// shortest pass beside kCallerMs of that, the longer of the GPU's time and the
-// host's.  It differs where a whole pass takes less than that: 6 channels of
-// 200 x 200, 12 calls and 55 us on the GPU with the multi-pass kernels, 4 and 78 us
-// cluster-resident; under autograd (host-bound) 446 against 406 us a pass.
-constexpr float kCallerMs = 0.06f;
+// callers do host work of their own between them: some 60 us where a loop only
+// forms its objective, some 300 us under autograd.  A pass then takes the longer
+// of the GPU's time and the host's, and the stream calls' choice has the least
+// sum over the two callers.  It differs from the step's where a pass takes less
+// than that: 6 channels of 200 x 200, 12 calls and 55 us on the GPU with the
+// multi-pass kernels, 4 and 78 us cluster-resident, 446 against 406 us a pass
+// under autograd; 15 of 191 x 191, 106 and 123 us, 425 against 397 us.
+constexpr float kCallerMs[2] = {0.06f, 0.3f};
+float call_cost(float gpu_ms, float host_ms) {
+  return std::max(gpu_ms, host_ms + kCallerMs[0]) + std::max(gpu_ms, host_ms + kCallerMs[1]);
+}
 
 // time forward(save) + backward of the current choice on zero thickness / zero
 // seed; with kind_ms, one more forward + backward with per-launch events gives
@@ -1233,7 +1237,7 @@ int choose_path(dos_ctx* x, int requested) {
       best_ms = ms;
       best = idx;
     }
-    const float call_ms = std::max(ms, host_ms + kCallerMs);
+    const float call_ms = call_cost(ms, host_ms);
     if (call_ms < best_call_ms || (call_ms == best_call_ms && best == idx)) {
       best_call_ms = call_ms;
       best_call = idx;
