@@ -145,10 +145,13 @@ struct dos_ctx {
   bool in_step = false;  // a step is being captured: its gradient reduction keeps the thickness
   dos::LossStats* stats = nullptr;
   double* d_loss = nullptr;
-  unsigned* col_work = nullptr;     // items drawn in the running column pass (zero between launches)
+  // items drawn in the running column pass and, from [1], chunks drawn per row
+  // block (at most one for each layer row) in the running row pass; zero
+  // between launches
+  unsigned* counters = nullptr;
   unsigned* loss_ticket = nullptr;  // channels done in the running loss kernel (zero between launches)
   double* h_loss = nullptr;  // pinned
-  // channels per block of the adjoint row pass, plain and prefetching
+  // channels per block of the plain adjoint row pass, and per chunk of the prefetching one
   int chunk_plain = 1, chunk_bulk = 1;
   // multi-pass passes that run their bulk-async prefetching kernels
   // (DOS_PATH_MULTIPASS_BULK: all three; the autotuner may mix them per kind)
@@ -285,7 +288,8 @@ struct dos_ctx {
     a.chunk = adj_chunk();
     a.n_chunks = chunks_of(a.chunk);
     a.err = d_err;
-    a.work = col_work;
+    a.work = counters;
+    a.row_work = counters + 1;
     a.tmap = have_tmap ? &tmap_S : nullptr;
     a.tmap_rows = n;
     a.hmap = have_tmap ? &tmap_H : nullptr;
@@ -436,7 +440,7 @@ int build(dos_ctx* x, const dos_config* c) {
   }
   x->n_slots = (int)slots.size();
   // channel chunks of the plain adjoint row pass: about 8 blocks per SM in
-  // flight; the prefetching one has its own (whole waves of its resident blocks)
+  // flight; the prefetching one has its own
   const int row_blocks = (x->n + x->ops->row_lines - 1) / x->ops->row_lines;
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
@@ -526,8 +530,8 @@ int build(dos_ctx* x, const dos_config* c) {
   if ((rc = x->alloc(&x->h_fwd, (size_t)x->K * n2, "saved thickness"))) return rc;
   if ((rc = x->alloc(&x->stats, (size_t)x->nw, "loss statistics"))) return rc;
   if ((rc = x->alloc(&x->d_loss, 1, "loss"))) return rc;
-  if ((rc = x->alloc(&x->col_work, 1, "column item counter"))) return rc;
-  DOS_CUDA(cudaMemsetAsync(x->col_work, 0, sizeof(unsigned), x->stream), "column item counter");
+  if ((rc = x->alloc(&x->counters, 1 + (size_t)x->n, "work counters"))) return rc;
+  DOS_CUDA(cudaMemsetAsync(x->counters, 0, sizeof(unsigned) * (1 + (size_t)x->n), x->stream), "work counters");
   if ((rc = x->alloc(&x->loss_ticket, 1, "loss ticket"))) return rc;
   DOS_CUDA(cudaMemsetAsync(x->loss_ticket, 0, sizeof(unsigned), x->stream), "loss ticket");
   if ((rc = x->alloc(&x->dLdI_step, (size_t)x->nw * x->fov * x->fov, "step seed"))) return rc;
@@ -582,7 +586,7 @@ int flag_after_sync(dos_ctx* c) {
   if (*c->h_err) {
     *c->h_err = 0;
     DOS_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream), "error flag");
-    DOS_CUDA(cudaMemsetAsync(c->col_work, 0, sizeof(unsigned), c->stream), "column item counter");
+    DOS_CUDA(cudaMemsetAsync(c->counters, 0, sizeof(unsigned) * (1 + (size_t)c->n), c->stream), "work counters");
     return fail(DOS_ERR_TIMEOUT, "a bounded wait gave up (mbarrier wait for a tensor-core commit or a bulk copy "
                                  "expired); results of the call are invalid");
   }

@@ -110,11 +110,12 @@ struct PassArgs {
   int n, m, nw, fov, of, hs;
   int in_r0, in_r1;       // column pass: rows that may be non-zero on input
   int out_r0, out_r1;     // column pass: rows stored on output
-  int chunk;              // channels per block of the adjoint row pass (the bulk forward ones set their own)
+  int chunk;              // channels per chunk of the adjoint row pass (the bulk forward ones set their own)
   int n_chunks;
   bool displaced;         // column pass: the gap carries a displacement that Hq does not hold (mis)
   Misalign mis;           // its lateral shift; and, with mis.sq, its length change (plain kernel only)
   unsigned* work;         // item counter of the bulk column pass, 0 between launches
+  unsigned* row_work;     // chunk counters of the bulk row passes, one per row block, 0 between launches
   int* err;               // set to 1 by a bulk-copy pass whose bounded wait expired
   int stall;              // fault injection (tests): 1 = the bulk pass expects bytes that are never
                           // copied; 2 = its copies land but odd threads give up their first wait;
@@ -145,7 +146,7 @@ struct PassOps {
   cudaError_t (*bulk_row_fwd)(const PassArgs&, bool save, cudaStream_t);
   cudaError_t (*bulk_row_adj)(const PassArgs&, bool first, cudaStream_t);
   cudaError_t (*bulk_row_first)(const PassArgs&, cudaStream_t);  // t(h) * field (fin) -> row spectra
-  int (*bulk_adj_chunk)(int n, int nw, int most);  // channels per block of bulk_row_adj (0: unknown)
+  int (*bulk_adj_chunk)(int n, int nw, int most);  // channels per chunk of bulk_row_adj (0: unknown)
   // boxes of the bulk column pass's tensor copies: spectra {col_group, rows, 1},
   // transfer table {h_box_cols, h_box_rows, 1} (h_box_cols 0: no staged H tile)
   int col_group, h_box_cols, h_box_rows;

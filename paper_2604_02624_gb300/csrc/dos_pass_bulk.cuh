@@ -380,18 +380,153 @@ struct PassBulk {
   }
 
   // ------------------------------------------------------------- row passes
-  // dynamic shared memory: stage[RL][SR] | exchange[RL][RZL] | tw[TWS] | barrier
+  // Block (x, y) of a forward pass holds the rows [x RL, +RL).  With up to 20
+  // elements per thread (DRAW) the blocks are persistent and take channel y,
+  // then whatever a counter of their row block says, as the column pass does:
+  // thread 0 draws two channels ahead, publishes the next one before the first
+  // barrier of the current one, and whoever draws the last number (a.nw of them
+  // per row block in all) leaves the counter at 0.  4096 x 200 launch 0.931 ->
+  // 0.901 ms, 1024 x 200 236 -> 225 us, 256 x 200 70.5 -> 67.5 us.  At M = 512 that
+  // was slower (2048 x 256 0.848 -> 0.866 ms): there block (x, y) takes the
+  // channels of chunk y.  (The adjoint passes sum a fixed chunk of channels per
+  // block, so that the gradient is reproducible; persistent blocks drawing such
+  // chunks were slower: 4096 x 200 1.05 -> 1.12 ms.)
+  static constexpr bool DRAW = LF::E <= 20;
+  struct Draw {
+    unsigned* work;  // this row block's counter
+    int* next_sh;    // published next channel
+    unsigned drawn;  // thread 0: the counter's answer for the channel after the current one
+    int w;           // current channel
+    int nw, end;     // channels; end of the chunk (not DRAW)
+    __device__ __forceinline__ Draw(const PassArgs& a, int* sh) : work(a.row_work + blockIdx.x), next_sh(sh), drawn(0) {
+      nw = a.nw;
+      if constexpr (DRAW) {
+        w = blockIdx.y;
+        if (threadIdx.x == 0) drawn = atomicAdd(work, 1u);
+      } else {
+        w = blockIdx.y * a.chunk;
+        end = min(nw, w + a.chunk);
+      }
+    }
+    // thread 0, before the first barrier of a channel
+    __device__ __forceinline__ void publish() {
+      if (!DRAW || threadIdx.x != 0) return;
+      *next_sh = (int)min(drawn + gridDim.y, (unsigned)nw);
+      if (drawn == (unsigned)nw - 1u) *work = 0u;
+    }
+    // every thread, after that barrier: the channel that follows (nw: none)
+    __device__ __forceinline__ int next() {
+      if constexpr (!DRAW) return w + 1 < end ? w + 1 : nw;
+      const int n = *next_sh;
+      if (threadIdx.x == 0 && n < nw) drawn = atomicAdd(work, 1u);
+      return n;
+    }
+  };
+
+  // dynamic shared memory: stage[RL][SR] | exchange[RL][RZL] | tw[TWS] | barrier | next channel
   static size_t row_smem() {
-    return sizeof(float2) * ((size_t)RL * SR + (size_t)RL * RZL + LF::TWS + 1) + sizeof(uint64_t);
+    return sizeof(float2) * ((size_t)RL * SR + (size_t)RL * RZL + LF::TWS + 1) + 2 * sizeof(uint64_t);
   }
 
-  // Rows [blockIdx.x * RL, +RL) of the channels of chunk blockIdx.y.
-  //   ADJ false : forward layer pass (as Pass::row_fwd), FLAG = save the checkpoint
-  //   ADJ true  : adjoint layer pass (as Pass::row_adj), FLAG = first layer; it
-  //               runs only for odd N (the checkpoint rows are then not 16-byte
-  //               multiples and are read directly), row_adj_staged otherwise
-  template <bool ADJ, bool FLAG>
-  __device__ static void row(const PassArgs& a) {
+  // Forward layer pass (as Pass::row_fwd), SAVE = save the checkpoint.
+  template <bool SAVE>
+  __device__ static void row_fwd(const PassArgs& a) {
+    extern __shared__ __align__(16) float2 smem[];
+    float2* stage = smem;
+    float2* zb = stage + (size_t)RL * SR;
+    float2* tw = tw_align(zb + (size_t)RL * RZL);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(tw + LF::TWS);
+    const int l = threadIdx.x / T, t = threadIdx.x % T;
+    float2* z = zb + l * RZL;
+    const int r0 = blockIdx.x * RL;
+    const int nrows = min(RL, a.n - r0);
+    const bool ok = l < nrows;
+    const int rr = ok ? r0 + l : r0;
+    const uint32_t bytes = (uint32_t)nrows * M * 8u;
+    if (threadIdx.x == 0) bulk_bar_init(bar);
+    for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
+    pdl_wait();
+    __syncthreads();
+    // thread 0 copies the block's rows of channel w, one bulk copy (M * 8 bytes) per row
+    auto fetch = [&](int w) {
+      if (threadIdx.x != 0) return;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      bulk_expect(bar, bytes);
+      if (a.stall == 1) return;  // injected fault: the expected bytes never arrive
+      const float2* src = a.S + ((size_t)w * a.n + r0) * M;
+      for (int q = 0; q < nrows; ++q) bulk_g2s(stage + (size_t)q * SR, src + (size_t)q * M, M * 8u, bar);
+    };
+    Draw draw(a, reinterpret_cast<int*>(bar + 1));
+    fetch(draw.w);
+    // the thickness row stays in registers
+    const float* hrow = a.h + (size_t)rr * a.n;
+    float hv[E];
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      const int x = t + T * i;
+      hv[i] = (i < EF && x < a.n) ? __ldg(hrow + x) : 0.f;
+    }
+    bool okw = true;
+    int k = 0;
+    // the next channel's constants are loaded one iteration ahead
+    ChanConst cnext = a.chan[draw.w];
+    for (; draw.w < a.nw; ++k) {
+      const int w = draw.w;
+      const ChanConst cc = cnext;
+      draw.publish();
+      // a thread whose wait expires goes on to the barrier with what is there,
+      // where the whole block stops
+      const bool got = bulk_wait(bar, (uint32_t)(k & 1), split_verdict(a, k));
+      float2 r[E];
+#pragma unroll
+      for (int i = 0; i < E; ++i) r[i] = stage[(size_t)(ok ? l : 0) * SR + t + T * i];
+      LF::template step1<true, LF::P, PKR>(r, t, z, tw);
+      // one verdict for the whole block; every thread is past its stage reads:
+      // the next channel may land there
+      okw = __syncthreads_and(got) != 0;
+      if (!okw) break;
+      const int wn = draw.next();
+      if (wn < a.nw) {
+        fetch(wn);
+        cnext = a.chan[wn];
+      }
+      // the forward DFT below writes the exchange matrix in the other layout
+      // (only what this thread reads here), and the next channel's inverse
+      // DFT again: no barrier between them
+      LF::template step2<true, NOI, PKR>(r, t, z);
+      float2* srow = a.S + ((size_t)w * a.n + rr) * M;
+      float2* ck = a.ckpt + ((size_t)w * a.n + rr) * a.n;
+#pragma unroll
+      for (int i = 0; i < E; ++i) {
+        const int x = t + T * i;
+        if (i < EF && x < a.n) {
+          const float2 v = r[i];
+          if (SAVE && ok) ck[x] = v;
+          r[i] = cmul(transmission(hv[i], cc), v);
+        } else {
+          r[i] = czero();
+        }
+      }
+      LF::template fft<false, NZF, LF::Q, false, PKR, true>(r, t, z, tw);
+      if (ok) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
+      }
+      draw.w = wn;
+    }
+    if (!okw && threadIdx.x == 0) {
+      // (the counter is left where it is: the host zeroes it with the flag)
+      (void)bulk_wait(bar, (uint32_t)(k & 1));  // a late copy lands (bounded) before the block leaves
+      atomicExch(a.err, 1);
+    }
+  }
+
+  // Adjoint layer pass (as Pass::row_adj) over the rows [blockIdx.x * RL, +RL)
+  // of the channels of chunk blockIdx.y, FIRST = first layer, for odd N (the
+  // checkpoint rows are then not 16-byte multiples and are read directly);
+  // row_adj_staged otherwise.
+  template <bool FIRST>
+  __device__ static void row_adj(const PassArgs& a) {
     extern __shared__ __align__(16) float2 smem[];
     float2* stage = smem;
     float2* zb = stage + (size_t)RL * SR;
@@ -420,18 +555,9 @@ struct PassBulk {
       const float2* src = a.S + ((size_t)w * a.n + r0) * M;
       for (int q = 0; q < nrows; ++q) bulk_g2s(stage + (size_t)q * SR, src + (size_t)q * M, M * 8u, bar);
     };
-    // the thickness row is held in registers by the forward pass; the adjoint
-    // pass (which also carries its gradient and the checkpoint) re-reads it
-    // from L1 per channel
+    // the thickness row is re-read from L1 per channel (beside the gradient
+    // sums and the checkpoint)
     const float* hrow = a.h + (size_t)rr * a.n;
-    float hv[ADJ ? 1 : E];
-    if constexpr (!ADJ) {
-#pragma unroll
-      for (int i = 0; i < E; ++i) {
-        const int x = t + T * i;
-        hv[i] = (i < EF && x < a.n) ? __ldg(hrow + x) : 0.f;
-      }
-    }
     float g[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) g[i] = 0.f;
@@ -460,44 +586,24 @@ struct PassBulk {
       // DFT again: no barrier between them
       LF::template step2<true, NOI, PKR>(r, t, z);
       float2* srow = a.S + ((size_t)w * a.n + rr) * M;
-      if constexpr (!ADJ) {
-        float2* ck = a.ckpt + ((size_t)w * a.n + rr) * a.n;
+      const float2* ck = a.ckpt + ((size_t)w * a.n + rr) * a.n;
 #pragma unroll
-        for (int i = 0; i < E; ++i) {
-          const int x = t + T * i;
-          if (i < EF && x < a.n) {
-            const float2 v = r[i];
-            if (FLAG && ok) ck[x] = v;
-            r[i] = cmul(transmission(hv[i], cc), v);
-          } else {
-            r[i] = czero();
-          }
+      for (int i = 0; i < E; ++i) {
+        const int x = t + T * i;
+        if (i < EF && x < a.n) {
+          r[i] = adjoint_pixel(r[i], transmission(__ldg(hrow + x), cc), ck[x], cc, g[i]);
+        } else {
+          r[i] = czero();
         }
+      }
+      if constexpr (!FIRST) {
         LF::template fft<false, NZF, LF::Q, false, PKR, true>(r, t, z, tw);
         if (ok) {
 #pragma unroll
           for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
         }
       } else {
-        const float2* ck = a.ckpt + ((size_t)w * a.n + rr) * a.n;
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-          const int x = t + T * i;
-          if (i < EF && x < a.n) {
-            r[i] = adjoint_pixel(r[i], transmission(__ldg(hrow + x), cc), ck[x], cc, g[i]);
-          } else {
-            r[i] = czero();
-          }
-        }
-        if constexpr (!FLAG) {
-          LF::template fft<false, NZF, LF::Q, false, PKR, true>(r, t, z, tw);
-          if (ok) {
-#pragma unroll
-            for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
-          }
-        } else {
-          __syncthreads();  // the next channel writes the exchange matrix in the same layout
-        }
+        __syncthreads();  // the next channel writes the exchange matrix in the same layout
       }
     }
     if (!okw) {
@@ -507,7 +613,7 @@ struct PassBulk {
       }
       return;
     }
-    if constexpr (ADJ) {
+    {
       if (ok) {
         float* prow = a.partial + ((size_t)blockIdx.y * a.n + row) * a.n;
 #pragma unroll
@@ -522,9 +628,9 @@ struct PassBulk {
   // -------------------------------------------------------- first row pass
   // t(h) * v1 -> pad -> DFT (as Pass::row_first) with the next channel's rows
   // of the input-field table v1 (fin) staged by bulk copies.  Needs N even.
-  // dynamic shared memory: stage[RL][cks] | exchange[RL][RZL] | tw[TWS] | barrier
+  // dynamic shared memory: stage[RL][cks] | exchange[RL][RZL] | tw[TWS] | barrier | next channel
   static size_t first_smem(int n) {
-    return sizeof(float2) * ((size_t)RL * ck_stride(n) + (size_t)RL * RZL + LF::TWS + 1) + sizeof(uint64_t);
+    return sizeof(float2) * ((size_t)RL * ck_stride(n) + (size_t)RL * RZL + LF::TWS + 1) + 2 * sizeof(uint64_t);
   }
 
   __device__ static void row_first_staged(const PassArgs& a) {
@@ -542,8 +648,6 @@ struct PassBulk {
     const bool ok = l < nrows;
     const int rr = ok ? row : r0;
     const int lr = ok ? l : 0;
-    const int w0 = blockIdx.y * a.chunk;
-    const int w1 = min(a.nw, w0 + a.chunk);
     const uint32_t bytes = (uint32_t)nrows * a.n * 8u;
     if (threadIdx.x == 0) bulk_bar_init(bar);
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = a.tw[i];
@@ -557,6 +661,8 @@ struct PassBulk {
       const float2* src = a.fin + ((size_t)w * a.n + r0) * a.n;
       for (int q = 0; q < nrows; ++q) bulk_g2s(stage + (size_t)q * cks, src + (size_t)q * a.n, a.n * 8u, bar);
     };
+    Draw draw(a, reinterpret_cast<int*>(bar + 1));
+    fetch(draw.w);
     const float* hrow = a.h + (size_t)rr * a.n;
     float hv[E];
 #pragma unroll
@@ -565,15 +671,17 @@ struct PassBulk {
       hv[i] = (i < EF && x < a.n) ? __ldg(hrow + x) : 0.f;
     }
     bool okw = true;
-    if (w0 < w1) fetch(w0);
     int k = 0;
     // the next channel's constants are loaded one iteration ahead
-    ChanConst cnext = a.chan[w0 < w1 ? w0 : 0];
-    for (int w = w0; w < w1; ++w, ++k) {
+    ChanConst cnext = a.chan[draw.w];
+    for (; draw.w < a.nw; ++k) {
+      const int w = draw.w;
       const ChanConst cc = cnext;
-      if (w + 1 < w1) cnext = a.chan[w + 1];
+      draw.publish();
       okw = __syncthreads_and(bulk_wait(bar, (uint32_t)(k & 1), split_verdict(a, k))) != 0;  // one verdict for the whole block
       if (!okw) break;
+      const int wn = draw.next();
+      if (wn < a.nw) cnext = a.chan[wn];
       float2 r[E];
 #pragma unroll
       for (int i = 0; i < E; ++i) {
@@ -582,13 +690,14 @@ struct PassBulk {
       }
       LF::template step1<false, NZF, PKR>(r, t, z, tw);
       __syncthreads();  // every thread is past its stage reads: the next channel may land there
-      if (w + 1 < w1) fetch(w + 1);
+      if (wn < a.nw) fetch(wn);
       LF::template step2<false, LF::Q, PKR>(r, t, z);  // next z write follows the loop-top barrier
       if (ok) {
         float2* srow = a.S + ((size_t)w * a.n + rr) * M;
 #pragma unroll
         for (int i = 0; i < E; ++i) srow[t + T * i] = r[i];
       }
+      draw.w = wn;
     }
     if (!okw && threadIdx.x == 0) {
       (void)bulk_wait(bar, (uint32_t)(k & 1));  // a late copy lands (bounded) before the block leaves
@@ -799,16 +908,20 @@ __global__ void __launch_bounds__(PassBulk<LF, RL, HALF>::GT, col_bulk_min_block
 // the row passes: as many resident blocks as their shared memory allows
 template <class LF, int RL>
 constexpr int row_bulk_min_blocks() { return LF::E <= 20 ? (RL <= 8 ? 4 : 2) : 1; }
-template <class LF, int RL, bool HALF, bool ADJ, bool FLAG>
+template <class LF, int RL, bool HALF, bool SAVE>
 __global__ void __launch_bounds__(LF::T * RL, row_bulk_min_blocks<LF, RL>()) k_row_bulk(PassArgs a) {
-  PassBulk<LF, RL, HALF>::template row<ADJ, FLAG>(a);
+  PassBulk<LF, RL, HALF>::template row_fwd<SAVE>(a);
+}
+template <class LF, int RL, bool HALF, bool FIRST>
+__global__ void __launch_bounds__(LF::T * RL, row_bulk_min_blocks<LF, RL>()) k_row_adj_bulk(PassArgs a) {
+  PassBulk<LF, RL, HALF>::template row_adj<FIRST>(a);
 }
 template <class LF, int RL, bool HALF>
 __global__ void __launch_bounds__(LF::T * RL, row_bulk_min_blocks<LF, RL>()) k_row_first_staged(PassArgs a) {
   PassBulk<LF, RL, HALF>::row_first_staged(a);
 }
 
-// Channels per block of a row pass.  A launch of rb row blocks x c chunks runs
+// Channels per block of a row pass in chunks.  A launch of rb row blocks x c chunks runs
 // in waves of `slots` resident blocks, each as long as one block's channels
 // plus about one channel's time to start (twiddles, thickness row, the first
 // copy's latency) and to finish: the split with the smallest waves x (channels
@@ -829,11 +942,10 @@ inline int balanced_chunk(int nw, int rb, int slots, int most) {
   }
   return best;
 }
-// Most channels per block.  The adjoint row pass sums its chunk's channels in
+// Most channels per block: the adjoint row pass sums its chunk's channels in
 // FP32 registers (before balanced_chunk: 45 at 4096 channels, so no more terms
-// than then); and in both passes long chunks spread the blocks that run
-// together over the whole spectra buffer: forward 0.95 -> 0.99 ms at 4096
-// channels with 171 per block.
+// than then), and long chunks spread the blocks that run together over the
+// whole spectra buffer.
 constexpr int kRowChunk = 48;
 
 // Launchers.  The column pass runs one persistent block per resident slot
@@ -879,8 +991,8 @@ struct PassBulkLaunch {
       return PassLaunch<LF>::col(a, adj, false, s);
     return half(a) ? col_h<true>(a, adj, sm, s) : col_h<false>(a, adj, sm, s);
   }
-  // Launch of a forward row kernel over all channels: the channels split into
-  // chunks (grid.y) that fill whole waves of the resident slots.
+  // Launch of a forward row kernel: persistent blocks (DRAW), as many per row
+  // block as are resident at once and at most one per channel, or one per chunk.
   template <typename K>
   static cudaError_t launch_rows(K kernel, size_t sm, const PassArgs& a, cudaStream_t s) {
     int n_slots = 0;
@@ -889,13 +1001,14 @@ struct PassBulkLaunch {
     PassArgs b = a;
     const int rb = (a.n + RL - 1) / RL;
     b.chunk = balanced_chunk(a.nw, rb, n_slots, kRowChunk);
-    return launch_next(kernel, dim3(rb, (a.nw + b.chunk - 1) / b.chunk), PB::RT, sm, s, b);
+    const int per = PB::DRAW ? std::min(a.nw, std::max(1, n_slots / rb)) : (a.nw + b.chunk - 1) / b.chunk;
+    return launch_next(kernel, dim3(rb, per), PB::RT, sm, s, b);
   }
   template <bool H>
   static cudaError_t row_fwd_h(const PassArgs& a, bool save, cudaStream_t s) {
     const size_t sm = PB::row_smem();
-    return save ? launch_rows(k_row_bulk<LF, RL, H, false, true>, sm, a, s)
-                : launch_rows(k_row_bulk<LF, RL, H, false, false>, sm, a, s);
+    return save ? launch_rows(k_row_bulk<LF, RL, H, true>, sm, a, s)
+                : launch_rows(k_row_bulk<LF, RL, H, false>, sm, a, s);
   }
   static cudaError_t row_fwd(const PassArgs& a, bool save, cudaStream_t s) {
     return half(a) ? row_fwd_h<true>(a, save, s) : row_fwd_h<false>(a, save, s);
@@ -922,8 +1035,8 @@ struct PassBulkLaunch {
     // odd N: the spectra rows staged, the checkpoint read directly
     const dim3 g((a.n + RL - 1) / RL, a.n_chunks);
     const size_t sm = PB::row_smem();
-    return first ? launch_k(k_row_bulk<LF, RL, H, true, true>, g, PB::RT, sm, a, s)
-                 : launch_k(k_row_bulk<LF, RL, H, true, false>, g, PB::RT, sm, a, s);
+    return first ? launch_k(k_row_adj_bulk<LF, RL, H, true>, g, PB::RT, sm, a, s)
+                 : launch_k(k_row_adj_bulk<LF, RL, H, false>, g, PB::RT, sm, a, s);
   }
   static cudaError_t row_adj(const PassArgs& a, bool first, cudaStream_t s) {
     return half(a) ? row_adj_h<true>(a, first, s) : row_adj_h<false>(a, first, s);
@@ -939,7 +1052,7 @@ struct PassBulkLaunch {
       rows = RLA;
       e = slots(k_row_adj_staged<LF, RLA, H, false>, PBA::RT, PBA::adj_staged_smem(n), &n_slots);
     } else {
-      e = slots(k_row_bulk<LF, RL, H, true, false>, PB::RT, PB::row_smem(), &n_slots);
+      e = slots(k_row_adj_bulk<LF, RL, H, false>, PB::RT, PB::row_smem(), &n_slots);
     }
     if (e != cudaSuccess) {
       (void)cudaGetLastError();

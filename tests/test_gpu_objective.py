@@ -18,7 +18,7 @@ from paper_2604_02624_gb300 import _lib as L
 from paper_2604_02624_gb300 import workloads as W
 from paper_2604_02624_gb300.api import DiffractiveStack
 
-from gpu_cases import TOL_GRAD_ORACLE, assert_close, custom, oracle_model
+from gpu_cases import TOL_GRAD_ORACLE, TOL_INTENSITY, assert_close, custom, oracle_model
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
@@ -62,18 +62,28 @@ def test_objective_matches_its_definition(n, m, fov, b, nw, loss):
     st.close()
 
 
-@pytest.mark.parametrize("nw", [1, 7, 8, 9, 63, 65, 130])
-def test_gradient_over_any_number_of_parts(nw):
-    """Small layers put one channel in a part: slices of the parts that are
-    empty, ragged, exactly one and more than one unrolled step long."""
-    w = custom(13, 32, 2, list(np.linspace(450, 740, nw)), 15, 7, name="parts")
+@pytest.mark.parametrize("path,n,nw", [
+    ("multipass", 13, 1), ("multipass", 13, 7), ("multipass", 13, 8), ("multipass", 13, 9), ("multipass", 13, 63),
+    ("multipass", 13, 65), ("multipass", 13, 130),
+    # the prefetching row passes, whose blocks draw chunks of channels: fewer channels than
+    # resident blocks, a few per block, and many (ragged last chunks), even and odd rows
+    ("multipass_bulk", 13, 1), ("multipass_bulk", 14, 5), ("multipass_bulk", 16, 700), ("multipass_bulk", 14, 3001),
+    ("multipass_bulk", 13, 3001), ("multipass_bulk", 16, 6007),
+])
+def test_gradient_over_any_number_of_parts(path, n, nw):
+    """Slices of the gradient parts that are empty, ragged, exactly one and more
+    than one unrolled step long; chunks of one channel, of several, and cut short."""
+    fov = n - 6
+    w = custom(n, 32, 2, list(np.linspace(450, 740, nw)), 15, fov, name="parts")
     h = W.thickness(w, 0)
-    T = np.random.default_rng(nw).uniform(0.0, 1.0, (nw, 7, 7))
-    st = DiffractiveStack.from_workload(w, device=DEV, path="multipass")
-    st.forward(torch.tensor(h, dtype=torch.float32, device=DEV))
-    _, _, g = st.loss(torch.tensor(T, dtype=torch.float32, device=DEV))
-    got = st.backward(g).cpu().numpy().astype(np.float64)
+    T = np.random.default_rng(nw).uniform(0.0, 1.0, (nw, fov, fov)).astype(np.float32)
+    st = DiffractiveStack.from_workload(w, device=DEV, path=path)
     hf = h.astype(np.float32).astype(np.float64)
-    _, _, ref, _ = O.loss_and_grad(hf, T.astype(np.float32).astype(np.float64), **oracle_model(w))
-    assert_close(got, ref, TOL_GRAD_ORACLE)
+    _, _, ref, fwd = O.loss_and_grad(hf, T.astype(np.float64), **oracle_model(w))
+    for _ in range(2):  # the counters start from zero again
+        I = st.forward(torch.tensor(h, dtype=torch.float32, device=DEV)).cpu().numpy().astype(np.float64)
+        _, _, g = st.loss(torch.tensor(T, device=DEV))
+        got = st.backward(g).cpu().numpy().astype(np.float64)
+        assert_close(I, fwd["I"], TOL_INTENSITY)
+        assert_close(got, ref, TOL_GRAD_ORACLE)
     st.close()
