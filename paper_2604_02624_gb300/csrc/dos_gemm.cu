@@ -494,7 +494,7 @@ __device__ __forceinline__ float2 prep_value(const PrepArgs& g, int n, int w, in
     const size_t at = ((size_t)w * n + y) * n + x;
     const float2 vv = g.v[at];
     g.ckpt[at] = vv;
-    return cmul(transmission(g.h[(size_t)y * n + x], g.chan[w]), vv);
+    return cmul(transmission<true>(g.h[(size_t)y * n + x], g.chan[w]), vv);
   }
 }
 
@@ -550,8 +550,8 @@ __global__ void __launch_bounds__(256) k_prep_field8(PrepArgs g, Parts X, int n,
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       c4[q] = v[q];
-      const float2 u0 = cmul(transmission(hv[2 * q], cc), make_float2(v[q].x, v[q].y));
-      const float2 u1 = cmul(transmission(hv[2 * q + 1], cc), make_float2(v[q].z, v[q].w));
+      const float2 u0 = cmul(transmission<true>(hv[2 * q], cc), make_float2(v[q].x, v[q].y));
+      const float2 u1 = cmul(transmission<true>(hv[2 * q + 1], cc), make_float2(v[q].z, v[q].w));
       re[2 * q] = u0.x, im[2 * q] = u0.y, re[2 * q + 1] = u1.x, im[2 * q + 1] = u1.y;
     }
   } else {
@@ -581,7 +581,7 @@ __global__ void k_field_adj(const float2* __restrict__ field, const float2* __re
   float acc = 0.f;
   for (int w = 0; w < nwc; ++w) {
     const ChanConst cc = chan[w];
-    const float2 u = adjoint_pixel(field[(size_t)w * n2 + p], transmission(hv, cc), ckpt[(size_t)w * n2 + p], cc, acc);
+    const float2 u = adjoint_pixel(field[(size_t)w * n2 + p], transmission<true>(hv, cc), ckpt[(size_t)w * n2 + p], cc, acc);
     if constexpr (!FIRST) {
       split_store(X, gemm_tiled((size_t)w * n + y, x, kp), u.x);
       split_store(X, gemm_tiled((size_t)w * n + y, n + x, kp), u.y);
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(128) k_field_adj8(const float2* __restrict__ f
     for (int e = 0; e < 8; ++e) {
       const float2 au = (e & 1) ? make_float2(f[e / 2].z, f[e / 2].w) : make_float2(f[e / 2].x, f[e / 2].y);
       const float2 v = (e & 1) ? make_float2(c[e / 2].z, c[e / 2].w) : make_float2(c[e / 2].x, c[e / 2].y);
-      const float2 u = adjoint_pixel(au, transmission(hv[e], cc), v, cc, acc[e]);
+      const float2 u = adjoint_pixel(au, transmission<true>(hv[e], cc), v, cc, acc[e]);
       re[e] = u.x, im[e] = u.y;
     }
     if constexpr (!FIRST) {

@@ -78,7 +78,8 @@ __device__ __forceinline__ float ten_log10(double x) {
 constexpr int kLossKeep = 4096;
 // Up to this many detector pixels a channel gets a block of 128 threads, so that
 // twice as many channels are in flight (a thread then adds at most ten terms,
-// as one of 256 does at 50 x 50).
+// as one of 256 does at 50 x 50).  Not with the scaled loss: its sigma, and with
+// it dL/dI, would round differently for another order of the sums.
 constexpr int kLossSmall = 1280;
 
 // One block per channel: sum (D-T)^2, sigma = sum D T / sum D^2, sum (sigma D
@@ -201,9 +202,9 @@ cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, 
   const float scale = (float)(2.0 / norm);  // dL/dD = 2 (D - T) / norm
   const int det2 = (fov / bin) * (fov / bin);
   const size_t sm = det2 <= kLossKeep ? sizeof(float) * det2 : 0;
-  const bool small = det2 <= kLossSmall;
-  return launch_next(small ? k_loss<128> : k_loss<kRedThreads>, dim3(nw), small ? 128 : kRedThreads, sm, s, o, T, st, fov, bin, dLdI, scale, norm, mode, psnr, d_loss,
-                     ticket);
+  const bool small = det2 <= kLossSmall && mode != DOS_LOSS_MSE_SCALED;
+  return launch_next(small ? k_loss<128> : k_loss<kRedThreads>, dim3(nw), small ? 128 : kRedThreads, sm, s, o, T, st,
+                     fov, bin, dLdI, scale, norm, mode, psnr, d_loss, ticket);
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_loss_final(const LossStats* __restrict__ st, int nw,

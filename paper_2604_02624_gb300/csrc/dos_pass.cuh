@@ -62,6 +62,12 @@ __device__ __forceinline__ void sincos_turns(float f, float* s, float* c) {
 // The phase in cycles is formed as a float-pair product (exact product error
 // by fma) and reduced modulo 1 before the sine, which keeps ~1e-7 cycle
 // accuracy for any thickness.
+// LIB: sine and cosine by the library, for the split-BF16 path: its second
+// parts keep 8 bits of what the first left, so that a last-bit difference in t
+// turns, GEMM by GEMM, into other roundings of every second part (as large an
+// error, but another one: gradients of few channels moved by 2.9e-5 of their
+// norm).  Its field kernels are bound by memory and do not gain by the polynomial.
+template <bool LIB = false>
 __device__ __forceinline__ float2 transmission(float h, const ChanConst& cc) {
   const float p = cc.a_hi * h;
   float e = fmaf(cc.a_hi, h, -p);
@@ -69,7 +75,8 @@ __device__ __forceinline__ float2 transmission(float h, const ChanConst& cc) {
   float f = (p - rintf(p)) + (e + cc.pc_base);
   f -= rintf(f);
   float s, c;
-  sincos_turns(f, &s, &c);
+  if constexpr (LIB) sincospif(2.0f * f, &s, &c);
+  else sincos_turns(f, &s, &c);
   const float amp = exp2f(cc.amp_k * h) * cc.amp_base;
   return make_float2(amp * c, -amp * s);
 }
