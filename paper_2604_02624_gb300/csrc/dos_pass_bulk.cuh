@@ -4,14 +4,15 @@
 // block.  Blocks loop over several work items and the bulk-copy engine
 // (cp.async.bulk global -> shared, completion counted in bytes on an
 // mbarrier) fetches the next item while the block computes the current one:
-//   column pass : item = a mirrored pair of 8-column groups of one channel
-//                 (persistent blocks); tensor copies (TMA) of both groups'
-//                 input rows and of the transfer-table tile they share;
-//   row passes  : item = the block's RL rows of the next channel of its chunk;
-//                 one cp.async.bulk per row (rows padded in shared memory
-//                 against bank conflicts): spectra rows, the rows of the
-//                 input-field table in the first forward pass, and spectra
-//                 plus checkpoint rows in the adjoint pass.
+//   column pass : item = a group of 8 columns of one channel (persistent
+//                 blocks, items drawn from a counter); tensor copies (TMA) of
+//                 the group's input rows and of the transfer-table tile;
+//   row passes  : item = the block's RL rows of its next channel (drawn from a
+//                 counter in the forward passes, the next of a chunk in the
+//                 adjoint ones); one cp.async.bulk per row (rows padded in
+//                 shared memory against bank conflicts): spectra rows, the rows
+//                 of the input-field table in the first forward pass, and
+//                 spectra plus checkpoint rows in the adjoint pass.
 // One staging buffer per input suffices: the item is moved from the stage to
 // registers and the next copy is issued at the first block barrier after
 // that (the one inside the item's first line DFT), so the copy overlaps most
@@ -21,8 +22,7 @@
 // barrier after the wait), so that no thread goes on with an item another
 // thread gave up on: when any wait expires the whole block issues no further
 // copy, leaves its loop without writing partial results, waits once more
-// (bounded) for the copy it was waiting for (its only one in flight) and sets
-// *err.
+// (bounded) for its copies in flight and sets *err.
 // PassArgs::stall (fault injection for tests): 1 makes the blocks announce
 // their bytes without copying them, so that the first wait of every block
 // expires; 2 lets the copies land but makes the odd threads of every block
@@ -949,8 +949,9 @@ inline int balanced_chunk(int nw, int rb, int slots, int most) {
 constexpr int kRowChunk = 48;
 
 // Launchers.  The column pass runs one persistent block per resident slot
-// (blocks per SM from the occupancy calculator x SMs); the row passes run
-// (row blocks) x (channel chunks) blocks, each looping over its chunk.
+// (blocks per SM from the occupancy calculator x SMs), the forward row passes
+// with DRAW the resident slots shared out over the row blocks; the other row
+// passes run (row blocks) x (channel chunks) blocks, each looping over its chunk.
 template <class LF, int RL>
 struct PassBulkLaunch {
   using PB = PassBulk<LF, RL>;
