@@ -1,12 +1,13 @@
 // dos_gemm.cu - split-BF16 DFT-GEMM form of the propagation (tcgen05, TMEM).
 //
 // See dos_gemm.cuh for the formulation.  The GEMM kernel is persistent and
-// warp-specialised: one CTA per SM walks its share of the 128 x 256 output
-// tiles.  Warp 0 (one lane) streams the operands: both are kept in global
+// warp-specialised: one CTA per SM walks its share of the output tiles, 128 x
+// 256 or, for few tiles, 128 x 128 (narrow_tiles; the figures here are the wide
+// tile's).  Warp 0 (one lane) streams the operands: both are kept in global
 // memory tile by tile in the tensor core's K-major core-matrix order
 // (gemm_tiled), so a K chunk of 64 is two bulk copies (16 KB of A, 32 KB of B,
 // cp.async.bulk with completion counted in bytes on the stage's "full"
-// mbarrier) into a GSTAGES-deep ring.  Warp 1 (one lane) issues the MMAs into
+// mbarrier) into a ring of four.  Warp 1 (one lane) issues the MMAs into
 // one of two TMEM accumulators (2 x 256 columns) and frees each stage through
 // tcgen05.commit on its "empty" mbarrier; a commit on "acc_full" hands a
 // finished accumulator to the sixteen epilogue warps, which drain it (warp w
@@ -26,8 +27,10 @@
 
 namespace dos {
 
-constexpr int GTM = 128, GTN = 256, GTK = 64;  // one tile and MMA: 128 x 256, K steps of 16
-constexpr int GSTAGES = 4;                      // 48 KB per stage
+// One tile and MMA: 128 x TN, K steps of 16; TN = 256, or 128 (narrow_tiles).
+constexpr int GTM = 128, GTK = 64;
+template <int TN>
+constexpr int gstages() { return TN == 256 ? 4 : 6; }  // of 48 or 32 KB
 constexpr int kEpiWarps = 16;                   // 4 per TMEM lane quarter, a quarter of the columns each
 constexpr int kGemmThreads = 32 * (2 + kEpiWarps);
 constexpr long kSpinLimit = 1L << 26;           // bounded mbarrier wait (a fraction of a second)
@@ -40,9 +43,11 @@ __device__ __forceinline__ uint64_t kmajor_desc(uint32_t saddr) {
          ((uint64_t)1 << 46);
 }
 
-// kind::f16 instruction descriptor: D f32, A and B bf16, both K-major, N = 256, M = 128
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GTN >> 3) << 17) |
-                            ((uint32_t)(GTM >> 4) << 24);
+// kind::f16 instruction descriptor: D f32, A and B bf16, both K-major, N = TN, M = 128
+template <int TN>
+constexpr uint32_t idesc() {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(GTM >> 4) << 24);
+}
 
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t done;
@@ -75,9 +80,11 @@ __device__ __forceinline__ void bulk_tile(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
+template <int TN>
 struct __align__(1024) GemmSmem {
+  static constexpr int GSTAGES = gstages<TN>();
   uint8_t a[GSTAGES][GTM * GTK * 2];  // 16 KB per stage
-  uint8_t b[GSTAGES][GTN * GTK * 2];  // 32 KB per stage
+  uint8_t b[GSTAGES][TN * GTK * 2];   // 32 or 16 KB per stage
   uint64_t full[GSTAGES];             // copies of the stage landed
   uint64_t empty[GSTAGES];            // MMAs reading the stage done
   uint64_t acc_full[2];               // accumulator ready for the epilogue
@@ -240,15 +247,16 @@ __device__ __forceinline__ void tmem_load(uint32_t addr, uint32_t (&u)[CW]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
-template <int MODE>
+template <int MODE, int TN>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_constant__ GemmArgs g) {
+  constexpr int GSTAGES = gstages<TN>();
   extern __shared__ __align__(1024) uint8_t gsm_raw[];
-  GemmSmem& sm = *reinterpret_cast<GemmSmem*>(gsm_raw);
+  GemmSmem<TN>& sm = *reinterpret_cast<GemmSmem<TN>*>(gsm_raw);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   volatile int* abort = &sm.abort;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sm.tmem)),
-                 "r"(2 * GTN));
+                 "r"(2 * TN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 32) {
@@ -272,7 +280,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
   const int total = g.nseg * kchunks;  // K chunks per tile
   // tiles, the DFT matrix's (few) tiles the fast index: the CTAs that share a
   // data tile run together
-  const int tilesA = g.rows / GTM, tilesB = (g.cols + GTN - 1) / GTN;
+  const int tilesA = g.rows / GTM, tilesB = (g.cols + TN - 1) / TN;
   const int ntiles = tilesA * tilesB;
   auto tile_of = [&](int t, int& mt, int& nt) {
     if (g.w_is_b) {
@@ -302,11 +310,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
           }
           const int seg = it / kchunks, kc = it % kchunks;
           const uint32_t fb = smem_addr(&sm.full[st]);
-          bar_expect_tx(fb, (GTM + GTN) * GTK * 2);
-          // 128-row A tile mt: half (mt & 1) of the stored 256-row tile mt / 2
+          bar_expect_tx(fb, (GTM + TN) * GTK * 2);
+          // 128-row A tile mt: half (mt & 1) of the stored 256-row tile mt / 2, and so B tile nt of TN = 128
           bulk_tile(sm.a[st], g.a[seg] + (((size_t)(mt >> 1) * kchunks + kc) << 14) + ((size_t)(mt & 1) << 13),
                     GTM * GTK * 2, fb);
-          bulk_tile(sm.b[st], g.b[seg] + (((size_t)nt * kchunks + kc) << 14), GTN * GTK * 2, fb);
+          const size_t bt = TN == 256 ? (((size_t)nt * kchunks + kc) << 14)
+                                      : (((size_t)(nt >> 1) * kchunks + kc) << 14) + ((size_t)(nt & 1) << 13);
+          bulk_tile(sm.b[st], g.b[seg] + bt, TN * GTK * 2, fb);
           last[st] = c;
         }
       }
@@ -328,7 +338,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t acc0 = tmem + (uint32_t)(b * GTN);
+        const uint32_t acc0 = tmem + (uint32_t)(b * TN);
         for (int it = 0; it < total; ++it, ++c) {
           const int st = c % GSTAGES;
           if (!mbar_wait(smem_addr(&sm.full[st]), (uint32_t)((c / GSTAGES) & 1), abort)) {
@@ -344,7 +354,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
             asm volatile(
                 "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc0),
-                "l"(da), "l"(db), "r"(kIdesc), "r"(acc));
+                "l"(da), "l"(db), "r"(idesc<TN>()), "r"(acc));
           }
           last_bar = smem_addr(&sm.empty[st]);
           last_par = (uint32_t)((c / GSTAGES) & 1);
@@ -370,26 +380,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
       int mt, nt;
       tile_of(t, mt, nt);
       const int r = mt * GTM + q * 32 + lane;  // accumulator row of this thread
-      const int cbeg = part * (GTN / 4), cend = cbeg + GTN / 4;
+      const int cbeg = part * (TN / 4), cend = cbeg + TN / 4;
       float2 hv[8];
       if constexpr (MODE == GEMM_OUT_SPECTRUM) {
-        if (r < g.vrows) spectrum_h(g, r, nt * GTN + cbeg, hv);  // before the wait for the accumulator
+        if (r < g.vrows) spectrum_h(g, r, nt * TN + cbeg, hv);  // before the wait for the accumulator
       }
       if (!mbar_wait(smem_addr(&sm.acc_full[b]), (uint32_t)((tc >> 1) & 1), abort)) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll 1
       for (int c0 = cbeg; c0 < cend; c0 += CW) {
         uint32_t u[CW];
-        tmem_load<CW>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * GTN + c0), u);
+        tmem_load<CW>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TN + c0), u);
         float2 hn[8];
         if constexpr (MODE == GEMM_OUT_SPECTRUM) {
-          if (c0 + CW < cend && r < g.vrows) spectrum_h(g, r, nt * GTN + c0 + CW, hn);
+          if (c0 + CW < cend && r < g.vrows) spectrum_h(g, r, nt * TN + c0 + CW, hn);
         }
         if (r < g.vrows) {
           float v[CW];
 #pragma unroll
           for (int j = 0; j < CW; ++j) v[j] = __uint_as_float(u[j]);
-          epilogue<MODE>(g, r, nt * GTN + c0, v, hv);
+          epilogue<MODE>(g, r, nt * TN + c0, v, hv);
         }
         if constexpr (MODE == GEMM_OUT_SPECTRUM) {
 #pragma unroll
@@ -405,21 +415,42 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_tc_gemm(const __grid_consta
   __syncthreads();
   if (tid == 0 && sm.abort) atomicExch(g.err, 1);
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * GTN));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TN));
+}
+
+// Column width of the tiles.  A launch runs in waves of one tile per SM.  A
+// narrow tile took 0.70 to 0.73 of a wide one's time in launches of many waves
+// (each MMA reads the whole A tile for half the columns), so narrow tiles are
+// taken where they need less than 1 / kNarrow as many waves: mostly where both
+// are one wave, or where the wide tiles leave half the chip idle.  A step of
+// three layers, wide / narrow in every launch / by this rule: 4 x 256 551 / 483 /
+// 483 us, 24 x 200 (three parts) 965 / 1345 / 960, 128 x 256 3742 / 5453 / 3749.
+constexpr double kNarrow = 0.8;
+static bool narrow_tiles(const GemmArgs& g, int sms) {
+  const long rows = g.rows / GTM;
+  const long wide = (rows * ((g.cols + 255) / 256) + sms - 1) / sms;
+  const long narrow = (rows * ((g.cols + 127) / 128) + sms - 1) / sms;
+  return kNarrow * (double)narrow < (double)wide;
+}
+
+template <int MODE, int TN>
+static cudaError_t launch_tiles(const GemmArgs& g, int sms, cudaStream_t s) {
+  const size_t sm = sizeof(GemmSmem<TN>) + 1024;
+  const cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<MODE, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const int tiles = (g.rows / GTM) * ((g.cols + TN - 1) / TN);
+  return launch_next(k_tc_gemm<MODE, TN>, dim3(std::min(tiles, sms)), kGemmThreads, sm, s, g);
 }
 
 template <int MODE>
 static cudaError_t launch_mode(const GemmArgs& g, cudaStream_t s) {
   // attribute and SM count of the current device, every launch (contexts may
   // live on different devices of one process; both calls are host-side only)
-  const size_t sm = sizeof(GemmSmem) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   int dev = 0, sms = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int tiles = (g.rows / GTM) * ((g.cols + GTN - 1) / GTN);
-  return launch_next(k_tc_gemm<MODE>, dim3(std::min(tiles, sms)), kGemmThreads, sm, s, g);
+  return narrow_tiles(g, sms) ? launch_tiles<MODE, 128>(g, sms, s) : launch_tiles<MODE, 256>(g, sms, s);
 }
 
 cudaError_t launch_tc_gemm(const GemmArgs& g, cudaStream_t s) {
