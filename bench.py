@@ -37,30 +37,23 @@ sys.path.insert(0, ROOT)
 TRAFFIC_PER_CHANNEL = {
     # One capture of every bulk pass of a step (dram__bytes_read + write per
     # launch / 256 channels), each kind averaged over its launches.
-    # 200 -> 400, K = 5: forward column 1.3875 / 1.3875 / 1.3887 / 1.3872 MB and
-    # 1.0646 MB (last gap, field-of-view output rows); adjoint column 0.9075 MB
-    # (first gap, field-of-view input rows) and 1.3876 / 1.3883 / 1.3874 / 1.3904 MB;
-    # forward row 0.7277 MB (first pass, from the input-field table) and 1.3579 /
-    # 1.3580 / 1.3577 / 1.3583 MB; adjoint row 1.4205 / 1.4195 / 1.4215 / 1.4203 MB
-    # and 0.9861 MB (layer 1: no spectra written back)
-    ("column_bulk", 200, 400, "column_forward"): ((1.3875e6 + 1.3875e6 + 1.3887e6 + 1.3872e6 + 1.0646e6) / 5,
-                                                  "profiles/column_pass_bulk_batched.md"),
-    ("column_bulk", 200, 400, "column_adjoint"): ((0.9075e6 + 1.3876e6 + 1.3883e6 + 1.3874e6 + 1.3904e6) / 5,
-                                                  "profiles/column_pass_bulk_batched.md"),
-    ("row_bulk", 200, 400, "row_forward"): ((0.7277e6 + 1.3579e6 + 1.3580e6 + 1.3577e6 + 1.3583e6) / 5,
-                                            "profiles/row_passes_batched.md"),
-    ("row_bulk", 200, 400, "row_adjoint"): ((1.4205e6 + 1.4195e6 + 1.4215e6 + 1.4203e6 + 0.9861e6) / 5,
-                                            "profiles/row_passes_batched.md"),
+    # 200 -> 400, K = 5: forward column 1.3893-1.3897 MB and 1.0663 MB (last gap,
+    # field-of-view output rows); adjoint column 0.9086 MB (first gap, field-of-view
+    # input rows) and 1.3891-1.3908 MB; forward row 0.7270 MB (first pass, from the
+    # input-field table) and 1.3586-1.3603 MB; adjoint row 1.3810-1.3826 MB and
+    # 0.9620 MB (layer 1: no spectra written back)
+    ("column_bulk", 200, 400, "column_forward"): (1.3248e6, "profiles/column_pass_bulk_batched.md"),
+    ("column_bulk", 200, 400, "column_adjoint"): (1.2936e6, "profiles/column_pass_bulk_batched.md"),
+    ("row_bulk", 200, 400, "row_forward"): (1.2330e6, "profiles/row_passes_batched.md"),
+    ("row_bulk", 200, 400, "row_adjoint"): (1.2978e6, "profiles/row_passes_batched.md"),
     # 256 -> 512, K = 8 (the precision geometry with 256 channels): forward column
-    # 2.4101 / 2.4105 / 2.4089 / 2.4096 / 2.4093 / 2.4098 / 2.4090 MB and 1.7779 MB;
-    # adjoint column 1.6248 MB and 2.4096 / 2.4094 / 2.4101 / 2.4092 / 2.4092 /
-    # 2.4092 / 2.4098 MB; forward row 1.3346 MB and 2.3736 / 2.3727 / 2.3729 /
-    # 2.3733 / 2.3738 / 2.3720 / 2.3721 MB; adjoint row 2.4562 / 2.4547 / 2.4545 /
-    # 2.4558 / 2.4562 / 2.4542 / 2.4540 MB and 1.6203 MB
-    ("column_bulk", 256, 512, "column_forward"): (2.33064e6, "profiles/column_pass_m512_precision.md"),
-    ("column_bulk", 256, 512, "column_adjoint"): (2.31141e6, "profiles/column_pass_m512_precision.md"),
-    ("row_bulk", 256, 512, "row_forward"): (2.24313e6, "profiles/row_passes_m512_precision.md"),
-    ("row_bulk", 256, 512, "row_adjoint"): (2.35074e6, "profiles/row_passes_m512_precision.md"),
+    # 2.4144-2.4159 MB and 1.7846 MB; adjoint column 1.6263 MB and 2.4142-2.4157 MB;
+    # forward row 1.3377 MB and 2.3698-2.3707 MB; adjoint row 2.4004-2.4105 MB and
+    # 1.5754 MB
+    ("column_bulk", 256, 512, "column_forward"): (2.3362e6, "profiles/column_pass_m512_precision.md"),
+    ("column_bulk", 256, 512, "column_adjoint"): (2.3162e6, "profiles/column_pass_m512_precision.md"),
+    ("row_bulk", 256, 512, "row_forward"): (2.2411e6, "profiles/row_passes_m512_precision.md"),
+    ("row_bulk", 256, 512, "row_adjoint"): (2.3030e6, "profiles/row_passes_m512_precision.md"),
 }
 
 

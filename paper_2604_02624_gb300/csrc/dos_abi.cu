@@ -145,7 +145,7 @@ struct dos_ctx {
   bool in_step = false;  // a step is being captured: its gradient reduction keeps the thickness
   dos::LossStats* stats = nullptr;
   double* d_loss = nullptr;
-  // items drawn in the running column pass and, from [1], chunks drawn per row
+  // items drawn in the running column pass and, from [1], channels drawn per row
   // block (at most one for each layer row) in the running row pass; zero
   // between launches
   unsigned* counters = nullptr;

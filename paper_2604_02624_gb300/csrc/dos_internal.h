@@ -115,7 +115,7 @@ struct PassArgs {
   bool displaced;         // column pass: the gap carries a displacement that Hq does not hold (mis)
   Misalign mis;           // its lateral shift; and, with mis.sq, its length change (plain kernel only)
   unsigned* work;         // item counter of the bulk column pass, 0 between launches
-  unsigned* row_work;     // chunk counters of the bulk row passes, one per row block, 0 between launches
+  unsigned* row_work;     // channel counters of the bulk forward row passes, one per row block, 0 between launches
   int* err;               // set to 1 by a bulk-copy pass whose bounded wait expired
   int stall;              // fault injection (tests): 1 = the bulk pass expects bytes that are never
                           // copied; 2 = its copies land but odd threads give up their first wait;
