@@ -555,6 +555,9 @@ int build(dos_ctx* x, const dos_config* c) {
   DOS_CUDA(dos::launch_arow(x->arow, x->m, x->oa, x->ap, x->stream), "aperture spectrum");
   DOS_CUDA(dos::launch_twiddles(x->tw, x->ops->P, x->ops->Q, dos::twiddle_pitch(x->ops->P), x->m, x->stream),
            "twiddles");
+  // Everything that a kernel launched by launch_next reads before pdl_wait (the
+  // twiddles) is complete before the first such launch of the context.
+  DOS_CUDA(cudaStreamSynchronize(x->stream), "create");
   if (!gemm) {
     // v1: the aperture's separable spectrum through gap 0, inverse row DFT, crop
     if ((rc = x->alloc(&x->v1, (size_t)x->nw * n2, "input field"))) return rc;

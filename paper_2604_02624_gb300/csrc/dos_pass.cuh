@@ -126,8 +126,9 @@ struct Pass {
   static constexpr size_t smem_bytes(int lines) { return sizeof(float2) * (LF::TWS + (size_t)lines * ZL); }
   static constexpr size_t row_smem_bytes(int lines) { return sizeof(float2) * (LF::TWS + (size_t)lines * RZL); }
 
-  // the start of every kernel: the twiddles (made at create) do not depend on
-  // the grid before this one
+  // the start of every kernel: the twiddles are read ahead of the wait; dos_create
+  // made them and synchronised before any of these kernels ran, so no grid before
+  // this one can still be writing them
   __device__ static __forceinline__ void load_tw(float2* tw, const float2* g) {
     for (int i = threadIdx.x; i < LF::TWS; i += blockDim.x) tw[i] = g[i];
     pdl_wait();
