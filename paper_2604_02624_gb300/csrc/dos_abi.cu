@@ -589,7 +589,6 @@ int flag_after_sync(dos_ctx* c) {
   if (*c->h_err) {
     *c->h_err = 0;
     DOS_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream), "error flag");
-    DOS_CUDA(cudaMemsetAsync(c->counters, 0, sizeof(unsigned) * (1 + (size_t)c->n), c->stream), "work counters");
     return fail(DOS_ERR_TIMEOUT, "a bounded wait gave up (mbarrier wait for a tensor-core commit or a bulk copy "
                                  "expired); results of the call are invalid");
   }

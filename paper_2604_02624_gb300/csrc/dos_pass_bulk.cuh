@@ -89,6 +89,40 @@ __device__ __forceinline__ bool split_verdict(const PassArgs& a, int item) {
   return a.stall == 2 && item == 0 && (threadIdx.x & 1);
 }
 
+// Items 0 .. items - 1 of a launch, taken in order by whichever of its blocks is
+// free: block b has item b, the others' numbers come from a counter that is zero
+// between launches.  A block's thread 0 draws ahead; every block draws until its
+// first number past the end, items draws in all, and whoever drew the last one
+// sets the counter back to zero.  A block that gives up (an expired wait) goes
+// on drawing without working (drain), so that this holds for it as well and the
+// next launch, which may be queued before the host has seen the error, starts
+// from zero.
+struct Draws {
+  unsigned* work;
+  unsigned blocks, items;
+  unsigned drawn;  // the counter's latest answer, taken by ahead()
+  DOS_HD void ahead() {
+#ifdef __CUDA_ARCH__
+    drawn = atomicAdd(work, 1u);
+#else
+    drawn = (*work)++;
+#endif
+  }
+  // the item of the latest number (items: none is left)
+  DOS_HD unsigned item() const {
+    if (drawn == items - 1u) *work = 0u;
+    const unsigned n = drawn + blocks;
+    return n < items ? n : items;
+  }
+  // gives up: n is the item of the latest number
+  DOS_HD void drain(unsigned n) {
+    while (n < items) {
+      ahead();
+      n = item();
+    }
+  }
+};
+
 // Row stride of the row passes' staging buffer: a warp reads the rows of two
 // or more lines at once, and these strides make those 8-byte reads free of
 // bank conflicts (enumerated on the host for the compiled line shapes).
@@ -268,21 +302,18 @@ struct PassBulk {
     };
     bool ok = true;
     int k = 0, issued_s = 0, issued_h = 0, done_s = 0, done_h = 0;  // copies per barrier (thread 0's view)
-    // Items are taken in order by whichever block is free: the first gridDim by
-    // block index, the others from a counter.  (Blocks that stepped through
-    // the items by gridDim finished far apart: SMs differ in how far they are
+    // Items are drawn (Draws).  (Blocks that stepped through the items by
+    // gridDim finished far apart: SMs differ in how far they are
     // from the memory they read, and 16 of 20 warps were resident on average.
     // 4096 x 200 launch 1.50 -> 1.34 ms, 256 x 200 103 -> 94 us, 2048 x 256
     // 1.19 -> 1.10 ms.)
     // Thread 0 draws two items ahead, so that the counter's answer is there
-    // when the next copy is issued.  Every block draws until its first number
-    // past the end, items draws in all: whoever drew the last one leaves the
-    // counter at 0.
-    unsigned drawn = 0;  // thread 0: the counter's answer for the item after the current one
+    // when the next copy is issued.
+    Draws draws{a.work, gridDim.x, (unsigned)items, 0u};  // thread 0: the item after the current one
     if (leader) {
       fetch_s(blockIdx.x);
       if constexpr (STAGE_H) fetch_h(blockIdx.x);
-      drawn = atomicAdd(a.work, 1u);
+      draws.ahead();
     }
     issued_s = 1;
     issued_h = STAGE_H ? 1 : 0;
@@ -291,10 +322,7 @@ struct PassBulk {
       place(it, w, c0);
       const int cc = c0 + lc;  // this line's column
       const int hc = min(cc, M - cc) - table_row(c0);  // |kx|'s row of the H tile
-      if (leader) {
-        *next_item = (int)min(drawn + gridDim.x, (unsigned)items);
-        if (drawn == (unsigned)items - 1u) *a.work = 0u;
-      }
+      if (leader) *next_item = (int)draws.item();
       // this item's input rows; a thread whose wait expires goes on to the
       // barrier with what is there, where the whole block stops
       const bool got_s = bulk_wait(&bar[0], (uint32_t)(k & 1), split_verdict(a, k));
@@ -318,7 +346,7 @@ struct PassBulk {
         if (leader) fetch_s(next);
         ++issued_s;
       }
-      if (leader && more) drawn = atomicAdd(a.work, 1u);
+      if (leader && more) draws.ahead();
       LF::template step2<false, LF::Q, PKC, false, ZX>(r, t, z);
       // (injected, tests: the wait of the block's last item gives up)
       const bool got_h = (a.stall == 3 && !more) ? false : bulk_wait(&bar[1], (uint32_t)(k & 1));
@@ -371,7 +399,9 @@ struct PassBulk {
       it = next;
     }
     if (!ok && leader) {
-      // (the counter is left where it is: the host zeroes it with the flag)
+      // the number drawn after the first barrier has not been looked at when the block leaves at the second
+      const unsigned n = *next_item;
+      draws.drain(done_s > done_h && n < draws.items ? draws.item() : n);
       // the copies in flight land (bounded waits) before the block leaves
       if (issued_s > done_s) (void)bulk_wait(&bar[0], (uint32_t)(done_s & 1));
       if (issued_h > done_h) (void)bulk_wait(&bar[1], (uint32_t)(done_h & 1));
@@ -382,10 +412,9 @@ struct PassBulk {
   // ------------------------------------------------------------- row passes
   // Block (x, y) of a forward pass holds the rows [x RL, +RL).  With up to 20
   // elements per thread (DRAW) the blocks are persistent and take channel y,
-  // then whatever a counter of their row block says, as the column pass does:
-  // thread 0 draws two channels ahead, publishes the next one before the first
-  // barrier of the current one, and whoever draws the last number (a.nw of them
-  // per row block in all) leaves the counter at 0.  4096 x 200 launch 0.931 ->
+  // then whatever a counter of their row block says (Draws), as the column pass
+  // does: thread 0 draws two channels ahead and publishes the next one before the
+  // first barrier of the current one.  4096 x 200 launch 0.931 ->
   // 0.901 ms, 1024 x 200 236 -> 225 us, 256 x 200 70.5 -> 67.5 us.  At M = 512 that
   // was slower (2048 x 256 0.848 -> 0.866 ms): there block (x, y) takes the
   // channels of chunk y.  (The adjoint passes sum a fixed chunk of channels per
@@ -393,16 +422,16 @@ struct PassBulk {
   // chunks were slower: 4096 x 200 1.05 -> 1.12 ms.)
   static constexpr bool DRAW = LF::E <= 20;
   struct Draw {
-    unsigned* work;  // this row block's counter
+    Draws draws;     // thread 0: this row block's counter, the channel after the current one
     int* next_sh;    // published next channel
-    unsigned drawn;  // thread 0: the counter's answer for the channel after the current one
     int w;           // current channel
     int nw, end;     // channels; end of the chunk (not DRAW)
-    __device__ __forceinline__ Draw(const PassArgs& a, int* sh) : work(a.row_work + blockIdx.x), next_sh(sh), drawn(0) {
+    __device__ __forceinline__ Draw(const PassArgs& a, int* sh)
+        : draws{a.row_work + blockIdx.x, gridDim.y, (unsigned)a.nw, 0u}, next_sh(sh) {
       nw = a.nw;
       if constexpr (DRAW) {
         w = blockIdx.y;
-        if (threadIdx.x == 0) drawn = atomicAdd(work, 1u);
+        if (threadIdx.x == 0) draws.ahead();
       } else {
         w = blockIdx.y * a.chunk;
         end = min(nw, w + a.chunk);
@@ -411,14 +440,17 @@ struct PassBulk {
     // thread 0, before the first barrier of a channel
     __device__ __forceinline__ void publish() {
       if (!DRAW || threadIdx.x != 0) return;
-      *next_sh = (int)min(drawn + gridDim.y, (unsigned)nw);
-      if (drawn == (unsigned)nw - 1u) *work = 0u;
+      *next_sh = (int)draws.item();
+    }
+    // thread 0, when the block gives up at that barrier
+    __device__ __forceinline__ void give_up() {
+      if constexpr (DRAW) draws.drain((unsigned)*next_sh);
     }
     // every thread, after that barrier: the channel that follows (nw: none)
     __device__ __forceinline__ int next() {
       if constexpr (!DRAW) return w + 1 < end ? w + 1 : nw;
       const int n = *next_sh;
-      if (threadIdx.x == 0 && n < nw) drawn = atomicAdd(work, 1u);
+      if (threadIdx.x == 0 && n < nw) draws.ahead();
       return n;
     }
   };
@@ -515,7 +547,7 @@ struct PassBulk {
       draw.w = wn;
     }
     if (!okw && threadIdx.x == 0) {
-      // (the counter is left where it is: the host zeroes it with the flag)
+      draw.give_up();
       (void)bulk_wait(bar, (uint32_t)(k & 1));  // a late copy lands (bounded) before the block leaves
       atomicExch(a.err, 1);
     }
@@ -700,6 +732,7 @@ struct PassBulk {
       draw.w = wn;
     }
     if (!okw && threadIdx.x == 0) {
+      draw.give_up();
       (void)bulk_wait(bar, (uint32_t)(k & 1));  // a late copy lands (bounded) before the block leaves
       atomicExch(a.err, 1);
     }
