@@ -248,6 +248,14 @@ struct dos_ctx {
     *p = static_cast<T*>(q);
     return DOS_OK;
   }
+  // gives back what alloc(p, count) took, and clears p
+  template <typename T>
+  void dealloc(T** p, size_t count) {
+    allocs.erase(std::find(allocs.begin(), allocs.end(), static_cast<void*>(*p)));
+    bytes -= std::max<size_t>(count, 1) * sizeof(T);
+    cudaFree(*p);
+    *p = nullptr;
+  }
   void release() {
     cudaStreamSynchronize(stream);
     if (gstream) cudaStreamSynchronize(gstream);
@@ -1356,19 +1364,27 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
     if (!std::isfinite(disp[i])) return fail(DOS_ERR_ARG, "displacements must be finite");
   if (!c->sq) {
     const size_t count = (size_t)c->nw * c->hs * c->hs;
-    if ((rc = c->alloc(&c->sq, count, "root table"))) return rc;
+    float* roots = nullptr;  // c->sq once its kernel is queued
+    if ((rc = c->alloc(&roots, count, "root table"))) return rc;
     // the column passes' tables: where they do not fit, the plain kernel does without
     if ((c->call_choice < 0 || c->step_choice < 0) &&  // the multi-pass choices
         c->alloc(&c->sq_lo, count, "root table") == DOS_OK) {
       for (int tables : {c->K + 1, 1}) {
         if (c->alloc(&c->hmis, tables * count, "displaced transfer tables") != DOS_OK) continue;
-        if (c->have_tmap && (rc = make_table_map(c, &c->tmap_Hm, c->hmis, tables))) return rc;
-        c->mis_tables = tables;
+        if (!c->have_tmap || make_table_map(c, &c->tmap_Hm, c->hmis, tables) == DOS_OK) c->mis_tables = tables;
+        else c->dealloc(&c->hmis, tables * count);  // as where they do not fit
         break;
       }
+      if (c->mis_tables == 0) c->dealloc(&c->sq_lo, count);
     }
-    DOS_CUDA(dos::launch_sqtable(c->sq, c->sq_lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream),
-             "root table");
+    const cudaError_t e = dos::launch_sqtable(roots, c->sq_lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream);
+    if (e != cudaSuccess) {
+      // nothing is kept: the next call makes the tables again
+      c->dealloc(&roots, count);
+      if (c->mis_tables) c->dealloc(&c->hmis, c->mis_tables * count), c->dealloc(&c->sq_lo, count), c->mis_tables = 0;
+      return fail(DOS_ERR_CUDA, std::string("root table: ") + cudaGetErrorString(e));
+    }
+    c->sq = roots;
   }
   // layer l (1..K) displaced by D_l; planes 0 (aperture) and K+1 (detector) fixed:
   // gap g carries the lateral shift D_g - D_{g+1} and the length change dz_{g+1} - dz_g

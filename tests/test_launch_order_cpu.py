@@ -39,3 +39,11 @@ def test_nothing_but_parameters_and_twiddles_is_read_before_the_wait():
             assert all(r in (("tw", ""),) for r in reads), (name, head[-400:])
             seen += 1
     assert seen >= 12
+
+
+def test_the_root_table_is_in_place_only_when_its_kernel_is_queued():
+    """A failed first use of displaced layers must not leave a table that looks
+    made: the context's pointer is set after the launch that fills it."""
+    src = _code("dos_abi.cu")
+    assert "alloc(&c->sq," not in src
+    assert 0 < src.index("launch_sqtable(") < src.index("c->sq = ")
