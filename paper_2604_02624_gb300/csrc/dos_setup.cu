@@ -17,6 +17,14 @@
 
 namespace dos {
 
+// (n/lambda)^2 - fx^2 - fy^2, the same bits in either order of fx and fy: the bulk
+// column pass reads a column of the quadrant tables made from it as a row.  Each
+// operation is rounded by itself (contracted to an FMA, the sum of the squares
+// would depend on their order), fx^2 + fy^2 first.
+__device__ __forceinline__ double bin_q(double k2, double fa, double fb) {
+  return __dsub_rn(k2, __dadd_rn(__dmul_rn(fa, fa), __dmul_rn(fb, fb)));
+}
+
 __global__ void k_htable(float2* __restrict__ Hq, const double* __restrict__ lam, double z,
                          double n_medium, double pitch, int m, int hs, int evanescent) {
   const int w = blockIdx.y;
@@ -28,9 +36,7 @@ __global__ void k_htable(float2* __restrict__ Hq, const double* __restrict__ lam
   const double fa = a * df;
   for (int b = threadIdx.x; b < hs; b += blockDim.x) {
     const double fb = b * df;
-    // fx^2 + fy^2 first: the table is exactly symmetric, H(a, b) = H(b, a)
-    // (the bulk column pass reads a quadrant column as a table row)
-    const double q = k2 - (fa * fa + fb * fb);
+    const double q = bin_q(k2, fa, fb);
     float2 h;
     if (q >= 0.0) {
       const double cyc = z * sqrt(q);
@@ -64,7 +70,7 @@ __global__ void k_sqtable(float* __restrict__ sq, float* __restrict__ sq_lo, con
   const double fa = a * df;
   for (int b = threadIdx.x; b < hs; b += blockDim.x) {
     const double fb = b * df;
-    const double q = k * k - fa * fa - fb * fb;
+    const double q = bin_q(k * k, fa, fb);
     const double r = q >= 0.0 ? sqrt(q) : -sqrt(-q);
     const size_t at = ((size_t)w * hs + a) * hs + b;
     sq[at] = (float)r;
