@@ -200,18 +200,21 @@ struct dos_ctx {
   double* d_lam = nullptr;      // wavelengths on the device (kept for the root table)
   float* sq = nullptr;          // signed sqrt(|q|) quadrant table, built on first use
   bool mis_on = false;
-  float* sq_lo = nullptr;       // what the roots' rounding to FP32 left (with hmis)
+  float* sq_lo = nullptr;       // what the roots' rounding to FP32 left (with the first of hmis)
   std::vector<double> mis;      // (K+1) x 3 per gap: lateral shift x, y and length change [m]
   long mis_gen = 0;
-  // transfer tables with the displaced gaps' length changes, for the column
-  // passes: [mis_tables][nw][hs][hs], gap g's in slot g % mis_tables; one per
-  // gap where they fit, else one that every pass rebuilds, else none (the plain
-  // kernel then forms the factor from sq).  A forward builds its gaps' tables
-  // anew; the adjoint of the same displacement reads them.
-  float2* hmis = nullptr;
-  int mis_tables = 0;
-  long mis_built = -1;        // mis_gen of the tables in place (mis_tables > 1)
-  CUtensorMap tmap_Hm;        // hmis as [mis_tables * nw][hs][hs], box as tmap_H
+  // Transfer tables [nw][hs][hs] with the displaced gaps' length changes, for the
+  // column passes, reserved when a displacement first needs them (need_tables):
+  // one for each gap whose length it changes, else one that every pass rebuilds
+  // (mis_shared), else none (the plain kernel then forms the factor from sq).  A
+  // forward builds its gaps' tables anew; the adjoint of the same displacement
+  // reads them.
+  std::vector<float2*> hmis;
+  std::vector<CUtensorMap> tmap_Hm;  // each as [nw][hs][hs], box as tmap_H
+  std::vector<int> mis_table;        // gap -> table under the current displacement, or -1
+  bool mis_shared = false;
+  int mis_most = 0;                  // tables that may be kept (DOS_DISPLACED_TABLES)
+  long mis_built = -1;               // mis_gen of the tables in place (not mis_shared)
   dos::Misalign gap_mis(int g) const {
     dos::Misalign m;
     std::memset(&m, 0, sizeof(m));
@@ -580,6 +583,8 @@ int build(dos_ctx* x, const dos_config* c) {
   DOS_CUDA(cudaStreamSynchronize(x->stream), "create");
   if ((rc = choose_path(x, c->path))) return rc;
   DOS_CUDA(cudaStreamSynchronize(x->stream), "create");
+  const char* most = std::getenv("DOS_DISPLACED_TABLES");
+  x->mis_most = (most && *most) ? std::atoi(most) : x->K + 1;
   const char* inj = std::getenv("DOS_INJECT_WAIT_TIMEOUT");
   x->inject_stall = (inj && *inj) ? (std::string(inj) == "2"   ? 2
                                      : std::string(inj) == "3" ? 3
@@ -759,7 +764,7 @@ void build_tables(dos_ctx* c, int g0, int g1, int w0, int nw, int kind, std::vec
     for (int g = g0; g <= g1; ++g) {
       const dos::Misalign m = c->gap_mis(g);
       if (c->gap_slot[g] != slot || m.dz == 0.f) continue;
-      t.out[t.n] = c->hmis + ((size_t)(g % c->mis_tables) * c->nw + w0) * hs2;
+      t.out[t.n] = c->hmis[c->mis_table[g]] + (size_t)w0 * hs2;
       t.dz[t.n++] = m.dz2;
       if (t.n == dos::kLongerTables) flush();
     }
@@ -782,16 +787,16 @@ void use_gap(dos_ctx* c, dos::PassArgs& a, int g, int w0, int kind, std::vector<
     a.mis.sq = nullptr;
     return;
   }
-  if (c->mis_tables == 0) {
+  const int slot = c->mis_table[g];
+  if (slot < 0) {
     a.mis.sq = c->sq + (size_t)w0 * hs2;
     a.displaced = true;
     return;
   }
-  if (c->mis_tables == 1 || c->mis_built != c->mis_gen) build_tables(c, g, g, w0, a.nw, kind, L);
-  const int slot = g % c->mis_tables;
-  a.Hq = c->hmis + ((size_t)slot * c->nw + w0) * hs2;
-  a.hmap = c->have_tmap ? &c->tmap_Hm : nullptr;
-  a.hmap_z0 = slot * c->nw + w0;
+  if (c->mis_shared || c->mis_built != c->mis_gen) build_tables(c, g, g, w0, a.nw, kind, L);
+  a.Hq = c->hmis[slot] + (size_t)w0 * hs2;
+  a.hmap = c->have_tmap ? &c->tmap_Hm[slot] : nullptr;
+  a.hmap_z0 = w0;
   a.mis.sq = nullptr;
   a.mis.dz = 0.f;
 }
@@ -802,7 +807,7 @@ std::vector<Launch> forward_launches(dos_ctx* c, const float* d_h, float* d_I, i
   const size_t n2 = (size_t)c->n * c->n;
   std::vector<Launch> L;
   dos::PassArgs a = range_args(c, w0, w1);
-  if (c->mis_on && c->mis_tables > 1) {
+  if (c->mis_on && !c->mis_shared && !c->hmis.empty()) {
     build_tables(c, 0, c->K, w0, a.nw, DOS_KERNEL_COLUMN_FORWARD, L);
     c->mis_built = c->mis_gen;
   }
@@ -1272,6 +1277,71 @@ int choose_path(dos_ctx* x, int requested) {
   return DOS_OK;
 }
 
+// The table of signed roots, made by the first displacement.
+int need_roots(dos_ctx* c) {
+  if (c->sq) return DOS_OK;
+  const size_t count = (size_t)c->nw * c->hs * c->hs;
+  float* roots = nullptr;  // c->sq once its kernel is queued
+  const int rc = c->alloc(&roots, count, "root table");
+  if (rc) return rc;
+  const cudaError_t e = dos::launch_sqtable(roots, nullptr, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream);
+  if (e != cudaSuccess) {
+    c->dealloc(&roots, count);
+    return fail(DOS_ERR_CUDA, std::string("root table: ") + cudaGetErrorString(e));
+  }
+  c->sq = roots;
+  return DOS_OK;
+}
+
+// n more tables for displaced gaps, and with the first ones the roots'
+// remainders; false, and nothing kept, where they do not fit.  They are taken
+// only while an eighth of the device's memory stays free: the column passes do
+// without them, a caller's own allocations may not.
+bool more_tables(dos_ctx* c, int n) {
+  const size_t count = (size_t)c->nw * c->hs * c->hs;
+  const bool first = !c->sq_lo;
+  // one allocation; the remainders (count floats, count even) behind the tables
+  const size_t total = n * count + (first ? count / 2 : 0);
+  size_t free_bytes = 0, device_bytes = 0;
+  if (cudaMemGetInfo(&free_bytes, &device_bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (free_bytes < total * sizeof(float2) + device_bytes / 8) return false;
+  float2* block = nullptr;
+  if (c->alloc(&block, total, "displaced transfer tables") != DOS_OK) return false;
+  std::vector<CUtensorMap> maps(n);
+  bool ok = true;
+  for (int i = 0; ok && c->have_tmap && i < n; ++i) ok = make_table_map(c, &maps[i], block + i * count, 1) == DOS_OK;
+  if (ok && first) {
+    float* lo = reinterpret_cast<float*>(block + n * count);
+    ok = dos::launch_sqtable(nullptr, lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream) == cudaSuccess;
+    if (ok) c->sq_lo = lo;
+  }
+  if (!ok) {
+    c->dealloc(&block, total);
+    return false;
+  }
+  for (int i = 0; i < n; ++i) c->hmis.push_back(block + i * count);
+  c->tmap_Hm.insert(c->tmap_Hm.end(), maps.begin(), maps.end());
+  return true;
+}
+
+// Tables for the gaps whose length the current displacement changes (c->mis).
+void need_tables(dos_ctx* c) {
+  c->mis_table.assign(c->K + 1, -1);
+  c->mis_shared = false;
+  if (c->call_choice >= 0 && c->step_choice >= 0) return;  // no multi-pass choice
+  int need = 0;
+  for (int g = 0; g <= c->K; ++g)
+    if (c->gap_mis(g).dz != 0.f) c->mis_table[g] = need++;
+  const int have = (int)c->hmis.size();
+  if (need <= have || (need <= c->mis_most && more_tables(c, need - have))) return;
+  c->mis_shared = have > 0 || (c->mis_most > 0 && more_tables(c, 1));
+  for (int& t : c->mis_table)
+    if (t >= 0) t = c->mis_shared ? 0 : -1;
+}
+
 int check_ctx(dos_ctx* c) {
   if (!c) return fail(DOS_ERR_ARG, "context is NULL");
   cudaError_t e = cudaSetDevice(c->device);
@@ -1362,30 +1432,7 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
   }
   for (int i = 0; i < 3 * c->K; ++i)
     if (!std::isfinite(disp[i])) return fail(DOS_ERR_ARG, "displacements must be finite");
-  if (!c->sq) {
-    const size_t count = (size_t)c->nw * c->hs * c->hs;
-    float* roots = nullptr;  // c->sq once its kernel is queued
-    if ((rc = c->alloc(&roots, count, "root table"))) return rc;
-    // the column passes' tables: where they do not fit, the plain kernel does without
-    if ((c->call_choice < 0 || c->step_choice < 0) &&  // the multi-pass choices
-        c->alloc(&c->sq_lo, count, "root table") == DOS_OK) {
-      for (int tables : {c->K + 1, 1}) {
-        if (c->alloc(&c->hmis, tables * count, "displaced transfer tables") != DOS_OK) continue;
-        if (!c->have_tmap || make_table_map(c, &c->tmap_Hm, c->hmis, tables) == DOS_OK) c->mis_tables = tables;
-        else c->dealloc(&c->hmis, tables * count);  // as where they do not fit
-        break;
-      }
-      if (c->mis_tables == 0) c->dealloc(&c->sq_lo, count);
-    }
-    const cudaError_t e = dos::launch_sqtable(roots, c->sq_lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream);
-    if (e != cudaSuccess) {
-      // nothing is kept: the next call makes the tables again
-      c->dealloc(&roots, count);
-      if (c->mis_tables) c->dealloc(&c->hmis, c->mis_tables * count), c->dealloc(&c->sq_lo, count), c->mis_tables = 0;
-      return fail(DOS_ERR_CUDA, std::string("root table: ") + cudaGetErrorString(e));
-    }
-    c->sq = roots;
-  }
+  if ((rc = need_roots(c))) return rc;
   // layer l (1..K) displaced by D_l; planes 0 (aperture) and K+1 (detector) fixed:
   // gap g carries the lateral shift D_g - D_{g+1} and the length change dz_{g+1} - dz_g
   c->mis.assign(3 * (c->K + 1), 0.0);
@@ -1396,6 +1443,7 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
     c->mis[3 * g + 2] = D(g + 1, 2) - D(g, 2);
   }
   c->mis_on = true;
+  need_tables(c);
   return DOS_OK;
 }
 

@@ -165,7 +165,7 @@ int supported_m_list(int* out, int cap);
 cudaError_t launch_htable(float2* Hq, const double* d_lambda, int nw, double z, double n_medium,
                           double pitch, int m, int hs, int evanescent, cudaStream_t s);
 cudaError_t launch_arow(float2* arow, int m, int offset, int width, cudaStream_t s);
-// sq_lo: what the rounding of sq left (null: not wanted)
+// sq: the roots, sq_lo: what their rounding left (either null: not wanted)
 cudaError_t launch_sqtable(float* sq, float* sq_lo, const double* d_lambda, int nw, double n_medium, double pitch, int m, int hs,
                            cudaStream_t s);
 // out[i] = Hq * H(dz[i]) over the count quadrant entries of the channels (from

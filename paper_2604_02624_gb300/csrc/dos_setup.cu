@@ -73,7 +73,7 @@ __global__ void k_sqtable(float* __restrict__ sq, float* __restrict__ sq_lo, con
     const double q = bin_q(k * k, fa, fb);
     const double r = q >= 0.0 ? sqrt(q) : -sqrt(-q);
     const size_t at = ((size_t)w * hs + a) * hs + b;
-    sq[at] = (float)r;
+    if (sq) sq[at] = (float)r;
     if (sq_lo) sq_lo[at] = (float)(r - (double)(float)r);
   }
 }
