@@ -312,11 +312,13 @@ DOS_API int dos_read_loss(dos_ctx *ctx, double *h_loss);
 DOS_API int dos_backward(dos_ctx *ctx, const float *d_dLdI, float *d_dLdh);
 
 /*
- * One design step: dos_forward(save) + dos_loss + dos_backward, replayed as a
- * CUDA graph.  The first call for a given set of pointers captures the step
- * on a stream private to the context (ordered after the context's stream by
- * an event, and the context's stream after it); later calls with the same
- * pointers replay the graph.
+ * One design step: dos_forward(save) + dos_loss + dos_backward.  A call whose
+ * pointers or displacement differ from the last step's queues the kernels on the
+ * context's stream; the next one with the same captures them as a CUDA graph,
+ * which later calls replay on a stream private to the context (ordered after the
+ * context's stream by an event, and the context's stream after it).  Steps of
+ * one context follow one another, whatever streams they are called on.  Same
+ * results either way.
  *   d_h [K][N][N], d_T [N_w][F_d][F_d] inputs; d_dLdh [K][N][N] output (all required).
  *   d_I [N_w][F][F] and d_psnr [N_w] optional outputs (NULL to skip).
  *   h_loss: when non-NULL receives L (waits for the stream).

@@ -162,8 +162,9 @@ class DiffractiveStack:
     def step(self, h: torch.Tensor, T: torch.Tensor, grad_out: Optional[torch.Tensor] = None,
              intensity_out: Optional[torch.Tensor] = None, psnr_out: Optional[torch.Tensor] = None,
              read: bool = False):
-        """Forward + loss + backward in one call, replayed as a CUDA graph.
-        Returns (loss or None, dL/dh).  Reusing the same tensors reuses the graph."""
+        """Forward + loss + backward in one call.  Returns (loss or None, dL/dh).
+        The second step with the same tensors (and displacement) is captured as a
+        CUDA graph, which later ones replay."""
         _need(h, torch.float32, (self.n_layers, self.n, self.n), "h", self.device)
         _need(T, torch.float32, (self.n_lambda, self.det, self.det), "T", self.device)
         g = grad_out if grad_out is not None else torch.empty_like(h)

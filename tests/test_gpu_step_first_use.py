@@ -1,0 +1,137 @@
+"""A step's first call with its tensors and displacement queues the kernels, its
+second captures them, later ones replay the graph: the same results bit for bit,
+no graph for steps that do not come again, and a caller's own capture may hold a
+step that has not run before."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import dos_oracle as O
+from paper_2604_02624_gb300 import _lib as L
+from paper_2604_02624_gb300 import workloads as W
+from paper_2604_02624_gb300.api import DiffractiveStack
+
+from gpu_cases import TOL_GRAD_ORACLE, assert_close, oracle_model
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+DISP = np.array([[40e-9, -25e-9, 80e-9]])
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not os.path.exists(L.LIB_PATH):
+        from paper_2604_02624_gb300 import build
+        build.build()
+    L.load()
+    torch.cuda.set_device(DEV)
+
+
+def _design():
+    w = W.workload("tiny")
+    h = W.thickness(w, 0).astype(np.float32).astype(np.float64)
+    T = W.targets(w, 1)
+    return w, h, T, torch.tensor(h, dtype=torch.float32, device=DEV), torch.tensor(T, dtype=torch.float32, device=DEV)
+
+
+def _outputs(w):
+    return (torch.empty((w.n_layers, w.n, w.n), device=DEV), torch.empty((len(w.lambdas), w.fov, w.fov), device=DEV),
+            torch.empty(len(w.lambdas), device=DEV))
+
+
+@pytest.mark.parametrize("path", ["multipass", "multipass_bulk", "fused", "dft_gemm_x3"])
+def test_queued_captured_and_replayed_steps_agree(path):
+    w, h, T, hd, Td = _design()
+    st = DiffractiveStack.from_workload(w, device=DEV, path=path)
+    a, b = _outputs(w), _outputs(w)
+    for disp in (None, DISP, None):
+        st.set_misalignment(disp)
+        _, _, ref, _ = O.loss_and_grad(h, T, displacements=disp, **oracle_model(w))
+        first = None
+        for out in (a, a, a, b, a, b, b, b, a, a):  # queued, captured, replayed; another key in between
+            for t in out:
+                t.fill_(-1.0)
+            val, _ = st.step(hd, Td, grad_out=out[0], intensity_out=out[1], psnr_out=out[2], read=True)
+            got = [val, st.last_launch_count] + [t.cpu().numpy().copy() for t in out]
+            if first is None:
+                first = got
+                assert_close(got[2].astype(np.float64), ref, TOL_GRAD_ORACLE)
+            for x, y in zip(first, got):
+                assert np.array_equal(x, y)
+    st.close()
+
+
+def test_steps_that_do_not_come_again_make_no_graph():
+    w, h, T, hd, Td = _design()
+    st = DiffractiveStack.from_workload(w, device=DEV)
+    out = _outputs(w)
+    grads = [torch.empty_like(out[0]) for _ in range(4)]
+
+    def calls(f):
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU,
+                                                torch.profiler.ProfilerActivity.CUDA]) as prof:
+            f()
+            torch.cuda.synchronize()
+        names = [e.name for e in prof.events()]
+        return (sum(n.startswith("cudaGraphInstantiate") for n in names), sum(n.startswith("cudaGraphLaunch") for n in names))
+
+    def new_displacements():
+        for i in range(4):
+            st.set_misalignment(DISP * (i + 1))
+            st.step(hd, Td, grad_out=out[0])
+
+    def new_tensors():
+        for g in grads:
+            st.step(hd, Td, grad_out=g)
+
+    def the_same():
+        for _ in range(4):
+            st.step(hd, Td, grad_out=out[0])
+
+    assert calls(new_displacements) == (0, 0)
+    assert calls(new_tensors) == (0, 0)
+    assert calls(the_same) == (1, 3)
+    st.close()
+
+
+@pytest.mark.parametrize("path", ["multipass_bulk", "fused"])
+def test_a_caller_captures_a_step_that_has_not_run(path):
+    w, h, T, hd, Td = _design()
+    st = DiffractiveStack.from_workload(w, device=DEV, path=path)
+    out = _outputs(w)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(2):  # the second call comes again, but under the caller's capture
+            st.step(hd, Td, grad_out=out[0], intensity_out=out[1], psnr_out=out[2])
+    _, _, ref, _ = O.loss_and_grad(h, T, **oracle_model(w))
+    for _ in range(2):
+        out[0].zero_()
+        graph.replay()
+        assert_close(out[0].cpu().numpy().astype(np.float64), ref, TOL_GRAD_ORACLE)
+    st.close()
+
+
+def test_steps_of_several_streams_follow_one_another():
+    """Queued, captured and replayed steps of one context from streams that nothing
+    else orders: each leaves its own outputs whole."""
+    w, h, T, hd, Td = _design()
+    st = DiffractiveStack.from_workload(w, device=DEV, path="multipass_bulk")
+    streams = [torch.cuda.Stream(DEV) for _ in range(3)]
+    outs = [_outputs(w) for _ in range(3)]
+    hs = [hd * s for s in (1.0, 0.5, 0.25)]
+    refs = []
+    for x in hs:
+        val, g = st.step(x, Td, read=True)
+        refs.append(g.cpu().numpy())
+    torch.cuda.synchronize()
+    for order in ((0, 1, 2), (0, 0, 0), (1, 0, 1), (0, 2, 2), (2, 0, 2), (1, 1, 1)):
+        for i in order:
+            with torch.cuda.stream(streams[i]):
+                outs[i][0].zero_()
+                st.step(hs[i], Td, grad_out=outs[i][0], intensity_out=outs[i][1], psnr_out=outs[i][2])
+        torch.cuda.synchronize()
+        for i in set(order):
+            assert np.array_equal(outs[i][0].cpu().numpy(), refs[i])
+    st.close()
