@@ -257,11 +257,11 @@ DOS_API int dos_loss_noalloc(const float *d_I, const float *d_T, int n_lambda, i
  * On the multi-pass paths a displacement that changes gaps' lengths reserves one
  * transfer table (N_w (M/2+2)^2 complex floats) for each of them, if the context
  * does not hold that many yet, and with the first half a table for what the
- * roots' rounding left; lateral displacements need none.  A table is taken only
- * while an eighth of the device's memory stays free; where the gaps' tables do
- * not fit they share one, where that does not either they do without (the
- * column passes are then slower).  DOS_DISPLACED_TABLES=<n> at dos_create keeps a
- * context to n tables (0: none).
+ * roots' rounding left; lateral displacements need none.  More than a gigabyte
+ * is taken only while an eighth of the device's memory stays free; where the
+ * gaps' tables do not fit they share one, where that does not either they do
+ * without (the column passes are then slower).  DOS_DISPLACED_TABLES=<n> at
+ * dos_create keeps a context to n tables (0: none).
  * Errors: DOS_ERR_ARG, DOS_ERR_OOM, DOS_ERR_CUDA.
  */
 DOS_API int dos_set_misalignment(dos_ctx *ctx, const double *h_disp);

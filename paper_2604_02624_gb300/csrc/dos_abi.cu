@@ -1340,47 +1340,41 @@ int capture_step(dos_ctx* c, const dos_ctx::StepKey& key, const float* d_h, cons
   return DOS_OK;
 }
 
-// The table of signed roots, made by the first displacement.
-int need_roots(dos_ctx* c) {
-  if (c->sq) return DOS_OK;
-  const size_t count = (size_t)c->nw * c->hs * c->hs;
-  float* roots = nullptr;  // c->sq once its kernel is queued
-  const int rc = c->alloc(&roots, count, "root table");
-  if (rc) return rc;
-  const cudaError_t e = dos::launch_sqtable(roots, nullptr, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream);
-  if (e != cudaSuccess) {
-    c->dealloc(&roots, count);
-    return fail(DOS_ERR_CUDA, std::string("root table: ") + cudaGetErrorString(e));
-  }
-  c->sq = roots;
+// Queues the kernel that fills the signed roots (roots, for c->sq) and what their
+// rounding left (lo, for c->sq_lo), either null if not wanted; the context's
+// pointers are set once it is queued.
+int make_roots(dos_ctx* c, float* roots, float* lo) {
+  DOS_CUDA(dos::launch_sqtable(roots, lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream), "root table");
+  if (roots) c->sq = roots;
+  if (lo) c->sq_lo = lo;
   return DOS_OK;
 }
 
 // n more tables for displaced gaps, and with the first ones the roots'
-// remainders; false, and nothing kept, where they do not fit.  They are taken
-// only while an eighth of the device's memory stays free: the column passes do
-// without them, a caller's own allocations may not.
-bool more_tables(dos_ctx* c, int n) {
+// remainders (with the roots themselves where those are still to be made: the
+// kernel is all FP64); false, and nothing kept, where they do not fit.  Large
+// ones are taken only while an eighth of the device's memory stays free: the
+// column passes do without them, a caller's own allocations may not.
+bool more_tables(dos_ctx* c, int n, float* roots) {
   const size_t count = (size_t)c->nw * c->hs * c->hs;
   const bool first = !c->sq_lo;
   // one allocation; the remainders (count floats, count even) behind the tables
   const size_t total = n * count + (first ? count / 2 : 0);
+  constexpr size_t kLarge = (size_t)1 << 30;  // asking for the free memory costs a first step host time
   size_t free_bytes = 0, device_bytes = 0;
-  if (cudaMemGetInfo(&free_bytes, &device_bytes) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return false;
+  if (total * sizeof(float2) > kLarge) {
+    if (cudaMemGetInfo(&free_bytes, &device_bytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
+    if (free_bytes < total * sizeof(float2) + device_bytes / 8) return false;
   }
-  if (free_bytes < total * sizeof(float2) + device_bytes / 8) return false;
   float2* block = nullptr;
   if (c->alloc(&block, total, "displaced transfer tables") != DOS_OK) return false;
   std::vector<CUtensorMap> maps(n);
   bool ok = true;
   for (int i = 0; ok && c->have_tmap && i < n; ++i) ok = make_table_map(c, &maps[i], block + i * count, 1) == DOS_OK;
-  if (ok && first) {
-    float* lo = reinterpret_cast<float*>(block + n * count);
-    ok = dos::launch_sqtable(nullptr, lo, c->d_lam, c->nw, c->n_med, c->pitch, c->m, c->hs, c->stream) == cudaSuccess;
-    if (ok) c->sq_lo = lo;
-  }
+  if (ok && first) ok = make_roots(c, roots, reinterpret_cast<float*>(block + n * count)) == DOS_OK;
   if (!ok) {
     c->dealloc(&block, total);
     return false;
@@ -1391,7 +1385,7 @@ bool more_tables(dos_ctx* c, int n) {
 }
 
 // Tables for the gaps whose length the current displacement changes (c->mis).
-void need_tables(dos_ctx* c) {
+void need_tables(dos_ctx* c, float* roots) {
   c->mis_table.assign(c->K + 1, -1);
   c->mis_shared = false;
   if (c->call_choice >= 0 && c->step_choice >= 0) return;  // no multi-pass choice
@@ -1399,8 +1393,8 @@ void need_tables(dos_ctx* c) {
   for (int g = 0; g <= c->K; ++g)
     if (c->gap_mis(g).dz != 0.f) c->mis_table[g] = need++;
   const int have = (int)c->hmis.size();
-  if (need <= have || (need <= c->mis_most && more_tables(c, need - have))) return;
-  c->mis_shared = have > 0 || (c->mis_most > 0 && more_tables(c, 1));
+  if (need <= have || (need <= c->mis_most && more_tables(c, need - have, roots))) return;
+  c->mis_shared = have > 0 || (c->mis_most > 0 && more_tables(c, 1, roots));
   for (int& t : c->mis_table)
     if (t >= 0) t = c->mis_shared ? 0 : -1;
 }
@@ -1495,7 +1489,9 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
   }
   for (int i = 0; i < 3 * c->K; ++i)
     if (!std::isfinite(disp[i])) return fail(DOS_ERR_ARG, "displacements must be finite");
-  if ((rc = need_roots(c))) return rc;
+  const size_t count = (size_t)c->nw * c->hs * c->hs;
+  float* roots = nullptr;  // made by the first displacement
+  if (!c->sq && (rc = c->alloc(&roots, count, "root table"))) return rc;
   // layer l (1..K) displaced by D_l; planes 0 (aperture) and K+1 (detector) fixed:
   // gap g carries the lateral shift D_g - D_{g+1} and the length change dz_{g+1} - dz_g
   c->mis.assign(3 * (c->K + 1), 0.0);
@@ -1506,7 +1502,12 @@ DOS_API int dos_set_misalignment(dos_ctx* c, const double* disp) {
     c->mis[3 * g + 2] = D(g + 1, 2) - D(g, 2);
   }
   c->mis_on = true;
-  need_tables(c);
+  need_tables(c, roots);
+  if (!c->sq && (rc = make_roots(c, roots, nullptr))) {
+    c->dealloc(&roots, count);
+    c->mis_on = false;
+    return rc;
+  }
   return DOS_OK;
 }
 
