@@ -8,6 +8,7 @@
 // thread sums at most a few hundred terms), the block tree and everything
 // after it in FP64 (GB300's FP64 rate is a small fraction of its FP32 rate);
 // every sum has a fixed order, so results are reproducible bit for bit.
+#include "dos_decibel.cuh"
 #include "dos_internal.h"
 
 #include "../../include/dos.h"
@@ -53,23 +54,6 @@ __device__ __forceinline__ double warp_total(const float* part, int lane) {
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
   return v;
-}
-
-// 10 log10(x) rounded to FP32.  An FP64 logarithm is a few hundred dependent
-// FP64 instructions, the longest chain of a small launch; here x = f (1 + d)
-// with f its FP32 rounding and f = m 2^e, m in [2/3, 4/3), so that log10 x =
-// e log10 2 + log10 m + d / ln 10 with |log10 m| <= 0.18: the FP32 terms are
-// wrong by at most 2e-8 (2e-7 dB; with e = 0 by a few units of FP32 rounding
-// of the result itself), the sum is FP64.
-__device__ __forceinline__ float ten_log10(double x) {
-  const float f = (float)x;
-  if (!(f > 1e-30f && f < 1e30f)) return (float)(10.0 * log10(x));  // also 0, infinities, NaN
-  const float d = (float)(x - (double)f) / f;
-  int e;
-  float m = frexpf(f, &e);  // [0.5, 1)
-  if (m < 0.66666667f) m *= 2.f, --e;
-  const float small = fmaf(d, 0.43429448190325182765f, log10f(m));
-  return (float)(10.0 * fma((double)e, 0.30102999566398119521, (double)small));
 }
 
 // Detector pixels a channel may have for its values to stay in shared memory
