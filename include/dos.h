@@ -97,10 +97,12 @@ enum {
  *    parts and six products kept (~1e-7 per GEMM, twice the tensor work).
  *  DOS_PATH_AUTO: dos_create times one forward+backward of every available
  *    multi-pass (plain and bulk) / cluster-resident configuration and keeps
- *    the fastest, for dos_step by its kernels' time, for the other calls by that
- *    and the host's time to queue them beside a caller's own work (small designs
- *    may then differ: dos_path names the other calls' implementation,
- *    dos_describe both); from per-kernel event times of the plain and the bulk
+ *    the fastest, for dos_step by its kernels' time, for the other calls another
+ *    one where its fewer launches clearly save a host-bound caller time (small
+ *    designs: dos_path names the other calls' implementation, dos_describe both,
+ *    with the times that decided; results of the two agree to rounding, not bit
+ *    for bit, and so do those of two contexts that chose differently); from
+ *    per-kernel event times of the plain and the bulk
  *    multi-pass runs it also times the mix that runs the faster kernel of
  *    each pass kind (column, forward row, adjoint row).
  * Environment: DOS_FORCE_CONFIG="multipass", "multipass:bulk",

@@ -1084,22 +1084,42 @@ std::string choice_detail(const dos_ctx* x, int idx) {
 
 // The step replays a graph, so its choice is the one whose kernels take the
 // least time.  The stream calls also cost the host their launches, and their
-// callers do host work of their own between them: some 60 us where a loop only
-// forms its objective, some 300 us under autograd.  A pass then takes the longer
-// of the GPU's time and the host's, and the stream calls' choice has the least
-// sum over the two callers.  It differs from the step's where a pass takes less
-// than that: 6 channels of 200 x 200, 12 calls and 55 us on the GPU with the
-// multi-pass kernels, 4 and 78 us cluster-resident, 446 against 406 us a pass
-// under autograd; 15 of 191 x 191, 106 and 123 us, 425 against 397 us.
+// callers do host work of their own between them, which the context cannot know:
+// some 60 us where a loop only forms its objective, some 300 us under autograd
+// (measured with torch).  A pass then takes the longer of the GPU's time and the
+// host's; its cost is the sum over the two callers.  The stream calls' choice is
+// the step's unless another costs them clearly less, by a twentieth, which only
+// fewer launches can bring about: 6 channels of 200 x 200, 12 launches and 55 us
+// on the GPU with the multi-pass kernels, 4 and 78 us cluster-resident, 446
+// against 406 us a pass under autograd; 15 of 191 x 191, 106 and 123 us, 425
+// against 397 us.  The host's time is the launches times one time for each, the
+// least seen at create: taken from each candidate's own run, its noise chose
+// between equal launches, 16 channels of 64 x 64 on two-block clusters, 146 us
+// for the three calls against 118 on four-block ones.
 constexpr float kCallerMs[2] = {0.06f, 0.3f};
+constexpr float kClearly = 0.95f;
 float call_cost(float gpu_ms, float host_ms) {
   return std::max(gpu_ms, host_ms + kCallerMs[0]) + std::max(gpu_ms, host_ms + kCallerMs[1]);
 }
+struct Timed {
+  int idx, launches;
+  float ms;
+};
+int choose_calls(const std::vector<Timed>& t, int best, float launch_ms) {
+  auto cost = [&](const Timed& c) { return call_cost(c.ms, (float)c.launches * launch_ms); };
+  const Timed* of_step = nullptr;
+  const Timed* least = nullptr;
+  for (const Timed& c : t) {
+    if (c.idx == best) of_step = &c;
+    if (!least || cost(c) < cost(*least) || (cost(c) == cost(*least) && c.ms < least->ms)) least = &c;
+  }
+  return least && of_step && cost(*least) < kClearly * cost(*of_step) ? least->idx : best;
+}
 
 // time forward(save) + backward of the current choice on zero thickness / zero
-// seed; with kind_ms, one more forward + backward with per-launch events gives
-// the time of every kernel kind
-int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, float* ms_out, float* host_ms_out,
+// seed, and the least host time of a launch so far; with kind_ms, one more
+// forward + backward with per-launch events gives the time of every kernel kind
+int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, Timed* out, float* launch_ms,
                 double* kind_ms = nullptr) {
   int rc;
   if ((rc = run_forward(x, h0, nullptr, 1)) || (rc = run_backward(x, h0, g0, d0))) return rc;
@@ -1110,7 +1130,10 @@ int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, float* 
   for (int rep = 0; rep < 2; ++rep) {
     const auto t0 = std::chrono::steady_clock::now();
     cudaEventRecord(a, x->stream);
-    if ((rc = run_forward(x, h0, nullptr, 1)) || (rc = run_backward(x, h0, g0, d0))) break;
+    if ((rc = run_forward(x, h0, nullptr, 1))) break;
+    out->launches = x->launches;
+    if ((rc = run_backward(x, h0, g0, d0))) break;
+    out->launches += x->launches;
     cudaEventRecord(b, x->stream);
     host = std::min(host, std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count());
     cudaError_t e = cudaEventSynchronize(b);
@@ -1144,8 +1167,8 @@ int time_choice(dos_ctx* x, const float* h0, const float* g0, float* d0, float* 
     x->timer.on = on0;
   }
   if (!rc) rc = err_check(x);
-  *ms_out = best;
-  *host_ms_out = host;
+  out->ms = best;
+  *launch_ms = std::min(*launch_ms, host / (float)std::max(1, out->launches));
   return rc;
 }
 
@@ -1232,8 +1255,9 @@ int choose_path(dos_ctx* x, int requested) {
   if (e == cudaSuccess) e = cudaMemsetAsync(g0, 0, sizeof(float) * (size_t)x->nw * x->fov * x->fov, x->stream);
   int rc = DOS_OK;
   if (e != cudaSuccess) rc = fail(DOS_ERR_CUDA, std::string("autotune buffers: ") + cudaGetErrorString(e));
-  int best = cands[0], best_call = cands[0];
-  float best_ms = 1e30f, best_call_ms = 1e30f;
+  int best = cands[0];
+  float best_ms = 1e30f, launch_ms = 1e30f;
+  std::vector<Timed> timed;
   std::ostringstream d;
   d << "tuned (fwd+bwd ms):";
   // per-kind times of the plain and the bulk-prefetching multi-pass kernels;
@@ -1242,9 +1266,10 @@ int choose_path(dos_ctx* x, int requested) {
   for (size_t k = 0; rc == DOS_OK && k < cands.size(); ++k) {
     const int idx = cands[k];
     set_choice(x, idx);
-    float ms = 0.f, host_ms = 0.f;
-    rc = time_choice(x, h0, g0, d0, &ms, &host_ms, idx == kPlain ? kind_plain : idx == kBulk ? kind_bulk : nullptr);
+    Timed t = {idx, 0, 0.f};
+    rc = time_choice(x, h0, g0, d0, &t, &launch_ms, idx == kPlain ? kind_plain : idx == kBulk ? kind_bulk : nullptr);
     if (rc) break;
+    timed.push_back(t);
     if (idx == kBulk && requested == DOS_PATH_AUTO) {
       unsigned mix = 0;
       if (kind_bulk[DOS_KERNEL_COLUMN_FORWARD] + kind_bulk[DOS_KERNEL_COLUMN_ADJOINT] <
@@ -1256,22 +1281,19 @@ int choose_path(dos_ctx* x, int requested) {
     }
     d << " " << choice_name(x, idx);
     if (idx >= 0) d << "x" << x->fcand_clusters[idx];
-    d << "=" << ms;
-    if (ms < best_ms) {
-      best_ms = ms;
+    d << "=" << t.ms;
+    if (t.ms < best_ms) {
+      best_ms = t.ms;
       best = idx;
-    }
-    const float call_ms = call_cost(ms, host_ms);
-    if (call_ms < best_call_ms || (call_ms == best_call_ms && best == idx)) {
-      best_call_ms = call_ms;
-      best_call = idx;
     }
   }
   cudaFree(h0);
   cudaFree(g0);
   cudaFree(d0);
   if (rc) return rc;
+  const int best_call = choose_calls(timed, best, launch_ms);
   keep_choices(x, best_call, best);
+  d << " launch=" << launch_ms;
   x->describe = choice_detail(x, best_call) + " | " + d.str();
   if (cache && *cache) {
     std::ofstream out(cache, std::ios::app);
