@@ -19,9 +19,10 @@ namespace dos {
 DOS_HD float ten_log10(double x) {
   const float f = (float)x;
   if (!(f > 1e-30f && f < 1e30f)) return (float)(10.0 * log10(x));  // also 0, infinities, NaN
-  const double d = x - 1.0;
-  if (d * d < 1e-6)  // close to one, where l is not small beside m - 1: ln(1 + d), four terms
+  if (fabsf(f - 1.f) < 1e-3f) {  // l is not small beside m - 1: ln(1 + d), four terms
+    const double d = x - 1.0;
     return (float)(4.3429448190325183 * (d * (1.0 - d * (0.5 - d * (1.0 / 3.0 - d * 0.25)))));
+  }
   int e;
   float m = frexpf(f, &e);  // [0.5, 1)
   if (m < 0.66666667f) m *= 2.f, --e;
