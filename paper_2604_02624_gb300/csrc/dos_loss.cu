@@ -41,30 +41,50 @@ __device__ __forceinline__ float detector(const float2* ow, int fov, int b, int 
   return s;
 }
 
-// Fixed-order FP64 total of the block's NT FP32 partials, by one warp: lane l
-// adds NT / 32 of them, a shuffle tree the 32 lanes.  The total is
+// (s, e) += x with s + e kept exact up to the rounding of e
+__device__ __forceinline__ void pair_add(float& s, float& e, float x) {
+  const float t = __fadd_rn(s, x);
+  const float z = __fadd_rn(t, -s);
+  e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(x, -z)));
+  s = t;
+}
+
+// Fixed-order FP64 total of the block's NT partials, by one warp: lane l
+// adds NT / 32 of them, a shuffle tree the 32 lanes.  A partial may be an FP32
+// pair, part + lo (lo not null); the small parts are summed in FP32.  The total is
 // valid in lane 0.  (An FP64 addition occupies the SM's FP64 pipe for many
 // cycles: one warp issues 13 of them here where a block-wide tree in shared
 // memory issues them from every warp and takes eight barriers per sum.)
 template <int NT>
-__device__ __forceinline__ double warp_total(const float* part, int lane) {
+__device__ __forceinline__ double warp_total(const float* part, const float* lo, int lane) {
   double v = 0.0;
+  float l = 0.f;
 #pragma unroll
-  for (int i = 0; i < NT / 32; ++i) v += (double)part[lane + 32 * i];
+  for (int i = 0; i < NT / 32; ++i) {
+    v += (double)part[lane + 32 * i];
+    if (lo) l += lo[lane + 32 * i];
+  }
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
-  return v;
+  for (int s = 16; s > 0; s >>= 1) {
+    v += __shfl_down_sync(0xffffffffu, v, s);
+    if (lo) l += __shfl_down_sync(0xffffffffu, l, s);
+  }
+  return lo ? v + (double)l : v;
 }
 
 // Detector pixels a channel may have for its values to stay in shared memory
 // between the two loops (16 KB: five blocks and more per SM); above it the
 // second loop forms them again.
 constexpr int kLossKeep = 4096;
-// Up to this many detector pixels a channel gets a block of 128 threads, so that
-// twice as many channels are in flight (a thread then adds at most ten terms,
-// as one of 256 does at 50 x 50).  Not with the scaled loss: its sigma, and with
-// it dL/dI, would round differently for another order of the sums.
-constexpr int kLossSmall = 1280;
+// Up to this many detector pixels, and above as many channels as blocks of 256
+// threads are resident at once (eight per SM), a channel gets a block of 128
+// threads, so that twice as many are in flight: 2048 channels of 32 x 32 on 4 x
+// 4-pixel detectors 37 -> 31 us, but 4 channels of 32 x 32 1.3 us more.  A thread
+// of it keeps its even and its odd strides apart, the two chains of FP32
+// multiply-adds that two threads of the larger block have, and adds them as an
+// FP32 pair: the sums have as few terms in FP32 as there, and the same value to
+// 2^-48.
+constexpr int kLossSmall = 1280, kLossMany = 1024;
 
 // One block per channel: sum (D-T)^2, sigma = sum D T / sum D^2, sum (sigma D
 // - T)^2, the PSNR (psnr not null) and (dLdI not null) dL/dI of the channel's
@@ -77,8 +97,8 @@ constexpr int kLossSmall = 1280;
 // division and one logarithm per channel, each in a block of its own (the
 // total kernel took them all in one block), and the detector sums formed once.
 // 4096 channels of 50 x 50: 157 -> 64 us; 2048 channels of 32 x 32 on
-// 4 x 4-pixel detectors 88 -> 31 us (37 us with blocks of 256 threads); 4 channels of 32 x 32 20 -> 11 us
-// (with the total and the PSNR, both launches before).
+// 4 x 4-pixel detectors 88 -> 31 us; 4 channels of 32 x 32 20 -> 11 us (with the
+// total and the PSNR, both launches before).
 template <int NT>
 __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const float* __restrict__ T,
                                                       LossStats* __restrict__ st, int fov, int b,
@@ -86,7 +106,9 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
                                                       float* __restrict__ psnr, double* __restrict__ d_loss,
                                                       unsigned* __restrict__ ticket) {
   extern __shared__ float dsh[];  // [det2] detector values, when det2 <= kLossKeep
+  constexpr int V = kRedThreads / NT;  // chains of a thread
   __shared__ float part[3][NT];
+  __shared__ float lows[V > 1 ? 3 : 1][V > 1 ? NT : 1];
   __shared__ double tot[3];
   __shared__ float sg_sh;
   __shared__ bool last;
@@ -96,22 +118,31 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
   const bool keep = det2 <= kLossKeep;
   const float2* ow = o + (size_t)w * fov * fov;
   const float* tw = T + (size_t)w * det2;
-  float fse = 0.f, fit = 0.f, fii = 0.f;
-  for (int p = threadIdx.x; p < det2; p += NT) {
-    const float I = detector(ow, fov, b, p);
-    const float t = tw[p];
-    const float d = I - t;
-    if (keep) dsh[p] = I;
-    fse = fmaf(d, d, fse);
-    fit = fmaf(I, t, fit);
-    fii = fmaf(I, I, fii);
+  float sum[3] = {}, low[3] = {};
+#pragma unroll 1
+  for (int i = threadIdx.x; i < kRedThreads; i += NT) {
+    float fse = 0.f, fit = 0.f, fii = 0.f;
+    for (int p = i; p < det2; p += kRedThreads) {
+      const float I = detector(ow, fov, b, p);
+      const float t = tw[p];
+      const float d = I - t;
+      if (keep) dsh[p] = I;
+      fse = fmaf(d, d, fse);
+      fit = fmaf(I, t, fit);
+      fii = fmaf(I, I, fii);
+    }
+    pair_add(sum[0], low[0], fse);
+    pair_add(sum[1], low[1], fit);
+    pair_add(sum[2], low[2], fii);
   }
-  part[0][threadIdx.x] = fse;
-  part[1][threadIdx.x] = fit;
-  part[2][threadIdx.x] = fii;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    part[k][threadIdx.x] = sum[k];
+    if constexpr (V > 1) lows[k][threadIdx.x] = isinf(sum[k]) ? 0.f : low[k];  // inf - inf is no rounding error
+  }
   __syncthreads();
   if (warp < 3) {
-    const double v = warp_total<NT>(part[warp], lane);
+    const double v = warp_total<NT>(part[warp], V > 1 ? lows[warp] : nullptr, lane);
     if (lane == 0) tot[warp] = v;
   }
   __syncthreads();
@@ -124,13 +155,18 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
   const float sg = sg_sh;
   const bool scaled = mode == DOS_LOSS_MSE_SCALED;
   float* gw = dLdI ? dLdI + (size_t)w * fov * fov : nullptr;
-  float fsc = 0.f;
-  for (int p = threadIdx.x; p < det2; p += NT) {
-    const float I = keep ? dsh[p] : detector(ow, fov, b, p);
-    const float t = tw[p];
-    const float d = fmaf(sg, I, -t);
-    fsc = fmaf(d, d, fsc);
-    if (gw && b == 1) gw[p] = scaled ? scale * sg * d : scale * (I - t);
+  sum[0] = low[0] = 0.f;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < kRedThreads; i += NT) {
+    float fsc = 0.f;
+    for (int p = i; p < det2; p += kRedThreads) {
+      const float I = keep ? dsh[p] : detector(ow, fov, b, p);
+      const float t = tw[p];
+      const float d = fmaf(sg, I, -t);
+      fsc = fmaf(d, d, fsc);
+      if (gw && b == 1) gw[p] = scaled ? scale * sg * d : scale * (I - t);
+    }
+    pair_add(sum[0], low[0], fsc);
   }
   if (gw && b > 1) {
     const int fov2 = fov * fov;
@@ -141,10 +177,11 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
       gw[q] = scaled ? scale * sg * fmaf(sg, I, -t) : scale * (I - t);
     }
   }
-  part[0][threadIdx.x] = fsc;
+  part[0][threadIdx.x] = sum[0];
+  if constexpr (V > 1) lows[0][threadIdx.x] = isinf(sum[0]) ? 0.f : low[0];
   __syncthreads();
   if (warp == 0) {
-    const double ssc = warp_total<NT>(part[0], lane);
+    const double ssc = warp_total<NT>(part[0], V > 1 ? lows[0] : nullptr, lane);
     if (lane == 0) {
       LossStats s;
       s.sse = tot[0];
@@ -186,7 +223,7 @@ cudaError_t launch_loss(const float2* o, const float* T, LossStats* st, int nw, 
   const float scale = (float)(2.0 / norm);  // dL/dD = 2 (D - T) / norm
   const int det2 = (fov / bin) * (fov / bin);
   const size_t sm = det2 <= kLossKeep ? sizeof(float) * det2 : 0;
-  const bool small = det2 <= kLossSmall && mode != DOS_LOSS_MSE_SCALED;
+  const bool small = det2 <= kLossSmall && nw > kLossMany;
   return launch_next(small ? k_loss<128> : k_loss<kRedThreads>, dim3(nw), small ? 128 : kRedThreads, sm, s, o, T, st,
                      fov, bin, dLdI, scale, norm, mode, psnr, d_loss, ticket);
 }
@@ -226,14 +263,6 @@ cudaError_t launch_loss_final(const LossStats* st, int nw, int fov2, double norm
 // A step's thickness is copied here too (h not null), which saves the step a
 // copy of its own.
 constexpr int kGradThreads = 256;
-
-// (s, e) += x with s + e kept exact up to the rounding of e
-__device__ __forceinline__ void pair_add(float& s, float& e, float x) {
-  const float t = __fadd_rn(s, x);
-  const float z = __fadd_rn(t, -s);
-  e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(x, -z)));
-  s = t;
-}
 
 template <int SLICES>
 __global__ void __launch_bounds__(kGradThreads) k_grad_reduce(const float* __restrict__ partial,
