@@ -115,8 +115,9 @@ enum {
  * Fault injection (tests): DOS_INJECT_WAIT_TIMEOUT=1 at dos_create makes the
  * first bulk-prefetch pass that the context launches announce its bytes
  * without copying them, so that the bounded waits of its blocks expire (one
- * second) and the next dos_read_loss reports DOS_ERR_TIMEOUT; later calls
- * run normally.  DOS_INJECT_WAIT_TIMEOUT=2 lets the copies land but makes the
+ * second) and the next dos_read_loss or dos_check reports DOS_ERR_TIMEOUT; later
+ * calls run normally (on the DFT-GEMM paths the first call sets the error flag
+ * as a kernel would).  DOS_INJECT_WAIT_TIMEOUT=2 lets the copies land but makes the
  * odd threads of every block give up their first wait; =3, for a first bulk
  * pass that is a column pass, lets the copies land but makes every thread
  * give up its wait for the transfer-table tile of its block's last item.
@@ -295,9 +296,19 @@ DOS_API int dos_quantize_thickness(const float *d_h, float *d_hq, size_t count, 
  * result of that work are then invalid.  The flag is cleared by the report.
  * On the DFT-GEMM paths dos_forward and dos_backward also report, in the same
  * way and before they queue anything, an expired wait of an earlier call that
- * the GPU has finished by then.
+ * the GPU has finished by then; the refused call may be made again.
  */
 DOS_API int dos_read_loss(dos_ctx *ctx, double *h_loss);
+
+/*
+ * Waits for the context's stream and reports, as dos_read_loss does, whether a
+ * kernel queued since the previous check gave up a bounded wait: for callers
+ * that read no loss (their own objective, dos_propagate, dos_layer_field), after
+ * the last call whose results they use.  Under stream capture it waits for
+ * nothing and returns DOS_OK; the next check reports.
+ * Errors: DOS_ERR_TIMEOUT, DOS_ERR_CUDA.
+ */
+DOS_API int dos_check(dos_ctx *ctx);
 
 /*
  * Gradient of a real objective with respect to the thickness, by the adjoint
@@ -348,6 +359,7 @@ DOS_API int dos_layer_field(dos_ctx *ctx, int layer, float *d_v);
  * fields over gap `gap` (0..K) for every channel, or its adjoint (the same
  * chain with conj(H)) when `adjoint` is nonzero.
  *   d_in, d_out [N_w][N][N] complex64; may not alias.
+ * An expired bounded wait is reported by dos_check.
  * Errors: DOS_ERR_ARG, DOS_ERR_CUDA.
  */
 DOS_API int dos_propagate(dos_ctx *ctx, int gap, const float *d_in, float *d_out, int adjoint);

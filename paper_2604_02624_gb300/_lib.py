@@ -28,7 +28,7 @@ EXPORTS = ("dos_supported_m", "dos_create", "dos_set_stream", "dos_forward", "do
            "dos_read_loss", "dos_backward", "dos_step", "dos_output_field", "dos_layer_field",
            "dos_propagate", "dos_set_timing", "dos_kernel_time", "dos_workspace_bytes",
            "dos_last_launch_count", "dos_path", "dos_describe", "dos_destroy", "dos_last_error",
-           "dos_loss_noalloc", "dos_efficiency", "dos_quantize_thickness", "dos_set_misalignment")
+           "dos_loss_noalloc", "dos_efficiency", "dos_quantize_thickness", "dos_set_misalignment", "dos_check")
 
 DOS_NOALLOC_MAX_LAMBDA = 65536
 
@@ -77,6 +77,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         "dos_forward": (c_int, [p, p, p, c_int]),
         "dos_loss": (c_int, [p, p, POINTER(c_double), p, p]),
         "dos_read_loss": (c_int, [p, POINTER(c_double)]),
+        "dos_check": (c_int, [p]),
         "dos_backward": (c_int, [p, p, p]),
         "dos_step": (c_int, [p, p, p, p, p, p, POINTER(c_double)]),
         "dos_output_field": (c_int, [p, p]),
@@ -146,6 +147,11 @@ def dos_read_loss(ctx: int) -> float:
     out = c_double()
     _check(load().dos_read_loss(ctx, ctypes.byref(out)), "dos_read_loss")
     return out.value
+
+
+def dos_check(ctx: int) -> None:
+    """Waits for the context's stream; raises DOS_ERR_TIMEOUT if a kernel gave up a wait."""
+    _check(load().dos_check(ctx), "dos_check")
 
 
 def dos_backward(ctx: int, d_dLdI: int, d_dLdh: int) -> None:

@@ -147,6 +147,14 @@ class DiffractiveStack:
         self._bind()
         return L.dos_read_loss(self._ctx)
 
+    def check(self) -> None:
+        """Waits for the work queued so far and raises DosError (DOS_ERR_TIMEOUT)
+        if one of its kernels gave up a bounded wait, so that its results are
+        invalid.  Reading the loss does the same; this is for programs that read
+        none (an objective of their own, propagation)."""
+        self._bind()
+        L.dos_check(self._ctx)
+
     def backward(self, dLdI: torch.Tensor, out: Optional[torch.Tensor] = None):
         """dL/dh of the last forward that saved its fields (the context kept
         that forward's thickness)."""

@@ -602,13 +602,13 @@ int build(dos_ctx* x, const dos_config* c) {
 // ------------------------------------------------------------ split-BF16 DFT-GEMM path
 // The error flag set by a kernel whose bounded wait expired (tensor-core
 // commit or bulk-copy completion), read after the stream has drained.
-int flag_after_sync(dos_ctx* c) {
+int flag_after_sync(dos_ctx* c, const char* whose = "results since the previous check are invalid") {
   c->err_pending = false;
   if (*c->h_err) {
     *c->h_err = 0;
     DOS_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream), "error flag");
-    return fail(DOS_ERR_TIMEOUT, "a bounded wait gave up (mbarrier wait for a tensor-core commit or a bulk copy "
-                                 "expired); results of the call are invalid");
+    return fail(DOS_ERR_TIMEOUT, std::string("a bounded wait gave up (mbarrier wait for a tensor-core commit or a "
+                                             "bulk copy expired); ") + whose);
   }
   return DOS_OK;
 }
@@ -624,10 +624,14 @@ int err_check(dos_ctx* c) {
 
 // The GEMM path's calls do not wait for the GPU: each queues a copy of the
 // error flag behind its kernels (err_post), and the next call on the context
-// that finds the copy done reports it (err_poll), as dos_read_loss does after
-// its own synchronisation.  (A stream synchronisation at the end of every call
+// that finds the copy done reports it (err_poll), as dos_check and dos_read_loss
+// do after their own synchronisation.  (A stream synchronisation at the end of every call
 // left the GPU idle while the host prepared the next one.)
 int err_post(dos_ctx* c) {
+  if (c->inject_stall) {  // fault injection (tests): the flag as a kernel would have set it
+    c->inject_stall = 0;
+    DOS_CUDA(cudaMemsetAsync(c->d_err, 1, 1, c->stream), "injected error flag");
+  }
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   DOS_CUDA(cudaStreamIsCapturing(c->stream, &cs), "capture status");
   if (cs != cudaStreamCaptureStatusNone) return DOS_OK;  // read by the next call that copies it
@@ -649,7 +653,7 @@ int err_poll(dos_ctx* c) {
     return DOS_OK;
   }
   DOS_CUDA(e, "error event");
-  return flag_after_sync(c);
+  return flag_after_sync(c, "an earlier call's results are invalid; this one queued nothing and may be made again");
 }
 
 // The thickness that a step's last kernel copies to h_fwd (null: nothing to copy)
@@ -1566,6 +1570,12 @@ DOS_API int dos_read_loss(dos_ctx* c, double* h_loss) {
   return flag_after_sync(c);
 }
 
+DOS_API int dos_check(dos_ctx* c) {
+  int rc = check_ctx(c);
+  if (rc) return rc;
+  return err_check(c);
+}
+
 DOS_API int dos_backward(dos_ctx* c, const float* d_dLdI, float* d_dLdh) {
   int rc = check_ctx(c);
   if (rc) return rc;
@@ -1686,6 +1696,7 @@ DOS_API int dos_propagate(dos_ctx* c, int gap, const float* d_in, float* d_out, 
   DOS_CUDA(op->row_in(a, c->stream), "propagate row pass");
   // the prefetching column kernel where either of the context's choices runs it
   const unsigned bulk = c->call_choice < 0 ? choice_mask(c->call_choice) : c->step_choice < 0 ? choice_mask(c->step_choice) : 0;
+  if (bulk & kBulkCol) a.stall = c->take_stall(kBulkCol);
   if (bulk & kBulkCol) DOS_CUDA(op->bulk_col(a, adjoint != 0, c->stream), "propagate column pass");
   else DOS_CUDA(op->col(a, adjoint != 0, false, c->stream), "propagate column pass");
   DOS_CUDA(op->row_back(a, c->stream), "propagate back row pass");
