@@ -49,27 +49,35 @@ __device__ __forceinline__ void pair_add(float& s, float& e, float x) {
   s = t;
 }
 
-// Fixed-order FP64 total of the block's NT partials, by one warp: lane l
-// adds NT / 32 of them, a shuffle tree the 32 lanes.  A partial may be an FP32
-// pair, part + lo (lo not null); the small parts are summed in FP32.  The total is
-// valid in lane 0.  (An FP64 addition occupies the SM's FP64 pipe for many
-// cycles: one warp issues 13 of them here where a block-wide tree in shared
-// memory issues them from every warp and takes eight barriers per sum.)
-template <int NT>
-__device__ __forceinline__ double warp_total(const float* part, const float* lo, int lane) {
+// Fixed-order FP64 total of 256 FP32 partials, by one warp: partials i and i + 128
+// are added as an FP32 pair, lane l adds four of the pairs in FP64 and
+// their low parts in FP32, a shuffle tree the 32 lanes.  The total is valid in
+// lane 0.  (An FP64 addition occupies the SM's FP64 pipe for many cycles: one warp
+// issues ten of them here where a block-wide tree in shared memory issues them
+// from every warp and takes eight barriers per sum.  With each of the 256 partials
+// added in FP64 the launch took 6.1 us for 4 channels, now 5.7.)
+__device__ __forceinline__ double warp_total(const float* part, int lane) {
   double v = 0.0;
   float l = 0.f;
 #pragma unroll
-  for (int i = 0; i < NT / 32; ++i) {
-    v += (double)part[lane + 32 * i];
-    if (lo) l += lo[lane + 32 * i];
+  for (int i = 0; i < 4; ++i) {
+    float s = part[lane + 32 * i], e = 0.f;
+    pair_add(s, e, part[lane + 32 * i + 128]);
+    v += (double)s;
+    l += e;
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) {
     v += __shfl_down_sync(0xffffffffu, v, s);
-    if (lo) l += __shfl_down_sync(0xffffffffu, l, s);
+    l += __shfl_down_sync(0xffffffffu, l, s);
   }
-  return lo ? v + (double)l : v;
+  l = __shfl_sync(0xffffffffu, l, 0);
+  if (!isnan(l)) return v + (double)l;
+  // an infinite partial, or a pair past FP32's range (no low part): all of it in FP64
+  v = 0.0;
+  for (int i = 0; i < kRedThreads / 32; ++i) v += (double)part[lane + 32 * i];
+  for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+  return v;
 }
 
 // Detector pixels a channel may have for its values to stay in shared memory
@@ -80,10 +88,8 @@ constexpr int kLossKeep = 4096;
 // threads are resident at once (eight per SM), a channel gets a block of 128
 // threads, so that twice as many are in flight: 2048 channels of 32 x 32 on 4 x
 // 4-pixel detectors 37 -> 31 us, but 4 channels of 32 x 32 1.3 us more.  A thread
-// of it keeps its even and its odd strides apart, the two chains of FP32
-// multiply-adds that two threads of the larger block have, and adds them as an
-// FP32 pair: the sums have as few terms in FP32 as there, and the same value to
-// 2^-48.
+// of it keeps its even and its odd strides apart, as the partials that two threads
+// of the larger block have: the sums are the same bit for bit.
 constexpr int kLossSmall = 1280, kLossMany = 1024;
 
 // One block per channel: sum (D-T)^2, sigma = sum D T / sum D^2, sum (sigma D
@@ -106,9 +112,7 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
                                                       float* __restrict__ psnr, double* __restrict__ d_loss,
                                                       unsigned* __restrict__ ticket) {
   extern __shared__ float dsh[];  // [det2] detector values, when det2 <= kLossKeep
-  constexpr int V = kRedThreads / NT;  // chains of a thread
-  __shared__ float part[3][NT];
-  __shared__ float lows[V > 1 ? 3 : 1][V > 1 ? NT : 1];
+  __shared__ float part[3][kRedThreads];  // chain i: pixels i, i + 256, ...
   __shared__ double tot[3];
   __shared__ float sg_sh;
   __shared__ bool last;
@@ -118,7 +122,6 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
   const bool keep = det2 <= kLossKeep;
   const float2* ow = o + (size_t)w * fov * fov;
   const float* tw = T + (size_t)w * det2;
-  float sum[3] = {}, low[3] = {};
 #pragma unroll 1
   for (int i = threadIdx.x; i < kRedThreads; i += NT) {
     float fse = 0.f, fit = 0.f, fii = 0.f;
@@ -131,18 +134,13 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
       fit = fmaf(I, t, fit);
       fii = fmaf(I, I, fii);
     }
-    pair_add(sum[0], low[0], fse);
-    pair_add(sum[1], low[1], fit);
-    pair_add(sum[2], low[2], fii);
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    part[k][threadIdx.x] = sum[k];
-    if constexpr (V > 1) lows[k][threadIdx.x] = isinf(sum[k]) ? 0.f : low[k];  // inf - inf is no rounding error
+    part[0][i] = fse;
+    part[1][i] = fit;
+    part[2][i] = fii;
   }
   __syncthreads();
   if (warp < 3) {
-    const double v = warp_total<NT>(part[warp], V > 1 ? lows[warp] : nullptr, lane);
+    const double v = warp_total(part[warp], lane);
     if (lane == 0) tot[warp] = v;
   }
   __syncthreads();
@@ -155,7 +153,6 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
   const float sg = sg_sh;
   const bool scaled = mode == DOS_LOSS_MSE_SCALED;
   float* gw = dLdI ? dLdI + (size_t)w * fov * fov : nullptr;
-  sum[0] = low[0] = 0.f;
 #pragma unroll 1
   for (int i = threadIdx.x; i < kRedThreads; i += NT) {
     float fsc = 0.f;
@@ -166,7 +163,7 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
       fsc = fmaf(d, d, fsc);
       if (gw && b == 1) gw[p] = scaled ? scale * sg * d : scale * (I - t);
     }
-    pair_add(sum[0], low[0], fsc);
+    part[0][i] = fsc;  // (its last reads were two barriers ago)
   }
   if (gw && b > 1) {
     const int fov2 = fov * fov;
@@ -177,11 +174,9 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
       gw[q] = scaled ? scale * sg * fmaf(sg, I, -t) : scale * (I - t);
     }
   }
-  part[0][threadIdx.x] = sum[0];
-  if constexpr (V > 1) lows[0][threadIdx.x] = isinf(sum[0]) ? 0.f : low[0];
   __syncthreads();
   if (warp == 0) {
-    const double ssc = warp_total<NT>(part[0], V > 1 ? lows[0] : nullptr, lane);
+    const double ssc = warp_total(part[0], lane);
     if (lane == 0) {
       LossStats s;
       s.sse = tot[0];
@@ -189,12 +184,14 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
       s.sse_sc = ssc;
       s.pad = 0;
       st[w] = s;
-      if (psnr) psnr[w] = ten_log10((double)det2 / ssc);
+      tot[1] = ssc;
       __threadfence();  // the record is visible before the ticket is taken
       last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
   }
   __syncthreads();
+  // the PSNR, off the path that the total waits for
+  if (psnr && threadIdx.x == NT - 32) psnr[w] = ten_log10((double)det2 / tot[1]);
   if (!last) return;
   // every channel's record is in place: the total, in a fixed order (each
   // thread a stride of the channels, the threads in order of one tree)
@@ -208,7 +205,8 @@ __global__ void __launch_bounds__(NT) k_loss(const float2* __restrict__ o, const
   if (warp == 0) {
     v = 0.0;
 #pragma unroll
-    for (int i = 0; i < NT / 32; ++i) v += acc[lane + 32 * i];
+    for (int i = 0; i < NT / 32; ++i)
+      if (32 * i < (int)gridDim.x) v += acc[lane + 32 * i];
 #pragma unroll
     for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
     if (lane == 0) {

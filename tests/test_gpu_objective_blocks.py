@@ -1,7 +1,7 @@
 """The objective's sums do not depend on the block that forms them.
 
-A sum is 256 FP32 partials, added in FP64 or, where a thread has two of them, as
-an FP32 pair: partial i holds the pixels i, i + 256, ... as a chain of FP32
+A sum is 256 FP32 partials, added two by two as FP32 pairs and then in FP64:
+partial i holds the pixels i, i + 256, ... as a chain of FP32
 multiply-adds.  The same is formed here, in NumPy, from the
 intensities that the engine returned: each multiply-add exactly (the product of
 two FP32 numbers is exact in FP64, and the FP64 sum with an FP32 number is rounded
@@ -64,4 +64,20 @@ def test_sums_are_256_chains(fov, loss, nw):
     p = 10.0 * np.log10(fov * fov / ssc)
     # half a unit in the last place of the result, and the kernel's 0.03 before it
     assert np.max(np.abs(psnr.cpu().numpy().astype(np.float64) - p) / np.spacing(np.abs(p).astype(np.float32))) <= 0.55
+    st.close()
+
+
+def test_sums_past_the_single_precision_range():
+    """Targets so large that two of a sum's FP32 partials leave FP32's range
+    together though neither does: the loss is the FP64 sum."""
+    w = custom(40, 128, 1, [600], 20, 20, name="range")
+    st = DiffractiveStack.from_workload(w, device=DEV, path="multipass")
+    st.forward(torch.tensor(W.thickness(w, 0), dtype=torch.float32, device=DEV))
+    T = np.full((1, 20, 20), 1.5e19, np.float32)  # (I - T)^2 = 2.25e38, 400 of them in 256 partials
+    T[0, 0, 256 % 20:] = 1.0
+    T = T.reshape(-1)
+    T[256:] = 1.0  # one large term a partial at most
+    val, _, _ = st.loss(torch.tensor(T.reshape(1, 20, 20), device=DEV), psnr=False, grad=False)
+    want = np.count_nonzero(T > 2.0) * float(np.float32(1.5e19)) ** 2 / 400.0
+    assert np.isfinite(val) and abs(val - want) <= 1e-6 * want
     st.close()
