@@ -252,6 +252,8 @@ cudaError_t launch_loss_final(const LossStats* st, int nw, int fov2, double norm
 // exact rounding errors of its additions, Knuth's two-sum), about 48 bits, and
 // rounded to FP32 once at the end like the FP64 sum before it: GB300 adds and
 // converts FP64 at a small fraction of its FP32 rate, which bound the kernel.
+// Where the running sum leaves FP32's range the parts are added in FP64 after all:
+// they may come back.
 // A block's 256 threads take 32 pixels x 8 slices of the parts, eight loads of a
 // slice in flight, so that small layers with many parts still fill the chip; or
 // 256 pixels each with all of them where the parts are few and the pixels many
@@ -264,9 +266,8 @@ constexpr int kGradThreads = 256;
 
 template <int SLICES>
 __global__ void __launch_bounds__(kGradThreads) k_grad_reduce(const float* __restrict__ partial,
-                                                              float* __restrict__ grad, int n_parts, size_t count,
-                                                              size_t n2, const float* __restrict__ h,
-                                                              float* __restrict__ h_keep) {
+                                                              float* grad, int n_parts, size_t count, size_t n2,
+                                                              const float* h, float* h_keep) {
   constexpr int PX = kGradThreads / SLICES;
   __shared__ float2 sh[SLICES][PX];
   pdl_wait();
@@ -300,8 +301,14 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_reduce(const float* __res
     e = __fadd_rn(e, v.y);
   }
   if (h) h_keep[g] = h[g];
-  // an infinite sum has no rounding error to add (inf - inf)
-  grad[g] = isinf(s) ? s : s + e;
+  float v = s + e;
+  if (!isfinite(v)) {
+    const float* p = partial + g / n2 * n_parts * n2 + g % n2;
+    double acc = 0.0;
+    for (int c = 0; c < n_parts; ++c) acc += (double)p[(size_t)c * n2];
+    v = (float)acc;
+  }
+  grad[g] = v;  // (the caller's gradient may lie where its thickness does: h is read first)
 }
 
 cudaError_t launch_grad_reduce(const float* partial, float* grad, int n_parts, size_t count, size_t n2, const float* h,
