@@ -82,8 +82,8 @@ struct Fused {
   // |k| = k below M/2 and M - k above, both affine in i at compile time.
   // MIS: displaced layers (kernels of their own: the displacement's phase per
   // element would more than double the column phase's code, which a short sweep
-  // fetches cold: step of 4 channels of 64 x 64 31.4 -> 27.7 us, a thickness copy
-  // saved in the same measurement).
+  // fetches cold: step of 4 channels of 64 x 64 31.4 -> 27.7 us together with one
+  // device copy less, measured as one).
   template <bool MIS>
   __device__ static __forceinline__ void load_h(float2 (&hreg)[E], const float2* __restrict__ Hw, int hs, int t,
                                                 int cc, const float* __restrict__ Sw, const Misalign& mg) {

@@ -45,7 +45,7 @@ __host__ __device__ inline size_t gemm_tiled(size_t row, int k, int kp) {
 
 // One GEMM D[rows][cols] (f32, row-major, leading dimension ldd) =
 //   sum over segments s of A_s[rows][K] * B_s[cols][K]^T, A_s / B_s bf16 in
-//   the tiled order above.  rows % 256 == 0, K % 64 == 0; cols may be ragged
+//   the tiled order above.  rows % 128 == 0, K % 64 == 0; cols may be ragged
 //   (B must then hold whole 256-row tiles; rows past cols are never stored).
 constexpr int kMaxGemmTerms = 6;
 
@@ -68,7 +68,7 @@ struct GemmArgs {
   const __nv_bfloat16* a[kMaxGemmTerms];
   const __nv_bfloat16* b[kMaxGemmTerms];
   int nseg;
-  int rows, cols, K;  // tiles of the A operand (rows) and B operand (cols), 256 each
+  int rows, cols, K;  // A operand in tiles of 128 rows, B operand in tiles of 256 or 128 columns
   int w_is_b;         // the DFT matrix is the B operand (raster: its tiles fastest)
   int* err;           // set to 1 when a bounded wait gave up
   int mode;           // GEMM_OUT_*

@@ -151,7 +151,7 @@ struct PassOps {
   cudaError_t (*bulk_row_first)(const PassArgs&, cudaStream_t);  // t(h) * field (fin) -> row spectra
   int (*bulk_adj_chunk)(int n, int nw, int most);  // channels per chunk of bulk_row_adj (0: unknown)
   // boxes of the bulk column pass's tensor copies: spectra {col_group, rows, 1},
-  // transfer table {h_box_cols, h_box_rows, 1} (h_box_cols 0: no staged H tile)
+  // transfer table {h_box_cols, h_box_rows, 1}
   int col_group, h_box_cols, h_box_rows;
 };
 

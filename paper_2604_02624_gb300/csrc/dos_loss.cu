@@ -4,10 +4,11 @@
 // every channel and its target; reconstruction quality is a PSNR.  The
 // detector (Section 4: the FOV divided into output pixels) reads pixel (y, x)
 // as the sum of the b x b simulation intensities it covers (b = 1: I itself).
-// Per-pixel arithmetic and each thread's strided partial sums run in FP32 (a
-// thread sums at most a few hundred terms), the block tree and everything
-// after it in FP64 (GB300's FP64 rate is a small fraction of its FP32 rate);
-// every sum has a fixed order, so results are reproducible bit for bit.
+// Per-pixel arithmetic and the 256 strided partial sums of a channel run in FP32 (at
+// most a few hundred terms each); partials are added in FP64, two by two as FP32
+// pairs first (GB300's FP64 rate is a small fraction of its FP32 rate), and what
+// follows is FP64 but for the PSNR's logarithm and the gradient parts' sums (FP32
+// pairs).  Every sum has a fixed order, so results are reproducible bit for bit.
 #include "dos_decibel.cuh"
 #include "dos_internal.h"
 

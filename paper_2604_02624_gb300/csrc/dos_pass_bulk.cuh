@@ -138,7 +138,7 @@ struct PassBulk {
   // packed FP32-pair butterflies in every bulk pass (faster than scalar ones
   // in each of them on the 400-point line)
   static constexpr bool PKR = true, PKC = true;
-  static constexpr int COLL = Pass<LF>::COLL, ZL = Pass<LF>::ZL, RZL = Pass<LF>::RZL;
+  static constexpr int RZL = Pass<LF>::RZL;
   static constexpr int SR = row_stage_stride(M);  // even: every staged row starts 16-byte aligned
   static_assert(SR % 2 == 0 && SR >= M, "staged rows must be 16-byte aligned and hold M values");
   static_assert(Pass<LF>::RZL >= LF::ZS, "exchange buffers must not overlap");
@@ -207,7 +207,7 @@ struct PassBulk {
     return s > h ? s : h;
   }
   static constexpr int GT = GW * T;                    // threads of a block
-  static constexpr bool GROUP_BARS = GT % 32 == 0;     // whole warps (all sizes but M = 200)
+  static constexpr bool GROUP_BARS = GT % 32 == 0;     // whole warps, all sizes but M = 200 (host checks of the layout)
   // Exchange matrices of the column lines: even pitch ZX (row entries k1,
   // k1 + 1 are one 16-byte access), stride ZLB between the lines at least
   // Q ZX and 2 mod 16.  A warp holds 8 lines x 4 consecutive element owners;
@@ -929,8 +929,12 @@ template <class LF, int RL, bool HALF, bool FIRST>
 __global__ void __launch_bounds__(LF::T * RL, 3) k_row_adj_staged(PassArgs a) {
   PassBulk<LF, RL, HALF>::template row_adj_staged<FIRST>(a);
 }
-// Column pass: four blocks of 8 lines per SM for every line shape (M = 400: 20
-// warps at up to 102 registers, M = 512: 16 at up to 128).
+// Column pass: resident blocks of 8 lines per SM that the registers are held to.
+// Four where lines have 16 owners and more (M = 400: 20 warps at up to 102
+// registers, M = 512: 16 at up to 128), six at M = 256 (85 registers: step of 1024
+// channels of 128 x 128 1495 us with four, 1484 with six), eight for shorter lines
+// (M = 200, 1024 channels of 100 x 100: 1132 us with four, 1111 with eight; M = 128
+// and 64 need no more registers than eight blocks leave: no difference).
 template <class LF>
 constexpr int col_bulk_min_blocks() { return LF::M == 256 ? 6 : LF::T >= 16 ? 4 : 8; }
 template <class LF, int RL, bool HALF, bool ADJ, bool MIS>
@@ -975,10 +979,13 @@ inline int balanced_chunk(int nw, int rb, int slots, int most) {
   }
   return best;
 }
-// Most channels per block: the adjoint row pass sums its chunk's channels in
-// FP32 registers (before balanced_chunk: 45 at 4096 channels, so no more terms
-// than then), and long chunks spread the blocks that run together over the
-// whole spectra buffer.
+// Most channels per block, unless the plain pass's chunk is larger: the adjoint row
+// pass sums its chunk's channels in FP32 registers, and long chunks spread the
+// blocks that run together over the whole spectra buffer.  The sums' terms are lost
+// in the fields' own rounding: 256 channels of 200 x 200, gradient error against 64
+// bits 4.516e-7 with three channels to a block (the plain pass's chunk there),
+// 4.529e-7 with the fifteen that balanced_chunk takes (mean of six designs); row
+// launches of 88 us with the first, 83 with the second.
 constexpr int kRowChunk = 48;
 
 // Launchers.  The column pass runs one persistent block per resident slot
