@@ -294,9 +294,10 @@ DOS_API int dos_quantize_thickness(const float *d_h, float *d_hq, size_t count, 
  * Returns DOS_ERR_TIMEOUT when a kernel queued since the previous check gave
  * up a bounded wait (bulk-copy or tensor-core completion); the loss and every
  * result of that work are then invalid.  The flag is cleared by the report.
- * On the DFT-GEMM paths dos_forward and dos_backward also report, in the same
- * way and before they queue anything, an expired wait of an earlier call that
- * the GPU has finished by then; the refused call may be made again.
+ * On the DFT-GEMM paths dos_forward, dos_backward and a dos_step that queues its
+ * kernels also report, in the same way and before they queue anything, an
+ * expired wait of an earlier call that the GPU has finished by then; the refused
+ * call may be made again.
  */
 DOS_API int dos_read_loss(dos_ctx *ctx, double *h_loss);
 
@@ -336,7 +337,7 @@ DOS_API int dos_backward(dos_ctx *ctx, const float *d_dLdI, float *d_dLdh);
  *   d_I [N_w][F][F] and d_psnr [N_w] optional outputs (NULL to skip).
  *   h_loss: when non-NULL receives L (waits for the stream).
  * Afterwards the context holds the same state as after the three calls.
- * Errors: DOS_ERR_ARG, DOS_ERR_CUDA.
+ * Errors: DOS_ERR_ARG, DOS_ERR_CUDA, DOS_ERR_TIMEOUT (h_loss, DFT-GEMM paths).
  */
 DOS_API int dos_step(dos_ctx *ctx, const float *d_h, const float *d_T, float *d_dLdh, float *d_I,
                      float *d_psnr, double *h_loss);
